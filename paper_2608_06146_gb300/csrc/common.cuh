@@ -80,6 +80,54 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
+// ------------------------------------------------------------------------------------------------
+// Thread-block clusters
+// ------------------------------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// The address (shared::cluster) of a CTA's own shared-memory address in the CTA of the given rank.
+__device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
+// Arrival on a barrier given by its shared::cluster address: kRelease with cluster scope (what this
+// thread wrote is visible to the waiting threads of the cluster), else with the CTA's (for barriers
+// that order tensor-memory accesses only: a cluster-scope release waits ~1000 cycles for the thread's
+// earlier accesses).
+template <bool kRelease>
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar)
+{
+    if constexpr (kRelease) asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+    else asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n"
+        " mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ void st_cluster_v4(uint32_t addr, int4 v)
+{
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+                 : "memory");
+}
+
 // Waits for the phase with the given parity to complete; false (and the error word set to
 // PADOC_DEVERR_TIMEOUT with `site` as the detail) if it does not complete within limit_ns.
 __device__ __forceinline__ bool mbar_wait_bounded_ns(uint32_t bar, uint32_t parity, int *err, int site,
@@ -90,6 +138,20 @@ __device__ __forceinline__ bool mbar_wait_bounded_ns(uint32_t bar, uint32_t pari
     for (uint32_t i = 1;; ++i) {
         if (mbar_try_wait(bar, parity)) return true;
         if ((i & 255u) == 0 && padoc_globaltimer() - t0 > limit_ns) {
+            padoc_record_error(err, PADOC_DEVERR_TIMEOUT, site);
+            return false;
+        }
+    }
+}
+
+// The same with cluster scope: what the arriving threads of the cluster's other CTAs wrote is visible.
+__device__ __forceinline__ bool mbar_wait_bounded_cluster(uint32_t bar, uint32_t parity, int *err, int site)
+{
+    if (mbar_try_wait_cluster(bar, parity)) return true;
+    const uint64_t t0 = padoc_globaltimer();
+    for (uint32_t i = 1;; ++i) {
+        if (mbar_try_wait_cluster(bar, parity)) return true;
+        if ((i & 255u) == 0 && padoc_globaltimer() - t0 > PADOC_WAIT_LIMIT_NS) {
             padoc_record_error(err, PADOC_DEVERR_TIMEOUT, site);
             return false;
         }
@@ -113,6 +175,30 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
         "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
         : "memory");
 }
+
+// tma_load_2d into this CTA's shared memory with the completion on a barrier of either CTA of the pair
+// (a shared::cluster address).
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap *map, int32_t x, int32_t y, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
+        : "memory");
+}
+
+// 2-D tile from shared to global memory (parts past the tensor's end are not written). The issuing
+// thread's copies form bulk groups: tma_store_commit closes one, tma_store_wait_read<N> waits until at
+// most the N latest still read shared memory.
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, int32_t x, int32_t y, uint32_t src)
+{
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                     reinterpret_cast<uint64_t>(map)),
+                 "r"(x), "r"(y), "r"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
 
 // L2 policy for data read once per call (the paged K/V): such lines are the first evicted, so the
 // split-K partials written in the same call stay in L2 for the merge that reads them.

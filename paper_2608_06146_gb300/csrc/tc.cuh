@@ -41,19 +41,31 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N, bool b_mn_m
 // ------------------------------------------------------------------------------------------------
 // TMEM
 // ------------------------------------------------------------------------------------------------
-// Executed by one full warp. Writes the allocated TMEM base address to shared memory.
+// Executed by one full warp (CG = 2: by one warp of each CTA of the pair). Writes the allocated TMEM
+// base address to shared memory.
+template <int CG = 1>
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols)
 {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols)
-                 : "memory");
+    if constexpr (CG == 2)
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols)
+                     : "memory");
+    else
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols)
+                     : "memory");
 }
+template <int CG = 1>
 __device__ __forceinline__ void tmem_relinquish()
 {
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (CG == 2) asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    else asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
+template <int CG = 1>
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols)
 {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+    if constexpr (CG == 2)
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+    else
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -101,6 +113,75 @@ __device__ __forceinline__ void umma_bf16_ts_warp(uint32_t d_tmem, uint32_t a_tm
         "{\n .reg .pred p, e;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n"
         " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d_tmem),
         "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// Eight K-steps (128 elements) of a K-major product in one block, D = A[smem] . B[smem]^T: a step adds
+// 32 bytes to both start addresses, the fifth one starts the second 64-element panel (PA and PB bytes
+// on). One election and in-block address arithmetic: with a statement per MMA the compiler hoists
+// every step's descriptors out of the caller's loop and spills them. CG = 2: one MMA over a CTA pair,
+// issued by the leader (M = 256, half of the rows and of D in each CTA, half of B's rows in each).
+template <int CG, int PA, int PB>
+__device__ __forceinline__ void umma_bf16_ss_k128_warp(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc)
+{
+    if constexpr (CG == 2)
+        asm volatile(
+            "{\n .reg .pred e, t, f;\n .reg .b64 a, b;\n elect.sync _|e, 0xffffffff;\n"
+            " setp.eq.u32 t, 0, 0;\n setp.ne.u32 f, 0, 0;\n"
+            " @e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, f;\n"
+            " add.s64 a, %1, 2;\n add.s64 b, %2, 2;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, t;\n"
+            " add.s64 a, %1, 4;\n add.s64 b, %2, 4;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, t;\n"
+            " add.s64 a, %1, 6;\n add.s64 b, %2, 6;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, t;\n"
+            " add.s64 a, %1, %4;\n add.s64 b, %2, %5;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, t;\n"
+            " add.s64 a, %1, %4+2;\n add.s64 b, %2, %5+2;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, t;\n"
+            " add.s64 a, %1, %4+4;\n add.s64 b, %2, %5+4;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, t;\n"
+            " add.s64 a, %1, %4+6;\n add.s64 b, %2, %5+6;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, t;\n}" ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "n"(PA >> 4), "n"(PB >> 4)
+            : "memory");
+    else
+        asm volatile(
+            "{\n .reg .pred e, t, f;\n .reg .b64 a, b;\n elect.sync _|e, 0xffffffff;\n"
+            " setp.eq.u32 t, 0, 0;\n setp.ne.u32 f, 0, 0;\n"
+            " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, f;\n"
+            " add.s64 a, %1, 2;\n add.s64 b, %2, 2;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n"
+            " add.s64 a, %1, 4;\n add.s64 b, %2, 4;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n"
+            " add.s64 a, %1, 6;\n add.s64 b, %2, 6;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n"
+            " add.s64 a, %1, %4;\n add.s64 b, %2, %5;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n"
+            " add.s64 a, %1, %4+2;\n add.s64 b, %2, %5+2;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n"
+            " add.s64 a, %1, %4+4;\n add.s64 b, %2, %5+4;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n"
+            " add.s64 a, %1, %4+6;\n add.s64 b, %2, %5+6;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n}" ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "n"(PA >> 4), "n"(PB >> 4)
+            : "memory");
+}
+// Four K-steps (64 elements) of D (+)= A[tmem] . B[smem], B MN-major (a step adds 16 rows, 2048 bytes)
+// and A 8 columns a step; `accumulate` 0: the first step overwrites D.
+template <int CG>
+__device__ __forceinline__ void umma_bf16_ts_k64_mn_warp(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                                         uint32_t accumulate)
+{
+    if constexpr (CG == 2)
+        asm volatile(
+            "{\n .reg .pred e, t, p;\n .reg .b64 b;\n .reg .b32 a;\n elect.sync _|e, 0xffffffff;\n"
+            " setp.eq.u32 t, 0, 0;\n setp.ne.b32 p, %4, 0;\n"
+            " @e tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n"
+            " add.s32 a, %1, 8;\n add.s64 b, %2, 128;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], [a], b, %3, t;\n"
+            " add.s32 a, %1, 16;\n add.s64 b, %2, 256;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], [a], b, %3, t;\n"
+            " add.s32 a, %1, 24;\n add.s64 b, %2, 384;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], [a], b, %3, t;\n}" ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+            : "memory");
+    else
+        asm volatile(
+            "{\n .reg .pred e, t, p;\n .reg .b64 b;\n .reg .b32 a;\n elect.sync _|e, 0xffffffff;\n"
+            " setp.eq.u32 t, 0, 0;\n setp.ne.b32 p, %4, 0;\n"
+            " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n"
+            " add.s32 a, %1, 8;\n add.s64 b, %2, 128;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
+            " add.s32 a, %1, 16;\n add.s64 b, %2, 256;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
+            " add.s32 a, %1, 24;\n add.s64 b, %2, 384;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n}" ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+            : "memory");
+}
+// As umma_commit_warp for MMAs over a CTA pair: arrives on the barrier at this offset in both CTAs.
+__device__ __forceinline__ void umma_commit_pair_warp(uint32_t mbar)
+{
+    asm volatile(
+        "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+        " @e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n}" ::"r"(mbar),
+        "h"((uint16_t)3)
         : "memory");
 }
 __device__ __forceinline__ void umma_commit_warp(uint32_t mbar)
@@ -189,6 +270,12 @@ __device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c)
 {
     uint64_t r;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
 __device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b)
