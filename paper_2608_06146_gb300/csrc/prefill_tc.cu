@@ -197,8 +197,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
     auto read_unit = [&](int n, Unit &u, int site) {
         const bool r = wait_or_abort<CG == 2>(bar(C::B_UFULL + (n & 1)), (n >> 1) & 1, prm.err, site, abort_flag);
         if (!__all_sync(0xffffffffu, r)) return false;
-        u = units[n & 1];
-        u.ne = __shfl_sync(0xffffffffu, u.ne, 0);
+        const Unit v = units[n & 1];
+        // (every lane's read has returned before the arrival lets the slot be written again)
+        u.h0 = __shfl_sync(0xffffffffu, v.h0, 0);
+        u.qt = __shfl_sync(0xffffffffu, v.qt, 0);
+        u.e0 = __shfl_sync(0xffffffffu, v.e0, 0);
+        u.ne = __shfl_sync(0xffffffffu, v.ne, 0);
+        __syncwarp();
         if (lane == 0) arrive_lead(C::B_UEMPTY + (n & 1));
         return true;
     };
