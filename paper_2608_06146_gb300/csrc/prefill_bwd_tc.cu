@@ -6,12 +6,11 @@
 // (-lse2 and D precomputed per head, [Hq][t_pad], padded rows -lse2 = -inf so that their P is 0):
 //   P = exp2(S c - lse2),  dS = P (dP - D),  S = Q K^T,  dP = dO V^T.
 //
-// dK/dV pass: one CTA per (128-key k-tile, KV head), k-tiles taken in the key-major map's order
-//   (most work first); a unit with more than PADOC_BWD_SPLIT_STEPS steps runs as two CTAs over its
-//   two halves of steps, which write fp32 partials that prefill_bwd_dkv_merge_kernel adds (the
-//   heaviest units otherwise set the pass's tail). K and V of the tile sit in tensor memory as A
-//   operands for the whole walk.
-//   For every (32-row q-tile that sees the k-tile, query head reading the KV head) step the tensor
+// dK/dV pass: a unit is a (128-key k-tile, KV head), units taken in the key-major map's order (most
+//   work first), run by a cluster of 1, 2, 4 or 8 CTAs that share out its steps and add their fp32 sums
+//   through distributed shared memory (pick_cluster below). K and V of the tile sit in shared memory
+//   for the whole walk.
+//   For every (64-row q-tile that sees the k-tile, query head reading the KV head) step the tensor
 //   cores form S^T = K Q^T and dP^T = V dO^T (M = 128 keys, N = 32 queries, B from shared memory),
 //   the softmax warps write P^T and dS^T back into tensor memory as bf16, and dV += P^T dO,
 //   dK += dS^T Q accumulate in tensor memory over the whole walk. Every query that sees a
@@ -62,8 +61,6 @@ struct BwdParams {
     int32_t num_q_heads, num_kv_heads, num_tiles;
     float scale_log2, scale;
     __nv_bfloat16 *out0, *out1;         // dK/dV pass: dK, dV; dQ pass: dQ
-    float *split;                       // dK/dV pass: fp32 partials of the split units
-    int32_t split_units;                // dK/dV pass: units of the key-major order below this may split
     int *err;
 };
 
@@ -97,6 +94,18 @@ __device__ __forceinline__ void tmem_st_cols(uint32_t taddr, const uint32_t (&r)
     if constexpr (N == 16) tmem_st16(taddr, r); else tmem_st8(taddr, r);
 }
 
+__device__ __forceinline__ void store_row_bf16(__nv_bfloat16 *dst, const float (&o)[16], float mul)
+{
+#pragma unroll
+    for (int i = 0; i < 16; i += 8) {
+        uint4 w;
+        w.x = pack_bf16x2(o[i] * mul, o[i + 1] * mul);
+        w.y = pack_bf16x2(o[i + 2] * mul, o[i + 3] * mul);
+        w.z = pack_bf16x2(o[i + 4] * mul, o[i + 5] * mul);
+        w.w = pack_bf16x2(o[i + 6] * mul, o[i + 7] * mul);
+        *reinterpret_cast<uint4 *>(dst + i) = w;
+    }
+}
 __device__ __forceinline__ void store_row_bf16(__nv_bfloat16 *dst, const uint32_t (&o)[32], float mul)
 {
 #pragma unroll
@@ -147,7 +156,7 @@ __device__ __forceinline__ uint32_t transpose32_warp(uint32_t x, int lane)
 namespace dkv {
 constexpr int kKT = PADOC_BWD_DKV_K_TILE;   // 128 keys: the M of every MMA
 constexpr int kQT = PADOC_BWD_DKV_Q_TILE;   // 64 queries per step
-constexpr int kStages = 3;
+constexpr int kStages = 4;   // (3: the Q of the step after next is still on its way, +1.5% time)
 constexpr uint32_t kColS = 0, kColDP = 128, kColAcc0 = 256, kColAcc1 = 384;
 constexpr int kKPanel = kKT * 128;           // [128 rows][64 bf16]
 constexpr int kQPanel = kQT * 128;           // [64 rows][64 bf16]
@@ -167,6 +176,8 @@ constexpr size_t kSmemBytes = 1024 + 2 * (size_t)kKTile + 2 * (size_t)kStages * 
                               B_COUNT * 8 + 64;
 }  // namespace dkv
 
+// NC: the CTAs of a unit's cluster.
+template <int NC>
 __global__ void __launch_bounds__(kThreads, 1)
 prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap gmap,
                        const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
@@ -186,16 +197,11 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int hkv = prm.num_kv_heads, group = prm.num_q_heads / hkv;
-    // CTA b: KV head b % hkv of the (b / hkv) % 2-th half of unit b / (2 hkv) of the key-major order;
-    // a unit of more than PADOC_BWD_SPLIT_STEPS steps (among the first split_units) runs as two
-    // halves that write fp32 partials, the others as one CTA (the second CTA leaves at once)
-    const int unit = (int)(blockIdx.x / (2 * hkv)), half = (int)((blockIdx.x / hkv) & 1), g = (int)(blockIdx.x % hkv);
-    const int kt = prm.order[unit];
-    const int e0 = prm.ptr[kt], ne = prm.ptr[kt + 1] - e0;
-    const bool split = ne * group > PADOC_BWD_SPLIT_STEPS && unit < prm.split_units;
-    if (half == 1 && !split) return;
-    const int ub = half ? ne * group / 2 : 0;                               // first step of this CTA
-    const int nu = split ? (half ? ne * group - ub : ne * group / 2) : ne * group;
+    // the cluster's unit, and this CTA's steps of it: ub .. ub + nu - 1
+    const int unit = (int)blockIdx.x / NC, rank = (int)blockIdx.x % NC, g = unit % hkv;
+    const int kt = prm.order[unit / hkv];
+    const int e0 = prm.ptr[kt], steps = (prm.ptr[kt + 1] - e0) * group;
+    const int ub = (int)((int64_t)steps * rank / NC), nu = (int)((int64_t)steps * (rank + 1) / NC) - ub;
     auto bar = [&](int i) { return smem_u32(&bars[i]); };
 
     if (tid == 0) {
@@ -211,14 +217,20 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    const int lq = warp & 3, ch = warp >> 2;          // softmax warps: TMEM lane quarter, column half
+    const int key = kt * kKT + lq * 32 + lane;
+    const uint32_t lanes = (uint32_t)(lq * 32) << 16;
+    bool sums = false;                                // softmax warps: this CTA's dV and dK are complete
 
     if (warp == 8) {
         // ---------------------------------------------------------------- TMA producer
+        if (lane == 0 && nu == 0) pdl_wait_prerequisite();
         if (lane == 0 && nu > 0) {
             tma_prefetch_desc(&qmap);
             tma_prefetch_desc(&gmap);
             tma_prefetch_desc(&kmap);
             tma_prefetch_desc(&vmap);
+            pdl_wait_prerequisite();   // -lse2 and D are the dQ pass's
             mbar_arrive_expect_tx(bar(B_KV), 2 * kKTile);
             tma_load_2d(smem_u32(sk), &kmap, g * kD, kt * kKT, bar(B_KV));
             tma_load_2d(smem_u32(sk) + kKPanel, &kmap, g * kD + 64, kt * kKT, bar(B_KV));
@@ -318,9 +330,6 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
         }
     } else {
         // ---------------------------------------------------------------- softmax + epilogue
-        const int lq = warp & 3, ch = warp >> 2;          // TMEM lane quarter, column half
-        const int key = kt * kKT + lq * 32 + lane;
-        const uint32_t lanes = (uint32_t)(lq * 32) << 16;
         const float c = prm.scale_log2;
         auto wait_all = [&](int b, uint32_t parity, int site) {
             const bool r = wait_or_abort(bar(b), parity, prm.err, site, abort_flag);
@@ -396,33 +405,73 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
             tc_fence_before();
             mbar_arrive(bar(B_PFULL + (u & 1)));
         }
-        // epilogue: column half 0 writes dV, half 1 writes dK (times scale), one key row per thread;
-        // a split unit's halves write their fp32 sums instead ([unit][g][half][dV, dK][key][dim])
-        if (ok && (nu == 0 || wait_all(B_FINAL, 0, 72))) {
+        sums = ok && (nu == 0 || wait_all(B_FINAL, 0, 72));
+        tc_fence_after();
+    }
+    // Epilogue. The 256 columns of dV | dK are split over the cluster's CTAs: each one's softmax threads
+    // (a key row and half of the columns each) send the other CTAs' parts to their shared memory, which
+    // nothing else uses any more, add what they receive to their own part in rank order and write it.
+    constexpr int kPart = 256 / NC, kHalfPart = kPart / 2;   // columns of a CTA, of a thread
+    auto part = [&](int p, int c, uint32_t (&o)[16]) {       // 16 of this CTA's sums of part p
+        if (nu > 0) {
+            tmem_ld16(tmem + lanes + kColAcc0 + kPart * p + kHalfPart * ch + c, o);
+            tmem_ld_wait();
+        } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) o[i] = 0u;
+        }
+    };
+    // the place of a thread's 16 columns from CTA `from` in the receiver's shared memory
+    auto slot = [&](int from, int to, int c) {
+        const int n = from < to ? from : from - 1;
+        return (uint32_t)(n * kPart * kKT * 4 + (kHalfPart * ch + c) * kKT * 4 + (lq * 32 + lane) * 16);
+    };
+    if (NC > 1) {
+        tc_fence_before();
+        cluster_sync();
+        if (sums) {
             tc_fence_after();
-            const bool isk = ch == 1;
-            __nv_bfloat16 *dst = (isk ? prm.out0 : prm.out1) + ((size_t)(key < prm.T ? key : 0) * hkv + g) * kD;
-            float *pdst = prm.split + ((((size_t)unit * hkv + g) * 2 + half) * 2 + (isk ? 1 : 0)) * (kKT * kD) +
-                          (size_t)(lq * 32 + lane) * kD;
-            const float mul = isk ? prm.scale : 1.f;
+#pragma unroll 1
+            for (int d = 1; d < NC; ++d) {
+                const int p = (rank + d) % NC;
+                const uint32_t dst = cluster_map(smem_u32(smem), p);
+#pragma unroll 1
+                for (int c = 0; c < kHalfPart; c += 16) {
+                    uint32_t o[16];
+                    part(p, c, o);
 #pragma unroll
-            for (int cc = 0; cc < 4; ++cc) {
-                uint32_t o[32];
-                if (nu > 0) {
-                    tmem_ld32(tmem + lanes + (isk ? kColAcc1 : kColAcc0) + 32 * cc, o);
-                    tmem_ld_wait();
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) o[i] = 0u;
-                }
-                if (split) {
-#pragma unroll
-                    for (int i = 0; i < 32; i += 4)
-                        *reinterpret_cast<uint4 *>(pdst + 32 * cc + i) = make_uint4(o[i], o[i + 1], o[i + 2], o[i + 3]);
-                } else if (key < prm.T) {
-                    store_row_bf16(dst + 32 * cc, o, mul);
+                    for (int i = 0; i < 16; i += 4)
+                        st_cluster_v4(dst + slot(rank, p, c + i), make_int4(o[i], o[i + 1], o[i + 2], o[i + 3]));
                 }
             }
+        }
+        cluster_sync();
+    }
+    if (sums) {
+#pragma unroll 1
+        for (int c = 0; c < kHalfPart; c += 16) {
+            uint32_t own[16];
+            part(rank, c, own);
+            float acc[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) acc[i] = 0.f;
+#pragma unroll
+            for (int from = 0; from < NC; ++from)
+#pragma unroll
+                for (int i = 0; i < 16; i += 4) {
+                    const float4 x = from == rank ? make_float4(__uint_as_float(own[i]), __uint_as_float(own[i + 1]),
+                                                                __uint_as_float(own[i + 2]), __uint_as_float(own[i + 3]))
+                                                  : *reinterpret_cast<const float4 *>(smem + slot(from, rank, c + i));
+                    acc[i] += x.x;
+                    acc[i + 1] += x.y;
+                    acc[i + 2] += x.z;
+                    acc[i + 3] += x.w;
+                }
+            const int col = kPart * rank + kHalfPart * ch + c;
+            const bool isk = col >= kD;                       // dV first, then dK (times scale)
+            if (key < prm.T)
+                store_row_bf16((isk ? prm.out0 : prm.out1) + ((size_t)key * hkv + g) * kD + (col & (kD - 1)), acc,
+                               isk ? prm.scale : 1.f);
         }
     }
     tc_fence_before();
@@ -430,31 +479,6 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
     if (warp == 9) {
         tc_fence_after();
         tmem_dealloc(tmem, kTmemCols);
-    }
-}
-
-// The split units' halves added (fp32), dK times scale, rounded once to bf16: one CTA per unit that
-// may split (those that did not leave at once).
-__global__ void __launch_bounds__(256) prefill_bwd_dkv_merge_kernel(const BwdParams prm)
-{
-    using namespace dkv;
-    const int hkv = prm.num_kv_heads, group = prm.num_q_heads / hkv;
-    const int unit = (int)(blockIdx.x / hkv), g = (int)(blockIdx.x % hkv);
-    const int kt = prm.order[unit];
-    const int ne = prm.ptr[kt + 1] - prm.ptr[kt];
-    if (!(ne * group > PADOC_BWD_SPLIT_STEPS && unit < prm.split_units)) return;
-    const float4 *p = reinterpret_cast<const float4 *>(prm.split + ((size_t)unit * hkv + g) * 4 * (kKT * kD));
-    constexpr int kQuads = kKT * kD / 4;                  // float4 per tensor and half
-    for (int x = threadIdx.x; x < 2 * kQuads; x += blockDim.x) {
-        const int isk = x / kQuads, r = (x % kQuads) / (kD / 4), c4 = x % (kD / 4);
-        const int64_t key = (int64_t)kt * kKT + r;
-        if (key >= prm.T) continue;
-        const float4 a = p[isk * kQuads + x % kQuads], b = p[(2 + isk) * kQuads + x % kQuads];
-        const float mul = isk ? prm.scale : 1.f;
-        uint2 w;
-        w.x = pack_bf16x2((a.x + b.x) * mul, (a.y + b.y) * mul);
-        w.y = pack_bf16x2((a.z + b.z) * mul, (a.w + b.w) * mul);
-        *reinterpret_cast<uint2 *>((isk ? prm.out0 : prm.out1) + ((size_t)key * hkv + g) * kD + 4 * c4) = w;
     }
 }
 
@@ -503,6 +527,7 @@ prefill_bwd_dq_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int hq = prm.num_q_heads, group = hq / prm.num_kv_heads;
     const int qt = prm.num_tiles - 1 - (int)(blockIdx.x / hq);   // heavier q-tiles (later in a page) first
+    pdl_launch_dependents();   // the dK/dV pass may take the SMs that run out of work here
     const int h = (int)(blockIdx.x % hq), g = h / group;
     const int e0 = prm.ptr[qt], nu = prm.ptr[qt + 1] - e0;
     auto bar = [&](int i) { return smem_u32(&bars[i]); };
@@ -725,13 +750,47 @@ prefill_bwd_dq_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
     }
 }
 
+// The CTAs that share a dK/dV unit. A page's first k-tiles are seen by all of its later queries, so the
+// largest unit is about twice the mean and a few units leave most of the chip idle: one page of 3419
+// tokens (54 units, 432 steps of 0.9 us the largest) takes 225 us with the largest units on two CTAs,
+// 105 on four, and no merge kernel follows (24 us). With more units than this the sharing's own cost (~8 us a CTA) is the larger: a
+// list-scheduling model over 60 page sets drawn from 1 to 6 pages puts the lines where they are (within
+// 10% of the best choice of the four on all of them).
+int pick_cluster(int64_t units)
+{
+    return units <= 45 ? 8 : units <= 160 ? 4 : units <= 560 ? 2 : 1;
+}
+
+template <int NC>
+padoc_status launch_dkv(const CUtensorMap &q64, const CUtensorMap &g64, const CUtensorMap &k128, const CUtensorMap &v128,
+                        const BwdParams &prm, int64_t units, cudaStream_t stream)
+{
+    auto kernel = prefill_bwd_dkv_kernel<NC>;
+    if (const padoc_status st = padoc_set_max_smem((const void *)kernel, (int)dkv::kSmemBytes)) return st;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)(units * NC));
+    lc.blockDim = dim3(kThreads);
+    lc.dynamicSmemBytes = dkv::kSmemBytes;
+    lc.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = NC;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see the producer's wait
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = attr;
+    lc.numAttrs = 2;
+    PADOC_CUDA_TRY(cudaLaunchKernelEx(&lc, kernel, q64, g64, k128, v128, prm));
+    return padoc_launch_status();
+}
+
 }  // namespace
 
 padoc_status padoc_launch_prefill_bwd_tc(const void *q, const void *k, const void *v, const void *out,
                                          const void *dout, const float *lse, int64_t total_tokens,
                                          int32_t num_q_heads, int32_t num_kv_heads, const int32_t *spans_dev,
                                          const padoc_tile_map_dev *q_map, const padoc_tile_map_dev *k_map, float *lt,
-                                         float *dt, float *split, int64_t t_pad, float scale, void *dq, void *dk,
+                                         float *dt, int64_t t_pad, float scale, void *dq, void *dk,
                                          void *dv, cudaStream_t stream)
 {
     constexpr int WQ = PADOC_BWD_DQ_K_TILE;
@@ -740,7 +799,7 @@ padoc_status padoc_launch_prefill_bwd_tc(const void *q, const void *k, const voi
     if (!err) return PADOC_ERR_CUDA;
     const int64_t T = total_tokens;
     const int64_t nkt = (T + dkv::kKT - 1) / dkv::kKT, nqt = (T + CQ::kQT - 1) / CQ::kQT;
-    if (2 * nkt * num_kv_heads > INT32_MAX || nqt * num_q_heads > INT32_MAX) return PADOC_ERR_UNSUPPORTED;
+    if (8 * nkt * num_kv_heads > INT32_MAX || nqt * num_q_heads > INT32_MAX) return PADOC_ERR_UNSUPPORTED;
     const uint64_t qcols = (uint64_t)num_q_heads * kD, kcols = (uint64_t)num_kv_heads * kD;
     CUtensorMap q64, g64, k128, v128, kmap, vmap;
     if (!padoc_make_tmap_bf16(&q64, q, qcols, T, qcols * 2, 64, dkv::kQT) ||
@@ -763,11 +822,6 @@ padoc_status padoc_launch_prefill_bwd_tc(const void *q, const void *k, const voi
     prm.err = err;
     prm.o = nullptr;
     prm.lse = nullptr;
-    prm.split = split;
-    // the units that may split: their partials (2 halves x 2 tensors x 64 KB per KV head) fit in the
-    // workspace's PADOC_BWD_SPLIT_BYTES_PER_TOKEN bytes per token of t_pad
-    prm.split_units = (int32_t)std::min<int64_t>(nkt, t_pad * PADOC_BWD_SPLIT_BYTES_PER_TOKEN /
-                                                          ((int64_t)num_kv_heads * 4 * dkv::kKT * kD * 4));
 
     // the dQ pass first: it also writes -lse2 and D of every row for the dK/dV pass
     BwdParams pq = prm;   // dQ pass over the query-major map; Q and dO go to tensor memory
@@ -782,8 +836,7 @@ padoc_status padoc_launch_prefill_bwd_tc(const void *q, const void *k, const voi
     pq.out1 = nullptr;
     pq.o = (const __nv_bfloat16 *)out;
     pq.lse = lse;
-    PADOC_CUDA_TRY(cudaFuncSetAttribute(prefill_bwd_dq_kernel<WQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)CQ::kSmemBytes));
+    if (const padoc_status sm = padoc_set_max_smem((const void *)prefill_bwd_dq_kernel<WQ>, (int)CQ::kSmemBytes)) return sm;
     prefill_bwd_dq_kernel<WQ><<<(unsigned)(nqt * num_q_heads), kThreads, CQ::kSmemBytes, stream>>>(kmap, vmap, pq);
     padoc_status st = padoc_launch_status();
     if (st != PADOC_OK) return st;
@@ -796,12 +849,11 @@ padoc_status padoc_launch_prefill_bwd_tc(const void *q, const void *k, const voi
     pk.num_tiles = (int32_t)nkt;
     pk.out0 = (__nv_bfloat16 *)dk;
     pk.out1 = (__nv_bfloat16 *)dv;
-    PADOC_CUDA_TRY(cudaFuncSetAttribute(prefill_bwd_dkv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)dkv::kSmemBytes));
-    prefill_bwd_dkv_kernel<<<(unsigned)(2 * nkt * num_kv_heads), kThreads, dkv::kSmemBytes, stream>>>(q64, g64, k128,
-                                                                                                       v128, pk);
-    st = padoc_launch_status();
-    if (st != PADOC_OK || pk.split_units == 0) return st;
-    prefill_bwd_dkv_merge_kernel<<<(unsigned)(pk.split_units * num_kv_heads), 256, 0, stream>>>(pk);
-    return padoc_launch_status();
+    const int64_t units = nkt * num_kv_heads;
+    switch (pick_cluster(units)) {
+        case 8: return launch_dkv<8>(q64, g64, k128, v128, pk, units, stream);
+        case 4: return launch_dkv<4>(q64, g64, k128, v128, pk, units, stream);
+        case 2: return launch_dkv<2>(q64, g64, k128, v128, pk, units, stream);
+        default: return launch_dkv<1>(q64, g64, k128, v128, pk, units, stream);
+    }
 }
