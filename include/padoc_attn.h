@@ -410,8 +410,9 @@ padoc_status padoc_append_inputs_e4m3(const padoc_kv_pool_e4m3 *pool, const void
 /* padoc_branch_decode_attn over an E4M3 pool: the same plans (padoc_build_decode_plan and the other
  * planners, built with the same padoc_decode_config), tables, workspace and results; q, out bf16
  * [num_streams][Hq][128], lse fp32. Attention is over the dequantized values code_value * scale:
- * codes become bf16 exactly in shared memory, the K scale multiplies each 16-token block's scores
- * and the V scale the block's probabilities in fp32 before they are rounded to bf16. Hq / Hkv = 8,
+ * codes become f16 exactly, each query row f16 under a power-of-two scale, the K scale multiplies each
+ * 16-token block's scores and the V scale the block's probabilities in fp32 before they are rounded to
+ * f16. Hq / Hkv = 8,
  * block_size 16, head_dim 128. Errors: INVALID_ARGUMENT, UNSUPPORTED, WORKSPACE_TOO_SMALL, CUDA. */
 padoc_status padoc_branch_decode_attn_e4m3(const padoc_kv_pool_e4m3 *pool, const padoc_decode_plan *info,
                                            const int32_t *plan_dev, const int32_t *page_block_table,

@@ -128,6 +128,20 @@ __device__ __forceinline__ void st_cluster_v4(uint32_t addr, int4 v)
                  : "memory");
 }
 
+// Whether the phase with the given parity has completed; never suspends.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n"
+        " mbarrier.test_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 // Waits for the phase with the given parity to complete; false (and the error word set to
 // PADOC_DEVERR_TIMEOUT with `site` as the detail) if it does not complete within limit_ns.
 __device__ __forceinline__ bool mbar_wait_bounded_ns(uint32_t bar, uint32_t parity, int *err, int site,
@@ -313,6 +327,14 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint32_t (&a
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+__device__ __forceinline__ void mma_f16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
 __device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr)
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
@@ -359,17 +381,29 @@ __device__ __forceinline__ uint32_t e4m3x2_to_f16x2(uint16_t c)
     return h;
 }
 
-// Two codes to a bf16x2 holding code_value * 2^-112, exactly: the f16 bits with the exponent and
-// the top 7 mantissa bits moved down three places (E4M3 values use only the top 3 of f16's 10
-// mantissa bits) read as bf16 with exponent field 0..23 instead of f16's biased exponent, i.e.
-// the value times 2^(15 - 127); every nonzero result is a bf16 normal (no subnormal operand
-// reaches the tensor cores). Callers fold 2^112 into the scale they apply.
-#define PADOC_E4M3_BF16_SHIFT_LOG2 112
-__device__ __forceinline__ uint32_t e4m3x2_to_bf16x2_shifted(uint16_t c)
+// Two fp32 values to an f16x2, nearest even (lo in the low half).
+__device__ __forceinline__ uint32_t pack_f16x2(float lo, float hi)
 {
-    const uint32_t h = e4m3x2_to_f16x2(c);
-    const uint32_t mag = (h & 0x7FFF7FFFu) >> 3;   // the high half's low mantissa bits are zero
-    return mag | (h & 0x80008000u);
+    const __half2 v = __floats2half2_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&v);
+}
+
+// f16 operands for the E4M3 path. A row of queries (bf16) is scaled by a power of two so that its
+// largest magnitude lies in [2^14, 2^15): elements down to 2^-28 of it stay f16 normals, so nothing is
+// rounded that fp32 sums of the products keep. `scale` and its inverse from the row's largest magnitude.
+__device__ __forceinline__ void f16_row_scale(float amax, float &scale, float &inverse)
+{
+    const int e = min(max((int)(__float_as_uint(amax) >> 23) - 127, -112), 127);
+    scale = __uint_as_float((uint32_t)(14 - e + 127) << 23);
+    inverse = __uint_as_float((uint32_t)(e - 14 + 127) << 23);
+}
+__device__ __forceinline__ uint32_t bf16x2_to_f16x2(uint32_t w, float scale)
+{
+    return pack_f16x2(__uint_as_float(w << 16) * scale, __uint_as_float(w & 0xFFFF0000u) * scale);
+}
+__device__ __forceinline__ float bf16x2_amax(float a, uint32_t w)
+{
+    return fmaxf(a, fmaxf(fabsf(__uint_as_float(w << 16)), fabsf(__uint_as_float(w & 0xFFFF0000u))));
 }
 
 // The exact fp32 value of one code.

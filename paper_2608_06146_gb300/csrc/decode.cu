@@ -23,32 +23,6 @@ namespace {
 
 using namespace padoc_warp;
 
-constexpr size_t kDecodeSmemE4M3 = 1024 + kRingBytesE4M3;   // + the slack to align the base by hand
-
-// The warp lists as a grid of their own (the E4M3 pool), 8 warps per CTA, launched as a programmatic
-// dependent of the tensor-core grid when there is one. Warp CTA c is CTA c: the first ones take the
-// SMs the tensor-core grid leaves free, the others start as its CTAs end.
-template <bool kE4M3>
-__global__ void __launch_bounds__(kWarps * 32, 1)
-decode_warp_kernel(const DecodeParams prm, int after_tc)
-{
-    // the merge that follows waits for this whole grid before it reads anything, so it may launch now
-    pdl_launch_dependents();
-    // Without a tensor-core grid this grid is a programmatic dependent of whatever kernel precedes
-    // it in the stream (the previous step's merge, which may still read partials, or the kernel
-    // that wrote the queries and the new K/V rows): it waits for that kernel before any global
-    // access, so only its launch overlaps the previous kernel. After a tensor-core grid (which waited
-    // for that kernel already) each warp waits for it before it ends, so that the merge sees both
-    // grids' partials.
-    if (!after_tc) pdl_wait_prerequisite();
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int wi = blockIdx.x * kWarps + warp;
-    if (wi < prm.num_warps) decode_warp_role<kE4M3>(prm, smem, warp, lane, wi);
-    if (after_tc) pdl_wait_prerequisite();
-}
-
 // ------------------------------------------------------------------------------------------------
 // Split-K merge (C4): one warp per output row, 4 consecutive dims per lane.
 // ------------------------------------------------------------------------------------------------
@@ -452,31 +426,12 @@ padoc_status decode_split_k(const DecodePool &pl, const padoc_decode_plan *info,
     prm.part_lse = part_lse;
     prm.scale_log2 = sl2;
     prm.err = err;
-    // the decode grid: tensor-core pieces, then (bf16: on those CTAs and on the SMs they leave free)
-    // the warp lists
+    // the decode grid: tensor-core pieces, then (on those CTAs and on the SMs they leave free) the warp lists
     padoc_status st = padoc_launch_decode_tc(&kmap, &vmap, &qmap, plan, info, page_block_table, page_table_stride,
                                              stream_block_table, stream_table_stride, pl.num_blocks,
                                              pl.e4m3 ? pl.k_scales : nullptr, pl.e4m3 ? pl.v_scales : nullptr,
                                              part_o, part_lse, (__nv_bfloat16 *)out, lse, sl2, err, &prm, cs);
     if (st != PADOC_OK) return st;
-    if (pl.e4m3 && prm.num_warps > 0) {   // E4M3: the warp lists in a grid of their own
-        const int after_tc = info->num_tc_items > 0 ? 1 : 0;
-        st = padoc_set_max_smem(reinterpret_cast<const void *>(decode_warp_kernel<true>), (int)kDecodeSmemE4M3);
-        if (st != PADOC_OK) return st;
-        cudaLaunchConfig_t lc = {};
-        lc.gridDim = dim3((unsigned)((prm.num_warps + kWarps - 1) / kWarps));
-        lc.blockDim = dim3(kWarps * 32);
-        lc.dynamicSmemBytes = kDecodeSmemE4M3;
-        lc.stream = cs;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        lc.attrs = attr;
-        lc.numAttrs = 1;
-        PADOC_CUDA_TRY(cudaLaunchKernelEx(&lc, decode_warp_kernel<true>, prm, after_tc));
-        st = padoc_launch_status();
-        if (st != PADOC_OK) return st;
-    }
     if (info->num_merge_keys > 0) {   // the keys with more than one partial (or a warp item's one)
         cudaLaunchConfig_t lc = {};
         lc.gridDim = dim3((unsigned)info->num_merge_keys);

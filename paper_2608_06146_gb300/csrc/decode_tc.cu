@@ -32,15 +32,21 @@
 // first item flagged PADOC_ITEM_CONT): the second item keeps the queries, the softmax state and O
 // (its first PV accumulates), and only it writes the partial.
 //
-// FP8 (E4M3) pool (kE4M3): each paged block's codes (16 rows x 128 bytes) land by TMA in the upper
-// half of the tile's ring slot, and the producer warp that loaded them expands them in place into
-// the bf16 panels the MMAs read (each lane owns whole rows, reads a row's codes before writing it;
-// codes times 2^-112 are exact bf16 values), then marks the slot full. A producer expands tile n - 2
-// (K) or n - 1 (V) before it issues tile n, so loads stay in flight while it converts. The K
-// producer also copies each block's K and V scales into a ring of 8 entries, one per tile; the
-// softmax applies the K scale to the block's scores and folds the V scale into the block's
-// probabilities before they are rounded to bf16, and removes it again from their row sum.
+// FP8 (E4M3) pool (kE4M3): the MMAs take f16 operands, into which codes convert exactly at one
+// instruction per two values (into bf16 it takes four, and the expanding warps set the pace: 59 us for
+// the serving batch's pieces alone, against 47 us for the whole bf16 grid). Each paged block's codes
+// (16 rows x 128 bytes) land by TMA in the upper half of the tile's ring slot, and the producer warp that
+// loaded them expands them in place into the f16 panels the MMAs read (each lane owns whole rows, reads a
+// row's codes before writing it), then marks the slot full. A producer expands what has
+// landed whenever it would wait. The softmax warps turn each
+// piece's queries into f16, every row scaled by a power of two. The K producer also copies each block's
+// K and V scales into a ring of 4 entries, one per tile; the softmax applies the K scale to the block's
+// scores and folds the V scale into the block's probabilities before they are rounded to f16, and
+// removes it again from their row sum. The running maximum is that of score + log2(V scale), so that the
+// probabilities, times 2^6, fill f16's range whatever the scales.
 #include <math.h>
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "decode_warp.cuh"
@@ -72,25 +78,28 @@ enum {
     B_FINAL = 18,
     B_KSTG = 19,     // [K stage] E4M3: the tile's codes have landed
     B_VSTG = 22,     // [V stage] E4M3
-    B_SCL = 24,      // [scale entry] E4M3: the tile's scales have landed (one arrival per loading lane)
-    B_COUNT = 32
+    B_SCLRAW = 24,   // [scale entry] E4M3: the tile's scales have landed (one arrival per loading lane)
+    B_SCL = 28,      // [scale entry] E4M3: the softmax's factors are in place
+    B_QCVT = 32,     // E4M3: the piece's queries are f16, one arrival per softmax warp
+    B_COUNT = 33
 };
-constexpr int kSclEntries = 8;   // scale ring: entry n % 8 for tile n
+// scale ring: entry n % 4 for tile n (tile n is issued after the QK^T of tile n - 3, which follows the
+// softmax of tile n - 4): the K and V scales of the tile's 8 blocks as they land (16 floats), then what
+// the softmax reads: K factors, log2 of the V scales, and their inverses (8 floats each)
+constexpr int kSclEntries = 4, kSclFloats = 40;
 
 constexpr int kSoftmaxWarps = 8;
 constexpr int kXchBytes = 2 * 2 * 128 * 4;   // row max / sum swap: [buffer][column half][row] floats
-// Q (two M-tiles), the K and V rings, then barriers (256 bytes), the TMEM address and abort flag,
-// the scale ring (E4M3: [8 entries][8 K scales, 8 V scales]) and the swap buffer: 232,448 bytes,
+// Q (two M-tiles), the K and V rings, then barriers, the TMEM address and abort flag,
+// the scale ring (E4M3: [4 entries][40 floats]) and the swap buffer: 232,448 bytes,
 // the most a CTA may have, so there is no room to align the start by hand; the kernel checks that
 // the driver placed it on a 1024-byte boundary (the base of a CTA's dynamic shared memory is) and
 // refuses to run otherwise.
 constexpr size_t kTilesBytes = (size_t)kTile * (2 + kKStages + kVStages);
-constexpr int kMiscScl = 320, kMiscXch = 1024;
+constexpr int kMiscTmem = 272, kMiscScl = 288, kMiscXch = 1024;
 constexpr size_t kSmemBytes = kTilesBytes + kMiscXch + kXchBytes;
 static_assert(kSmemBytes <= 232448, "shared memory per CTA");
-static_assert(B_COUNT * 8 <= 256 && kMiscScl + kSclEntries * 16 * 4 <= kMiscXch, "misc layout");
-constexpr float kTwo112 = 5.192296858534828e33f;   // 2^112: the bf16 expansion's factor
-static_assert(PADOC_E4M3_BF16_SHIFT_LOG2 == 112, "expansion factor");
+static_assert(B_COUNT * 8 <= kMiscTmem && kMiscScl + kSclEntries * kSclFloats * 4 <= kMiscXch, "misc layout");
 
 struct TcDecodeParams {
     const int32_t *shared_len, *private_len, *slot_ptr, *cta_ptr;
@@ -141,7 +150,7 @@ __device__ __forceinline__ const int32_t *item_row(const TcDecodeParams &prm, co
     return (priv ? prm.stream_table : prm.page_table) + (size_t)it.index * stride;
 }
 
-// E4M3: expands one landed tile of codes in place into the slot's two bf16 panels. Lane l owns
+// E4M3: expands one landed tile of codes in place into the slot's two f16 panels. Lane l owns
 // rows l, l + 32, l + 64, l + 96; it reads a row's eight 16-byte chunks of codes (swizzled by row,
 // in the upper half of the slot, where the row's panel-1 bytes go) before it writes the row.
 __device__ __forceinline__ void expand_tile(uint8_t *slot, int lane)
@@ -160,10 +169,10 @@ __device__ __forceinline__ void expand_tile(uint8_t *slot, int lane)
             for (int hh = 0; hh < 2; ++hh) {   // dims 16c + 8hh .. + 7: chunk 2c + hh of the row
                 const int kk = 2 * c + hh;
                 uint4 o;
-                o.x = e4m3x2_to_bf16x2_shifted((uint16_t)(w[2 * hh] & 0xFFFFu));
-                o.y = e4m3x2_to_bf16x2_shifted((uint16_t)(w[2 * hh] >> 16));
-                o.z = e4m3x2_to_bf16x2_shifted((uint16_t)(w[2 * hh + 1] & 0xFFFFu));
-                o.w = e4m3x2_to_bf16x2_shifted((uint16_t)(w[2 * hh + 1] >> 16));
+                o.x = e4m3x2_to_f16x2((uint16_t)(w[2 * hh] & 0xFFFFu));
+                o.y = e4m3x2_to_f16x2((uint16_t)(w[2 * hh] >> 16));
+                o.z = e4m3x2_to_f16x2((uint16_t)(w[2 * hh + 1] & 0xFFFFu));
+                o.w = e4m3x2_to_f16x2((uint16_t)(w[2 * hh + 1] >> 16));
                 *reinterpret_cast<uint4 *>(slot + (kk >> 3) * kPanel + r * 128 + (((kk & 7) ^ (r & 7)) << 4)) = o;
             }
         }
@@ -200,9 +209,9 @@ __device__ __forceinline__ void prefetch_warp_lists(const padoc_warp::DecodePara
 }
 
 // The pieces of tensor-core CTA blockIdx.x (every thread of the CTA; smem 1024-byte aligned).
-// kFused: the CTA runs warp lists next (their first blocks are pulled into L2 meanwhile). kSole:
-// the plan has PADOC_ITEM_SOLE items (otherwise their output path is compiled out).
-template <bool kE4M3, bool kFused, bool kSole>
+// The CTA runs warp lists next (their first blocks are pulled into L2 meanwhile). kSole: the plan has
+// PADOC_ITEM_SOLE items (otherwise their output path is compiled out).
+template <bool kE4M3, bool kSole>
 __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CUtensorMap &vmap, const CUtensorMap &qmap,
                                                const TcDecodeParams &prm, const padoc_warp::DecodeParams &wprm,
                                                uint8_t *smem)
@@ -212,8 +221,8 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
     uint8_t *sv = sk + kKStages * kTile;
     uint8_t *misc = smem + kTilesBytes;
     uint64_t *bars = (uint64_t *)misc;
-    uint32_t *tmem_slot = (uint32_t *)(misc + 256);
-    volatile int *abort_flag = (volatile int *)(misc + 260);
+    uint32_t *tmem_slot = (uint32_t *)(misc + kMiscTmem);
+    volatile int *abort_flag = (volatile int *)(misc + kMiscTmem + 4);
     float *scl = (float *)(misc + kMiscScl);   // E4M3: [entry][K scales of 8 blocks, V scales of 8 blocks]
     float *xch = (float *)(misc + kMiscXch);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -252,7 +261,8 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                                           : (i == B_QFREE || (i >= B_KEMPTY && i < B_KEMPTY + kKStages) ||
                                              (i >= B_VEMPTY && i < B_VEMPTY + kVStages) || i == B_FINAL)
                                                 ? 2     // one commit from each MMA warp
-                                          : (i >= B_SCL) ? kKT / kBlk   // one per lane that loads a block
+                                          : (i >= B_SCLRAW && i < B_SCLRAW + kSclEntries) ? kKT / kBlk   // one per lane that loads a block
+                                          : (i == B_QCVT) ? kSoftmaxWarps
                                                 : 1);
         *abort_flag = 0;
         fence_barrier_init();
@@ -320,21 +330,61 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
         };
         if (u0 < u1) fetch_id(u0, 0);
         int n = 0, nq = 0;   // tiles and query sets issued
-        // E4M3: tiles expanded so far; a tile is expanded `lag` tiles after it is issued (K runs
-        // further ahead: its ring has three slots)
+        // E4M3: tiles expanded so far. While the producer waits for a barrier it expands every tile whose
+        // codes have landed, so that a slot is refilled as soon as it is free and no expansion waits for
+        // the next one to be (expanding tile n - 1 before issuing tile n kept one V load in flight).
         int nc = 0;
-        const int lag = is_k ? 2 : 1;
+        float vl_last = -90.f;   // (K producer) log2 of the last nonzero V scale
         const int b_stg = is_k ? B_KSTG : B_VSTG;
         auto expand_next = [&]() {   // whole warp; nc counts only tiles whose codes have landed
-            const int t = nc;
-            const int st = t % nst;
-            bool r = wait_or_abort(bar(b_stg + st), (t / nst) & 1, prm.err, is_k ? 56 : 57, abort_flag);
-            r = __all_sync(0xffffffffu, r);
-            if (!r) return false;
+            const int st = nc % nst;
             ++nc;
             expand_tile(ring + st * kTile, lane);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(b_full + st));
+            if (is_k) {
+                // the tile's factors for the softmax, block l by lane l. A zero scale marks a block without
+                // a nonzero value (its codes are zeros): any positive factor gives the same result there,
+                // and the last nonzero V scale keeps the range.
+                const int t = nc - 1, e = t % kSclEntries;
+                mbar_wait_bounded(bar(B_SCLRAW + e), (t / kSclEntries) & 1, prm.err, 58);
+                float *f = scl + e * kSclFloats;
+                const int b = lane & 7;
+                const float ks = f[b], vs = f[8 + b];
+                float vl = vs > 0.f ? fmaxf(__log2f(vs), -100.f) : INFINITY;
+#pragma unroll
+                for (int d = 1; d < 8; ++d) {   // a zero scale takes the nearest block's before it
+                    const float o = __shfl_up_sync(0xffffffffu, vl, 1, 8);
+                    if (vl == INFINITY && b > 0) vl = o;
+                }
+                if (vl == INFINITY) vl = vl_last;
+                vl_last = __shfl_sync(0xffffffffu, vl, 7, 8);
+                if (lane < 8) {
+                    f[16 + b] = ks > 0.f ? ks : 1.f;
+                    f[24 + b] = vl;
+                    f[32 + b] = fast_exp2(-vl);
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(B_SCL + e));
+            }
+        };
+        auto landed = [&]() { return __all_sync(0xffffffffu, mbar_test(bar(b_stg + nc % nst), (nc / nst) & 1)); };
+        auto wait_expanding = [&](int b, uint32_t parity, int issued, int site) {
+            if (!kE4M3) return wait_or_abort(bar(b), parity, prm.err, site, abort_flag);
+            const uint64_t t0 = padoc_globaltimer();
+            for (uint32_t i = 1; !__all_sync(0xffffffffu, mbar_test(bar(b), parity)); ++i) {
+                if (nc < issued && landed()) {
+                    expand_next();
+                } else if ((i & 255u) == 0) {
+                    bool out = *abort_flag != 0;
+                    if (!out && padoc_globaltimer() - t0 > PADOC_WAIT_LIMIT_NS) {
+                        padoc_record_error(prm.err, PADOC_DEVERR_TIMEOUT, site);
+                        *abort_flag = 1;
+                        out = true;
+                    }
+                    if (__any_sync(0xffffffffu, out)) return false;
+                }
+            }
             return true;
         };
         // the first piece's queries go out before anything else (they wait for nothing)
@@ -364,10 +414,7 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                     else if (is_k) padoc_record_error(prm.err, PADOC_DEVERR_BLOCK_ID, id);
                 }
                 const int s = n % nst, use = n / nst;
-                if (kE4M3)
-                    while (ok && nc <= n - lag) ok = expand_next();
-                if (!ok) break;
-                if (use > 0) ok = wait_or_abort(bar(b_empty + s), (use - 1) & 1, prm.err, is_k ? 50 : 53, abort_flag);
+                if (use > 0) ok = wait_expanding(b_empty + s, (use - 1) & 1, n, is_k ? 50 : 53);
                 if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
                 const uint64_t kv_policy = (it.kind & PADOC_ITEM_REREAD) ? shared_policy : once_policy;
                 if constexpr (kE4M3) {
@@ -382,10 +429,10 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                         if (is_k) {
                             const bool okid = row != prm.pool_rows;
                             const size_t si = okid ? (size_t)id * prm.num_kv_heads + it.kv_head : 0;
-                            float *e = scl + (n % kSclEntries) * 16;
+                            float *e = scl + (n % kSclEntries) * kSclFloats;
                             cp_async_4(smem_u32(e + lane), prm.k_scales + si, okid ? 4u : 0u);
                             cp_async_4(smem_u32(e + 8 + lane), prm.v_scales + si, okid ? 4u : 0u);
-                            cp_async_mbar_arrive(bar(B_SCL + n % kSclEntries));
+                            cp_async_mbar_arrive(bar(B_SCLRAW + n % kSclEntries));
                         }
                     }
                 } else {
@@ -399,12 +446,8 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                 }
                 ++n;
                 if (is_k && j == 0 && !(q_first && u == u0) && !cont_in) {
-                    // E4M3: the previous piece's tiles must be expanded before its last QK^T can run
-                    if (kE4M3)
-                        while (ok && nc < n - 1) ok = expand_next();
-                    if (!ok) break;
                     // this piece's queries, once the previous piece's last QK^T has read the buffer
-                    if (nq > 0) ok = wait_or_abort(bar(B_QFREE), (nq - 1) & 1, prm.err, 55, abort_flag);
+                    if (nq > 0) ok = wait_expanding(B_QFREE, (nq - 1) & 1, n, 55);
                     if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
                     if (lane == 0) load_q(it, u);
                     ++nq;
@@ -414,11 +457,14 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
         // the K producer is done first (its ring runs two tiles ahead): it warms L2 for the warp lists
         // this CTA runs next (E4M3: after the last expansions below)
         const int wc = prm.early_ctas + (int)blockIdx.x;
-        if (kFused && !kE4M3 && is_k && wc < prm.warp_ctas) prefetch_warp_lists<kE4M3>(wprm, kmap, vmap, wc, lane);
+        if (!kE4M3 && is_k && wc < prm.warp_ctas) prefetch_warp_lists<kE4M3>(wprm, kmap, vmap, wc, lane);
         if constexpr (kE4M3) {
             // the last tiles' expansion; after a failed wait only their copies are waited for
-            while (ok && nc < n) ok = expand_next();
-            if (kFused && is_k && wc < prm.warp_ctas) prefetch_warp_lists<kE4M3>(wprm, kmap, vmap, wc, lane);
+            while (ok && nc < n) {
+                ok = __all_sync(0xffffffffu, wait_or_abort(bar(b_stg + nc % nst), (nc / nst) & 1, prm.err, is_k ? 56 : 57, abort_flag));
+                if (ok) expand_next();
+            }
+            if (is_k && wc < prm.warp_ctas) prefetch_warp_lists<kE4M3>(wprm, kmap, vmap, wc, lane);
             if (lane == 0)
                 for (int J = nc; J < n; ++J)
                     mbar_wait_bounded(bar(b_stg + J % nst), (J / nst) & 1, prm.err, is_k ? 51 : 52);
@@ -437,8 +483,8 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
         // MMAs on the tensor pipe. Both commit to the K/V-release, query-release and final
         // barriers (two arrivals each); on a one-M-tile piece warp 11 only commits.
         const int mi = warp == 9 ? 0 : 1;
-        constexpr uint32_t idS = umma_idesc_bf16(128, kKT, false);
-        constexpr uint32_t idPV = umma_idesc_bf16(128, kD, true);
+        constexpr uint32_t idS = kE4M3 ? umma_idesc_f16(128, kKT, false) : umma_idesc_bf16(128, kKT, false);
+        constexpr uint32_t idPV = kE4M3 ? umma_idesc_f16(128, kD, true) : umma_idesc_bf16(128, kD, true);
         const uint64_t dq = umma_desc_sw128(smem_u32(sq + mi * kTile), 16, 1024);
         // stage descriptors differ only in the start-address field (address >> 4)
         const uint64_t dk0 = umma_desc_sw128(smem_u32(sk), 16, 1024);
@@ -468,7 +514,7 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
             const bool cont_in = u > u0 && (prm.items[u - 1].kind & PADOC_ITEM_CONT);
             const bool cont_out = (it.kind & PADOC_ITEM_CONT) != 0;
             if (ne == 0) continue;
-            if ((!cont_in && !wait_w(B_Q, nq & 1, 60)) || !wait_w(B_KFULL + J % kKStages, (J / kKStages) & 1, 61)) {
+            if ((!cont_in && !wait_w(kE4M3 ? B_QCVT : B_Q, nq & 1, 60)) || !wait_w(B_KFULL + J % kKStages, (J / kKStages) & 1, 61)) {
                 ok = false;
                 break;
             }
@@ -567,6 +613,37 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
             fetch_cut();
         }
         float m0 = -INFINITY, l0 = 0.f, m1 = -INFINITY, l1 = 0.f;   // running softmax state of the piece
+        // E4M3: the queries of a piece of mt M-tiles into f16, and what takes their rows' scales off again;
+        // done for the next piece before this one's output, which then overlaps its first QK^T
+        float qk0 = 1.f, qk1 = 1.f;
+        int nqc = 0;                 // query sets converted
+        bool q_done = false;         // the next piece's are
+        auto convert_q = [&](int mt) {
+            ok = ok && wait_all(B_Q, nqc & 1, 73);
+            ++nqc;
+#pragma unroll
+            for (int mi = 0; mi < 2; ++mi) {
+                if (mi >= mt) break;
+                uint8_t *q = sq + mi * kTile + hc * kPanel + row * 128;
+                uint4 w[8];
+                float amax = 0.f, qs, qi;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    w[k] = *reinterpret_cast<const uint4 *>(q + ((k ^ (row & 7)) << 4));
+                    amax = bf16x2_amax(bf16x2_amax(bf16x2_amax(bf16x2_amax(amax, w[k].x), w[k].y), w[k].z), w[k].w);
+                }
+                f16_row_scale(fmaxf(amax, swap_row(amax)), qs, qi);
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    *reinterpret_cast<uint4 *>(q + ((k ^ (row & 7)) << 4)) =
+                        make_uint4(bf16x2_to_f16x2(w[k].x, qs), bf16x2_to_f16x2(w[k].y, qs), bf16x2_to_f16x2(w[k].z, qs),
+                                   bf16x2_to_f16x2(w[k].w, qs));
+                (mi ? qk1 : qk0) = c * qi;
+            }
+            fence_proxy_async_smem();   // the MMAs read the panels through the async proxy
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(B_QCVT));
+        };
         bool cont_in = false;   // the previous item continues into this one
         for (int u = u0; u < u1; ++u) {
             const int tb = n_tb, te = n_te, nstr = n_nstr, first = n_first, kvh = n_kvh, slot = n_slot;
@@ -582,35 +659,30 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
             };
             if (!cont_in) {   // a new piece (an item continuing the previous one keeps the state)
                 m0 = -INFINITY; l0 = 0.f; m1 = -INFINITY; l1 = 0.f;
+                if (kE4M3 && ne > 0) {
+                    if (!q_done) convert_q(mt);
+                    q_done = false;
+                }
             }
             for (int j = 0; j < ne; ++j) {
                 if (j == 1 && u + 1 < u1) fetch_cut();
                 if (j == ne - 1) fetch_slots();
-                // E4M3: for the 16-column blocks 4 hc .. 4 hc + 3 of this thread's column half, the
-                // multiplier of the raw scores (log2 units, K scale and 2^112 folded in), the V factor
-                // folded into P (as a log2 offset of the exponent) and its inverse for the row sum. A
-                // zero scale marks a block without a nonzero value (its codes are zeros): any positive
-                // factor gives the same result there.
-                float kcb[4], vlb[4], vib[4];
+                // E4M3: for the 16-column blocks 4 hc .. 4 hc + 3 of this thread's column half, the K factor,
+                // the V scale's log2 (an offset of the exponent) and its inverse for the row sum
+                float4 kcb = {}, vlb = {}, vib = {};
                 if constexpr (kE4M3) {
                     const int e = cnt0 % kSclEntries;   // cnt0: tiles so far (every piece has M-tile 0)
                     ok = ok && wait_all(B_SCL + e, (cnt0 / kSclEntries) & 1, 72);
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) {
-                        const float ks = scl[e * 16 + 4 * hc + b], vs = scl[e * 16 + 8 + 4 * hc + b];
-                        kcb[b] = c * (ks > 0.f ? ks : 1.f) * kTwo112;
-                        const float vf = (vs > 0.f ? vs : 1.f) * kTwo112;
-                        vlb[b] = __log2f(vf);
-                        vib[b] = fast_exp2(-vlb[b]);
-                    }
+                    const float4 *f = reinterpret_cast<const float4 *>(scl + e * kSclFloats + 16) + hc;
+                    kcb = f[0];
+                    vlb = f[2];
+                    vib = f[4];
                 }
-#pragma unroll
-                for (int mi = 0; mi < 2; ++mi) {
-                    if (mi >= mt) break;
+                // one M-tile's turn
+                auto turn = [&](auto mi_, float &m_ref, float &l) {
+                    const int mi = mi_;
                     const uint32_t tS = tmem + lanes + 128 * mi, tO = tS + 256;
                     const int cnt = mi ? cnt1 : cnt0;
-                    float &m_ref = mi ? m1 : m0;
-                    float &l = mi ? l1 : l0;
                     // visible columns of this half: [0, w)
                     const int w = min(max((mi ? cut1 : cut0) - (tb + j * kKT) - 64 * hc, 0), 64);
                     const bool full = __all_sync(0xffffffffu, w == 64);
@@ -618,7 +690,7 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                     if (mi) ++cnt1; else ++cnt0;
                     if (!ok) {
                         swap_row(0.f);
-                        continue;
+                        return;
                     }
                     tc_fence_after();
                     uint32_t sr[2][32];
@@ -634,7 +706,7 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                         }
                     }
                     float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-                    float mx;
+                    float mx, mul[4], vl4[4];   // E4M3: a block's score multiplier in log2 units, log2 of its V scale
                     if constexpr (kE4M3) {
                         // block b = columns 16b .. 16b + 15 of the half: its max, then times its multiplier
 #pragma unroll
@@ -645,7 +717,11 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                                 mx4[b] = fmax3f(mx4[b], __uint_as_float(sr[uu][i]), __uint_as_float(sr[uu][i + 1]));
                                 mx4[b] = fmax3f(mx4[b], __uint_as_float(sr[uu][i + 2]), __uint_as_float(sr[uu][i + 3]));
                             }
-                        mx = fmaxf(fmaxf(mx4[0] * kcb[0], mx4[1] * kcb[1]), fmaxf(mx4[2] * kcb[2], mx4[3] * kcb[3]));
+                        const float qk = mi ? qk1 : qk0;
+                        vl4[0] = vlb.x; vl4[1] = vlb.y; vl4[2] = vlb.z; vl4[3] = vlb.w;
+                        mul[0] = kcb.x * qk; mul[1] = kcb.y * qk; mul[2] = kcb.z * qk; mul[3] = kcb.w * qk;
+                        mx = fmaxf(fmax3f(fmaf(mx4[0], mul[0], vlb.x), fmaf(mx4[1], mul[1], vlb.y), fmaf(mx4[2], mul[2], vlb.z)),
+                                   fmaf(mx4[3], mul[3], vlb.w));
                     } else {
 #pragma unroll
                         for (int uu = 0; uu < 2; ++uu)
@@ -671,63 +747,76 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                         l *= alpha;
                         m_ref = m_new;
                     }
-                    const float moff = m_ref == -INFINITY ? 0.f : m_ref * cm;
-                    float rs[4] = {0.f, 0.f, 0.f, 0.f};
+                    // (E4M3: P times 2^6)
+                    const float moff = m_ref == -INFINITY ? 0.f : kE4M3 ? m_ref - 6.f : m_ref * cm;
+                    // two columns per packed instruction; E4M3: P of block b carries its V factor (the
+                    // exponent's log2 offset), which comes off again in the row sum
+                    uint64_t rs2[4] = {0ull, 0ull, 0ull, 0ull};
                     uint32_t pk[32];
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) {
+                        const float mb = kE4M3 ? mul[b] : c, ob = kE4M3 ? vl4[b] - moff : -moff;
+                        const uint64_t m2 = f2_pack(mb, mb), o2 = f2_pack(ob, ob);
+#pragma unroll
+                        for (int i = 16 * (b & 1); i < 16 * (b & 1) + 16; i += 2) {
+                            float x0, x1;
+                            f2_unpack(f2_fma(f2_pack(__uint_as_float(sr[b >> 1][i]), __uint_as_float(sr[b >> 1][i + 1])), m2, o2),
+                                      x0, x1);
+                            const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
+                            rs2[b] = f2_add(rs2[b], f2_pack(p0, p1));
+                            pk[16 * (b >> 1) + (i >> 1)] = kE4M3 ? pack_f16x2(p0, p1) : pack_bf16x2(p0, p1);
+                        }
+                    }
+                    tmem_st32(tS + 32 * hc, pk);   // P (pairs) of columns [64 hc, 64 hc + 64)
                     if constexpr (kE4M3) {
-                        // P of block b carries its V factor (the exponent's log2 offset); rs[b] sums the
-                        // block's carried values, and the factor comes off again in the row sum
-#pragma unroll
-                        for (int qq = 0; qq < 2; ++qq) {
-#pragma unroll
-                            for (int i = 0; i < 32; i += 2) {
-                                const int b = 2 * qq + (i >> 4);
-                                const float off = vlb[b] - moff;
-                                const float p0 = fast_exp2(fmaf(__uint_as_float(sr[qq][i]), kcb[b], off));
-                                const float p1 = fast_exp2(fmaf(__uint_as_float(sr[qq][i + 1]), kcb[b], off));
-                                rs[b] += p0 + p1;
-                                pk[qq * 16 + (i >> 1)] = pack_bf16x2(p0, p1);
-                            }
-                        }
-                        tmem_st32(tS + 32 * hc, pk);
-                        l += (rs[0] * vib[0] + rs[1] * vib[1]) + (rs[2] * vib[2] + rs[3] * vib[3]);
+                        float a, b;
+                        f2_unpack(f2_fma(rs2[0], f2_pack(vib.x, vib.x), f2_fma(rs2[1], f2_pack(vib.y, vib.y),
+                                         f2_fma(rs2[2], f2_pack(vib.z, vib.z), f2_mul(rs2[3], f2_pack(vib.w, vib.w))))), a, b);
+                        l += a + b;
                     } else {
-#pragma unroll
-                        for (int qq = 0; qq < 2; ++qq) {
-#pragma unroll
-                            for (int i = 0; i < 32; i += 2) {
-                                const float p0 = fast_exp2(fmaf(__uint_as_float(sr[qq][i]), c, -moff));
-                                const float p1 = fast_exp2(fmaf(__uint_as_float(sr[qq][i + 1]), c, -moff));
-                                rs[(i >> 1) & 3] += p0 + p1;
-                                pk[qq * 16 + (i >> 1)] = pack_bf16x2(p0, p1);
-                            }
-                        }
-                        tmem_st32(tS + 32 * hc, pk);   // P (bf16 pairs) of columns [64 hc, 64 hc + 64)
-                        l += (rs[0] + rs[1]) + (rs[2] + rs[3]);
+                        float a, b;
+                        f2_unpack(f2_add(f2_add(rs2[0], rs2[1]), f2_add(rs2[2], rs2[3])), a, b);
+                        l += a + b;
                     }
                     if (__any_sync(0xffffffffu, rescale)) {
                         // PV_i(j-1) completed before S_i(j) (issue order) and PV_i(j) waits for this
                         // warp's P, so O_i is quiescent here
-#pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            uint32_t o[32];
-                            tmem_ld32(tO + 64 * hc + q * 32, o);
+#pragma unroll 1   // (rare; unrolled it takes registers from every tile)
+                        for (int q = 0; q < 4; ++q) {
+                            uint32_t o[16];
+                            tmem_ld16(tO + 64 * hc + q * 16, o);
                             tmem_ld_wait();
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-                            tmem_st32(tO + 64 * hc + q * 32, o);
+                            for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                            tmem_st16(tO + 64 * hc + q * 16, o);
                         }
                     }
                     tmem_st_wait();
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(B_PFULL + mi));
+                };
+                if constexpr (kE4M3) {   // one copy of the longer code (53.7 -> 51.5 us for the serving batch)
+#pragma unroll 1
+                    for (int mi = 0; mi < mt; ++mi) {
+                        float m = mi ? m1 : m0, ll = mi ? l1 : l0;
+                        turn(mi, m, ll);
+                        if (mi) { m1 = m; l1 = ll; }
+                        else { m0 = m; l0 = ll; }
+                    }
+                } else {                 // (one copy of the bf16 code spills: chunks 680 against 640 us)
+                    turn(std::integral_constant<int, 0>{}, m0, l0);
+                    if (mt == 2) turn(std::integral_constant<int, 1>{}, m1, l1);
                 }
             }
             if (ne < 2 && u + 1 < u1) fetch_cut();
             if (ne == 0) fetch_slots();
             cont_in = cont_out;
             if (cont_out) continue;   // the piece goes on in the next item
+            if (kE4M3 && u + 1 < u1 && n_te > n_tb) {
+                convert_q(n_nstr > 16 ? 2 : 1);
+                q_done = true;
+            }
             // partials of this piece: O / l (fp32) and the natural-log LSE of every row
 #pragma unroll
             for (int mi = 0; mi < 2; ++mi) {
@@ -778,7 +867,7 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                     }
                 }
                 if (valid && hc == 0) {
-                    const float lv = empty ? -INFINITY : (m_ref * cm + log2f(l)) * PADOC_LN2;
+                    const float lv = empty ? -INFINITY : (m_ref * cm - (kE4M3 ? 6.f : 0.f) + log2f(l)) * PADOC_LN2;
                     if (sole) prm.lse[orow] = lv; else prm.part_lse[prow] = lv;
                 }
             }
@@ -801,14 +890,12 @@ static_assert(padoc_warp::kRingBytes <= kSmemBytes && padoc_warp::kRingBytesE4M3
 static_assert(padoc_warp::kWarps * 32 == 256, "the warp path runs on warpgroups 0 and 1");
 
 
-// The decode grid (kFused): a CTA runs its tensor-core pieces (CTAs below tc_ctas), then one warp
-// CTA's lists on warps 0-7 with the larger register budget (decode_warp.cuh); warps 8-11 give their
-// registers back and end. A plan without tensor-core work runs warp CTAs only. Without kFused the
-// grid runs the tensor-core pieces only (the E4M3 pool, whose warp lists run in a grid of their own:
-// there the warp path needs more registers than the split leaves it). kPreWait: the previous kernel
-// in the stream is the step's append (a decoding loop's step), and the warps of CTAs without
-// tensor-core pieces start their first paged blocks before they wait for it.
-template <bool kE4M3, bool kFused, bool kSole, bool kPreWait>
+// The decode grid: a CTA runs its tensor-core pieces (CTAs below tc_ctas), then one warp CTA's lists on
+// warps 0-7 with the larger register budget (decode_warp.cuh); warps 8-11 give their registers back and
+// end. A plan without tensor-core work runs warp CTAs only. kPreWait: the previous kernel in the stream is
+// the step's append (a decoding loop's step), and the warps of CTAs without tensor-core pieces start their
+// first paged blocks before they wait for it.
+template <bool kE4M3, bool kSole, bool kPreWait>
 __global__ void __launch_bounds__(kThreads, 1)
 decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                  const __grid_constant__ CUtensorMap qmap, const TcDecodeParams prm,
@@ -820,12 +907,8 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
         return;
     }
     const bool has_tc = (int)blockIdx.x < prm.tc_ctas;
-    if constexpr (!kFused) {
-        if (has_tc) decode_tc_role<kE4M3, false, kSole>(kmap, vmap, qmap, prm, wprm, smem);
-        return;
-    }
     if (has_tc) {
-        decode_tc_role<kE4M3, true, kSole>(kmap, vmap, qmap, prm, wprm, smem);
+        decode_tc_role<kE4M3, kSole>(kmap, vmap, qmap, prm, wprm, smem);
     } else if constexpr (!kPreWait) {
         // a CTA with warp lists only: the same wait for the previous kernel in the stream (kPreWait:
         // each warp of the warp path waits itself, after its first loads)
@@ -861,8 +944,7 @@ padoc_status padoc_launch_decode_tc(const CUtensorMap *kmap, const CUtensorMap *
                                     const padoc_warp::DecodeParams *wprm, cudaStream_t stream)
 {
     const bool e4m3 = k_scales != nullptr;   // an E4M3 pool: the maps hold codes
-    const bool fused = !e4m3;
-    if (info->num_tc_items == 0 && (!fused || wprm->num_warps == 0)) return PADOC_OK;
+    if (info->num_tc_items == 0 && wprm->num_warps == 0) return PADOC_OK;
     TcDecodeParams prm;
     prm.shared_len = plan + info->off_shared_len;
     prm.private_len = plan + info->off_private_len;
@@ -889,16 +971,16 @@ padoc_status padoc_launch_decode_tc(const CUtensorMap *kmap, const CUtensorMap *
     prm.scale_log2 = scale_log2;
     prm.err = err;
     prm.tc_ctas = info->num_tc_items > 0 ? info->tc_ctas : 0;
-    prm.warp_ctas = fused ? (wprm->num_warps + padoc_warp::kWarps - 1) / padoc_warp::kWarps : 0;
+    prm.warp_ctas = (wprm->num_warps + padoc_warp::kWarps - 1) / padoc_warp::kWarps;
     prm.early_ctas = padoc_fused_early_ctas(prm.tc_ctas, prm.warp_ctas, padoc_default_ctas());
     // plans with sole items (chunked prefill) take the variant that writes their outputs
     const bool sole = (int64_t)info->num_merge_keys < (int64_t)info->num_streams * info->cfg.num_kv_heads;
     // a decoding-loop step right after its append (no sole items): warps of warp-only CTAs load
     // before they wait
-    const bool pre_wait = fused && wprm->pre_wait && !sole;
-    auto kern = e4m3       ? (sole ? decode_tc_kernel<true, false, true, false> : decode_tc_kernel<true, false, false, false>)
-                : pre_wait ? decode_tc_kernel<false, true, false, true>
-                           : (sole ? decode_tc_kernel<false, true, true, false> : decode_tc_kernel<false, true, false, false>);
+    const bool pre_wait = !e4m3 && wprm->pre_wait && !sole;
+    auto kern = e4m3       ? (sole ? decode_tc_kernel<true, true, false> : decode_tc_kernel<true, false, false>)
+                : pre_wait ? decode_tc_kernel<false, false, true>
+                           : (sole ? decode_tc_kernel<false, true, false> : decode_tc_kernel<false, false, false>);
     {
         const padoc_status ast = padoc_set_max_smem(reinterpret_cast<const void *>(kern), (int)kSmemBytes);
         if (ast != PADOC_OK) return ast;

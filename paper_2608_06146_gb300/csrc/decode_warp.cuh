@@ -29,16 +29,14 @@ constexpr int kBoxBytes = kBlk * 128;  // one 16-row x 64-column box
 constexpr int kWStageBytes = 4 * kBoxBytes;   // K lo, K hi, V lo, V hi
 constexpr int kWarpRing = kWStages * kWStageBytes;
 // E4M3 pool: a stage holds a block's K and V codes ([16 rows][128 bytes] each, 16-byte chunks
-// swizzled by row) and its two scales; each warp expands the block it works on into one bf16
-// buffer laid out as a bf16 stage, which the MMAs read.
+// swizzled by row) and its two scales. Half the bytes a block: six stages keep as much in flight.
+constexpr int kE8Stages = 6;
 constexpr int kE8Rows = kBlk * 128;                  // 2 KB of codes per tensor
 constexpr int kE8StageBytes = 2 * kE8Rows + 128;     // K codes, V codes, scales (k, v)
-constexpr int kE8WarpBytes = kWStages * kE8StageBytes + kWStageBytes;
+constexpr int kE8WarpBytes = kE8Stages * kE8StageBytes;
 // shared memory of the kWarps warps' rings, from a 1024-byte-aligned base
 constexpr size_t kRingBytes = (size_t)kWarps * kWarpRing;
 constexpr size_t kRingBytesE4M3 = (size_t)kWarps * kE8WarpBytes;
-constexpr float kTwo112 = 5.192296858534828e33f;     // 2^112: the bf16 expansion's factor
-static_assert(PADOC_E4M3_BF16_SHIFT_LOG2 == 112, "expansion factor");
 
 struct DecodeParams {
     const int32_t *stream_page, *shared_len, *private_len, *slot_ptr;
@@ -78,7 +76,7 @@ template <bool kE4M3, bool kPreWait = false>
 __device__ __forceinline__ void decode_warp_role(const DecodeParams &prm, uint8_t *smem, int warp, int lane, int wi)
 {
     uint8_t *wbuf = smem + (size_t)warp * (kE4M3 ? kE8WarpBytes : kWarpRing);
-    uint8_t *cbuf = wbuf + kWStages * kE8StageBytes;   // E4M3: the expanded bf16 block
+    constexpr int kStages = kE4M3 ? kE8Stages : kWStages;
     const padoc_item *items = prm.items + prm.first_item;
     const int i0 = prm.warp_ptr[wi], i1 = prm.warp_ptr[wi + 1];
     // Every global read the loop depends on is issued at least one item ahead: item headers two
@@ -100,7 +98,7 @@ __device__ __forceinline__ void decode_warp_role(const DecodeParams &prm, uint8_
     };
     auto ids_of = [&](const Walk &w) { return lane < w.nblk ? w.table[w.blk0 + lane] : 0; };
 
-    // The warp walks its items with one ring of kWStages paged blocks that runs on from one item
+    // The warp walks its items with one ring of kStages paged blocks that runs on from one item
     // into the next. Producer: the next block to fetch is block pb of item pu (walk pc, ids ids_c);
     // item pu + 1 (walk pn, ids ids_n) and the header of item pu + 2 (hn2) are already on the way.
     // kPreWait with first_blocks: lane k < 4 holds the pool row of block k of the first item (>= 0),
@@ -137,7 +135,7 @@ __device__ __forceinline__ void decode_warp_role(const DecodeParams &prm, uint8_
                 // chunk q = lane + 32k of the block's 256 16-byte chunks of codes: tensor q / 128,
                 // row (q / 8) % 16, chunk q % 8 (swizzled by row); lanes 0 and 1 also copy the K and
                 // V scales of the (block, KV head) (zeros for a bad id, whose codes are zeros too)
-                const uint32_t base = smem_u32(wbuf + (ring % kWStages) * kE8StageBytes);
+                const uint32_t base = smem_u32(wbuf + (ring % kStages) * kE8StageBytes);
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     const int q = lane + 32 * k;
@@ -152,7 +150,7 @@ __device__ __forceinline__ void decode_warp_role(const DecodeParams &prm, uint8_
                                okid ? 4u : 0u);
                 }
             } else {
-                const uint32_t base = smem_u32(wbuf + (ring % kWStages) * kWStageBytes);
+                const uint32_t base = smem_u32(wbuf + (ring % kStages) * kWStageBytes);
 #pragma unroll
                 for (int k = 0; k < 16; ++k) {
                     const int q = lane + 32 * k;
@@ -204,7 +202,7 @@ __device__ __forceinline__ void decode_warp_role(const DecodeParams &prm, uint8_
         pdl_wait_prerequisite();
         pdl_launch_dependents();
     }
-    for (int k = pre; k < kWStages; ++k) issue_next();
+    for (int k = pre; k < kStages; ++k) issue_next();
 
     // Consumer: header of the next item (ch_n) and of the one after (ch_n2), and the next item's
     // query fragments (B operand Q^T[128 dims x 8 heads]) and first partial row.
@@ -214,10 +212,19 @@ __device__ __forceinline__ void decode_warp_role(const DecodeParams &prm, uint8_
     auto load_q = [&](const padoc_item &it) {
         const __nv_bfloat16 *qrow =
             prm.q + ((size_t)it.first_stream * prm.num_q_heads + it.kv_head * kGroup + (lane >> 2)) * kD;
+        if constexpr (kE4M3) {   // a lane's share of a row is 32 contiguous dims, four to a k-step (see below)
+            const uint4 *src = reinterpret_cast<const uint4 *>(qrow + (lane & 3) * 32);
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
-            qn[ks][0] = *reinterpret_cast<const uint32_t *>(qrow + ks * 16 + (lane & 3) * 2);
-            qn[ks][1] = *reinterpret_cast<const uint32_t *>(qrow + ks * 16 + 8 + (lane & 3) * 2);
+            for (int c = 0; c < 4; ++c) {
+                const uint4 x = src[c];
+                qn[2 * c][0] = x.x; qn[2 * c][1] = x.y; qn[2 * c + 1][0] = x.z; qn[2 * c + 1][1] = x.w;
+            }
+        } else {
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks) {
+                qn[ks][0] = *reinterpret_cast<const uint32_t *>(qrow + ks * 16 + (lane & 3) * 2);
+                qn[ks][1] = *reinterpret_cast<const uint32_t *>(qrow + ks * 16 + 8 + (lane & 3) * 2);
+            }
         }
         row_n = (size_t)(prm.slot_ptr[(size_t)it.first_stream * prm.num_kv_heads + it.kv_head] + it.slot) * kGroup;
     };
@@ -239,107 +246,211 @@ __device__ __forceinline__ void decode_warp_role(const DecodeParams &prm, uint8_
         const int blk0 = it.tok_begin / kBlk;
         const int nblk = cutoff > it.tok_begin ? (cutoff - it.tok_begin + kBlk - 1) / kBlk : 0;
         float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};   // heads h0 = 2*(lane%4), h0+1
+        // E4M3: the queries as f16, their scale off again in the score multipliers of heads h0, h0 + 1;
+        // the exponent of the last nonzero V scale
+        float qk0 = prm.scale_log2, qk1 = prm.scale_log2;
+        int ev = -90;
+        if constexpr (kE4M3) {
+            float amax = 0.f, qs, qi;
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks) amax = bf16x2_amax(bf16x2_amax(amax, qb[ks][0]), qb[ks][1]);
+            amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
+            amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
+            f16_row_scale(amax, qs, qi);
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks) {
+                qb[ks][0] = bf16x2_to_f16x2(qb[ks][0], qs);
+                qb[ks][1] = bf16x2_to_f16x2(qb[ks][1], qs);
+            }
+            qk0 *= __shfl_sync(0xffffffffu, qi, 8 * (lane & 3));
+            qk1 *= __shfl_sync(0xffffffffu, qi, 8 * (lane & 3) + 4);
+        }
         float o[8][4];
 #pragma unroll
         for (int mt = 0; mt < 8; ++mt) o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.f;
 
-        for (int bi = 0; bi < nblk; ++bi, ++gc) {
-            cp_async_wait<kWStages - 1>();   // block gc has landed (one group per block)
-            __syncwarp();
-            // per block: the multiplier of the raw scores (scale in log2 units) and, for an E4M3
-            // pool, the factor folded into P (the V scale; both carry the expansion's 2^112)
-            float kmul = prm.scale_log2, vfac = 1.f;
-            uint32_t base;
-            if constexpr (kE4M3) {
-                const uint8_t *stg = wbuf + (gc % kWStages) * kE8StageBytes;
-                const float ks = *reinterpret_cast<const float *>(stg + 2 * kE8Rows);
-                const float vs = *reinterpret_cast<const float *>(stg + 2 * kE8Rows + 4);
-                // a zero scale marks a block without a nonzero value (its codes are all zero):
-                // any positive factor then gives the same scores and keeps masked ones at -inf
-                kmul = prm.scale_log2 * (ks > 0.f ? ks : 1.f) * kTwo112;
-                vfac = (vs > 0.f ? vs : 1.f) * kTwo112;
-                // lane l expands row l % 16 of tensor l / 16 (K, V) into the bf16 panels
-                const int tn = lane >> 4, r = lane & 15;
-                uint4 raw[8];
+        if constexpr (kE4M3) {
+            // The MMAs' operands come straight from the codes. The order of a contraction's elements is free
+            // as long as both operands share it, so k-step ks of S^T takes dims 32 j + 4 ks .. + 3 of lane
+            // j = lane % 4 (its rows' 32 contiguous bytes), and M row (m, half) of m-tile mt of O^T is dim
+            // 16 m + 2 mt + half (16 contiguous bytes of each of its four tokens, two tokens' bytes
+            // interleaved into pairs): one conversion instruction per two values, exact in f16, and no
+            // expanded copy in shared memory. The serving batch's lists alone: 52 us with the copy, 36 us so;
+            // kStep blocks share one turn of the softmax (2 and 3 are no faster: 38 and 41 us).
+            const int r = lane >> 2, j = lane & 3;
+            auto word = [](const uint4 &v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; };
+            constexpr int kStep = 1;
+            for (int bi = 0; bi < nblk; bi += kStep) {
+                const int nb = min(kStep, nblk - bi);
+                cp_async_wait<kStages - kStep>();   // the step's blocks have landed (one group per block)
+                __syncwarp();
+                uint4 kc[kStep][2][2], vc[kStep][4];
+                float km0[kStep], km1[kStep], evf[kStep], lf[kStep], pf[kStep];
 #pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    raw[c] = *reinterpret_cast<const uint4 *>(stg + tn * kE8Rows + r * 128 + ((c ^ (r & 7)) << 4));
-                __syncwarp();   // every lane has its row: the stage may be refilled
-                issue_next();
+                for (int b = 0; b < kStep; ++b) {
+                    km0[b] = km1[b] = evf[b] = lf[b] = pf[b] = 0.f;
+                    if (b >= nb) {
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const uint32_t w[4] = {raw[c].x, raw[c].y, raw[c].z, raw[c].w};
+                        for (int c = 0; c < 4; ++c) kc[b][c >> 1][c & 1] = vc[b][c] = make_uint4(0u, 0u, 0u, 0u);
+                        continue;
+                    }
+                    const uint8_t *stg = wbuf + ((gc + b) % kStages) * kE8StageBytes;
+                    const float ks = *reinterpret_cast<const float *>(stg + 2 * kE8Rows);
+                    const float vs = *reinterpret_cast<const float *>(stg + 2 * kE8Rows + 4);
 #pragma unroll
-                    for (int hh = 0; hh < 2; ++hh) {   // dims 16c + 8hh .. + 7: bf16 chunk 2c + hh
-                        const int k = 2 * c + hh, panel = 2 * tn + (k >> 3), kk = k & 7;
-                        uint4 o;
-                        o.x = e4m3x2_to_bf16x2_shifted((uint16_t)(w[2 * hh] & 0xFFFFu));
-                        o.y = e4m3x2_to_bf16x2_shifted((uint16_t)(w[2 * hh] >> 16));
-                        o.z = e4m3x2_to_bf16x2_shifted((uint16_t)(w[2 * hh + 1] & 0xFFFFu));
-                        o.w = e4m3x2_to_bf16x2_shifted((uint16_t)(w[2 * hh + 1] >> 16));
-                        *reinterpret_cast<uint4 *>(cbuf + panel * kBoxBytes + r * 128 + ((kk ^ (r & 7)) << 4)) = o;
+                    for (int c = 0; c < 2; ++c)
+#pragma unroll
+                        for (int hh = 0; hh < 2; ++hh)
+                            kc[b][c][hh] = *reinterpret_cast<const uint4 *>(stg + (r + 8 * hh) * 128 + (((2 * j + c) ^ r) << 4));
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const int t = 2 * j + (c & 1) + 8 * (c >> 1);
+                        vc[b][c] = *reinterpret_cast<const uint4 *>(stg + kE8Rows + t * 128 + ((r ^ (t & 7)) << 4));
+                    }
+                    // A zero scale marks a block without a nonzero value (its codes are zeros): any positive
+                    // factor gives the same result. The V scale 2^ev x pf rides on P: the running maximum is
+                    // that of score + ev, so that P (times 2^6) fills the f16 range whatever the scales, and
+                    // the row sum takes the factor off again.
+                    if (vs > 0.f) ev = max((int)(__float_as_uint(vs) >> 23) - 127, -100);
+                    lf[b] = __uint_as_float((uint32_t)(127 - ev) << 23);
+                    pf[b] = vs * lf[b] * 64.f;
+                    evf[b] = (float)ev;
+                    km0[b] = qk0 * (ks > 0.f ? ks : 1.f);
+                    km1[b] = qk1 * (ks > 0.f ? ks : 1.f);
+                }
+                __syncwarp();   // every lane has its part: the stages may be refilled
+                for (int b = 0; b < nb; ++b) issue_next();
+                // S^T = K . Q^T, two independent MMA chains a block
+                float acc[kStep][2][4];
+#pragma unroll
+                for (int b = 0; b < kStep; ++b)
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) acc[b][c][0] = acc[b][c][1] = acc[b][c][2] = acc[b][c][3] = 0.f;
+#pragma unroll
+                for (int ks = 0; ks < 8; ++ks)
+#pragma unroll
+                    for (int b = 0; b < kStep; ++b) {
+                        const uint32_t x0 = word(kc[b][ks >> 2][0], ks & 3), x1 = word(kc[b][ks >> 2][1], ks & 3);
+                        const uint32_t a[4] = {e4m3x2_to_f16x2((uint16_t)x0), e4m3x2_to_f16x2((uint16_t)x1),
+                                               e4m3x2_to_f16x2((uint16_t)(x0 >> 16)), e4m3x2_to_f16x2((uint16_t)(x1 >> 16))};
+                        mma_f16_16816(acc[b][ks & 1], a, qb[ks][0], qb[ks][1]);
+                    }
+                float sc[kStep][4], mx0 = -INFINITY, mx1 = -INFINITY;
+#pragma unroll
+                for (int b = 0; b < kStep; ++b) {
+                    const int t0 = (blk0 + bi + b) * kBlk + r, t1 = t0 + 8;
+                    sc[b][0] = t0 < cutoff ? fmaf(acc[b][0][0] + acc[b][1][0], km0[b], evf[b]) : -INFINITY;
+                    sc[b][1] = t0 < cutoff ? fmaf(acc[b][0][1] + acc[b][1][1], km1[b], evf[b]) : -INFINITY;
+                    sc[b][2] = t1 < cutoff ? fmaf(acc[b][0][2] + acc[b][1][2], km0[b], evf[b]) : -INFINITY;
+                    sc[b][3] = t1 < cutoff ? fmaf(acc[b][0][3] + acc[b][1][3], km1[b], evf[b]) : -INFINITY;
+                    mx0 = fmaxf(mx0, fmaxf(sc[b][0], sc[b][2]));
+                    mx1 = fmaxf(mx1, fmaxf(sc[b][1], sc[b][3]));
+                }
+#pragma unroll
+                for (int sh = 4; sh < 32; sh <<= 1) {
+                    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, sh));
+                    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, sh));
+                }
+                const float mn0 = fmaxf(m[0], mx0), mn1 = fmaxf(m[1], mx1);
+                // a head whose columns are all masked so far keeps m = -inf and contributes 0
+                const float al0 = mn0 == -INFINITY ? 1.f : fast_exp2(m[0] - mn0);
+                const float al1 = mn1 == -INFINITY ? 1.f : fast_exp2(m[1] - mn1);
+                const float r0 = mn0 == -INFINITY ? 0.f : mn0, r1 = mn1 == -INFINITY ? 0.f : mn1;
+                m[0] = mn0; m[1] = mn1;
+                l[0] *= al0;
+                l[1] *= al1;
+                uint32_t bf[kStep][2];
+#pragma unroll
+                for (int b = 0; b < kStep; ++b) {
+                    const float p0 = fast_exp2(sc[b][0] - r0), p1 = fast_exp2(sc[b][1] - r1);
+                    const float p2 = fast_exp2(sc[b][2] - r0), p3 = fast_exp2(sc[b][3] - r1);
+                    l[0] = fmaf(p0 + p2, lf[b], l[0]);
+                    l[1] = fmaf(p1 + p3, lf[b], l[1]);
+                    bf[b][0] = movmatrix_trans(pack_f16x2(p0 * pf[b], p1 * pf[b]));
+                    bf[b][1] = movmatrix_trans(pack_f16x2(p2 * pf[b], p3 * pf[b]));
+                }
+                if (__any_sync(0xffffffffu, al0 != 1.f || al1 != 1.f)) {   // a head's running max moved
+#pragma unroll
+                    for (int mt = 0; mt < 8; ++mt) {
+                        o[mt][0] *= al0; o[mt][1] *= al1; o[mt][2] *= al0; o[mt][3] *= al1;
                     }
                 }
+#pragma unroll
+                for (int b = 0; b < kStep; ++b) {
+                    if (b >= nb) break;
+#pragma unroll
+                    for (int w = 0; w < 4; ++w)
+#pragma unroll
+                        for (int hh = 0; hh < 2; ++hh) {   // dims 4 w + 2 hh, + 1 of the lane's 16
+                            const uint32_t lo = __byte_perm(word(vc[b][0], w), word(vc[b][1], w), hh ? 0x7362 : 0x5140);
+                            const uint32_t hi = __byte_perm(word(vc[b][2], w), word(vc[b][3], w), hh ? 0x7362 : 0x5140);
+                            const uint32_t a[4] = {e4m3x2_to_f16x2((uint16_t)lo), e4m3x2_to_f16x2((uint16_t)(lo >> 16)),
+                                                   e4m3x2_to_f16x2((uint16_t)hi), e4m3x2_to_f16x2((uint16_t)(hi >> 16))};
+                            mma_f16_16816(o[2 * w + hh], a, bf[b][0], bf[b][1]);
+                        }
+                }
+                gc += nb;
+            }
+        } else {
+            for (int bi = 0; bi < nblk; ++bi, ++gc) {
+                cp_async_wait<kStages - 1>();   // block gc has landed (one group per block)
                 __syncwarp();
-                base = smem_u32(cbuf);
-            } else {
-                base = smem_u32(wbuf + (gc % kWStages) * kWStageBytes);
-            }
-            const int tokbase = (blk0 + bi) * kBlk;
-            // S^T = K . Q^T, as two independent MMA chains (even / odd k-steps) added at the end
-            float acc[4] = {0.f, 0.f, 0.f, 0.f}, acc2[4] = {0.f, 0.f, 0.f, 0.f};
+                const uint32_t base = smem_u32(wbuf + (gc % kStages) * kWStageBytes);
+                const int tokbase = (blk0 + bi) * kBlk;
+                // S^T = K . Q^T, as two independent MMA chains (even / odd k-steps) added at the end
+                float acc[4] = {0.f, 0.f, 0.f, 0.f}, acc2[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int ks = 0; ks < 8; ++ks) {
-                const uint32_t row = lane & 15;
-                const uint32_t col = (ks & 3) * 16 + (lane >> 4) * 8;
-                uint32_t a[4];
-                ldmatrix_x4(a, base + (ks >> 2) * kBoxBytes + sw128_offset(row, col));
-                mma_bf16_16816((ks & 1) ? acc2 : acc, a, qb[ks][0], qb[ks][1]);
-            }
+                for (int ks = 0; ks < 8; ++ks) {
+                    const uint32_t row = lane & 15;
+                    const uint32_t col = (ks & 3) * 16 + (lane >> 4) * 8;
+                    uint32_t a[4];
+                    ldmatrix_x4(a, base + (ks >> 2) * kBoxBytes + sw128_offset(row, col));
+                    mma_bf16_16816((ks & 1) ? acc2 : acc, a, qb[ks][0], qb[ks][1]);
+                }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) acc[i] += acc2[i];
-            const int t0 = tokbase + (lane >> 2), t1 = t0 + 8;
-            float sc[4];
-            sc[0] = t0 < cutoff ? acc[0] * kmul : -INFINITY;
-            sc[1] = t0 < cutoff ? acc[1] * kmul : -INFINITY;
-            sc[2] = t1 < cutoff ? acc[2] * kmul : -INFINITY;
-            sc[3] = t1 < cutoff ? acc[3] * kmul : -INFINITY;
-            float mx0 = fmaxf(sc[0], sc[2]), mx1 = fmaxf(sc[1], sc[3]);
+                for (int i = 0; i < 4; ++i) acc[i] += acc2[i];
+                const int t0 = tokbase + (lane >> 2), t1 = t0 + 8;
+                float sc[4];
+                sc[0] = t0 < cutoff ? acc[0] * prm.scale_log2 : -INFINITY;
+                sc[1] = t0 < cutoff ? acc[1] * prm.scale_log2 : -INFINITY;
+                sc[2] = t1 < cutoff ? acc[2] * prm.scale_log2 : -INFINITY;
+                sc[3] = t1 < cutoff ? acc[3] * prm.scale_log2 : -INFINITY;
+                float mx0 = fmaxf(sc[0], sc[2]), mx1 = fmaxf(sc[1], sc[3]);
 #pragma unroll
-            for (int sh = 4; sh < 32; sh <<= 1) {
-                mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, sh));
-                mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, sh));
-            }
-            const float mn0 = fmaxf(m[0], mx0), mn1 = fmaxf(m[1], mx1);
-            // a head whose columns are all masked so far keeps m = -inf and contributes 0
-            const float al0 = mn0 == -INFINITY ? 1.f : fast_exp2(m[0] - mn0);
-            const float al1 = mn1 == -INFINITY ? 1.f : fast_exp2(m[1] - mn1);
-            const float r0 = mn0 == -INFINITY ? 0.f : mn0, r1 = mn1 == -INFINITY ? 0.f : mn1;
-            const float p0 = fast_exp2(sc[0] - r0), p1 = fast_exp2(sc[1] - r1);
-            const float p2 = fast_exp2(sc[2] - r0), p3 = fast_exp2(sc[3] - r1);
-            m[0] = mn0; m[1] = mn1;
-            l[0] = l[0] * al0 + p0 + p2;
-            l[1] = l[1] * al1 + p1 + p3;
-            // the V scale rides on P (E4M3); l keeps the plain probabilities
-            const uint32_t b0 = movmatrix_trans(kE4M3 ? pack_bf16x2(p0 * vfac, p1 * vfac) : pack_bf16x2(p0, p1));
-            const uint32_t b1 = movmatrix_trans(kE4M3 ? pack_bf16x2(p2 * vfac, p3 * vfac) : pack_bf16x2(p2, p3));
-            if (__any_sync(0xffffffffu, al0 != 1.f || al1 != 1.f)) {   // a head's running max moved
+                for (int sh = 4; sh < 32; sh <<= 1) {
+                    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, sh));
+                    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, sh));
+                }
+                const float mn0 = fmaxf(m[0], mx0), mn1 = fmaxf(m[1], mx1);
+                // a head whose columns are all masked so far keeps m = -inf and contributes 0
+                const float al0 = mn0 == -INFINITY ? 1.f : fast_exp2(m[0] - mn0);
+                const float al1 = mn1 == -INFINITY ? 1.f : fast_exp2(m[1] - mn1);
+                const float r0 = mn0 == -INFINITY ? 0.f : mn0, r1 = mn1 == -INFINITY ? 0.f : mn1;
+                const float p0 = fast_exp2(sc[0] - r0), p1 = fast_exp2(sc[1] - r1);
+                const float p2 = fast_exp2(sc[2] - r0), p3 = fast_exp2(sc[3] - r1);
+                m[0] = mn0; m[1] = mn1;
+                l[0] = l[0] * al0 + p0 + p2;
+                l[1] = l[1] * al1 + p1 + p3;
+                const uint32_t b0 = movmatrix_trans(pack_bf16x2(p0, p1));
+                const uint32_t b1 = movmatrix_trans(pack_bf16x2(p2, p3));
+                if (__any_sync(0xffffffffu, al0 != 1.f || al1 != 1.f)) {   // a head's running max moved
+#pragma unroll
+                    for (int mt = 0; mt < 8; ++mt) {
+                        o[mt][0] *= al0; o[mt][1] *= al1; o[mt][2] *= al0; o[mt][3] *= al1;
+                    }
+                }
 #pragma unroll
                 for (int mt = 0; mt < 8; ++mt) {
-                    o[mt][0] *= al0; o[mt][1] *= al1; o[mt][2] *= al0; o[mt][3] *= al1;
+                    const int i = lane >> 3;
+                    const uint32_t row = (lane & 7) + (i >= 2 ? 8 : 0);
+                    const uint32_t col = (mt & 3) * 16 + (i & 1) * 8;
+                    uint32_t a[4];
+                    ldmatrix_x4_trans(a, base + (2 + (mt >> 2)) * kBoxBytes + sw128_offset(row, col));
+                    mma_bf16_16816(o[mt], a, b0, b1);
                 }
+                __syncwarp();   // every lane is done with the stage
+                issue_next();
             }
-#pragma unroll
-            for (int mt = 0; mt < 8; ++mt) {
-                const int i = lane >> 3;
-                const uint32_t row = (lane & 7) + (i >= 2 ? 8 : 0);
-                const uint32_t col = (mt & 3) * 16 + (i & 1) * 8;
-                uint32_t a[4];
-                ldmatrix_x4_trans(a, base + (2 + (mt >> 2)) * kBoxBytes + sw128_offset(row, col));
-                mma_bf16_16816(o[mt], a, b0, b1);
-            }
-            __syncwarp();   // every lane is done with the stage (bf16) or the expanded block (E4M3)
-            if constexpr (!kE4M3) issue_next();   // (E4M3: the stage was refilled after its expansion)
         }
         // complete the row sums over the 8 token lanes of each head
 #pragma unroll
@@ -351,7 +462,21 @@ __device__ __forceinline__ void decode_warp_role(const DecodeParams &prm, uint8_
         // l / 4 of heads h0, h0 + 1 (h0 = 2 (l % 4)); with its partner l ^ 4 (the next or previous dim)
         // a lane of an even dim writes the dim pair of head h0, one of an odd dim that of head
         // h0 + 1, so that the warp writes each chunk's [8 heads][8 dims] as one 128-byte run
-        {
+        if constexpr (kE4M3) {
+            // a lane holds dims 16 (l / 4) .. + 15 of both heads: two 16-byte pieces of each
+            const int h0 = (lane & 3) * 2;
+            const float i0f = l[0] > 0.f ? 0x1p-6f / l[0] : 0.f, i1f = l[1] > 0.f ? 0x1p-6f / l[1] : 0.f;
+            __nv_bfloat16 *p = prm.part_o + row0 * kD + (lane >> 2) * 128 + h0 * 8;   // chunk 2 (l / 4)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                *reinterpret_cast<uint4 *>(p + 64 * c) =
+                    make_uint4(pack_bf16x2(o[4 * c][0] * i0f, o[4 * c][2] * i0f), pack_bf16x2(o[4 * c + 1][0] * i0f, o[4 * c + 1][2] * i0f),
+                               pack_bf16x2(o[4 * c + 2][0] * i0f, o[4 * c + 2][2] * i0f), pack_bf16x2(o[4 * c + 3][0] * i0f, o[4 * c + 3][2] * i0f));
+                *reinterpret_cast<uint4 *>(p + 64 * c + 8) =
+                    make_uint4(pack_bf16x2(o[4 * c][1] * i1f, o[4 * c][3] * i1f), pack_bf16x2(o[4 * c + 1][1] * i1f, o[4 * c + 1][3] * i1f),
+                               pack_bf16x2(o[4 * c + 2][1] * i1f, o[4 * c + 2][3] * i1f), pack_bf16x2(o[4 * c + 3][1] * i1f, o[4 * c + 3][3] * i1f));
+            }
+        } else {
             const int h0 = (lane & 3) * 2, dm = lane >> 2;
             const bool ev = (dm & 1) == 0;
             const float i0f = l[0] > 0.f ? 1.f / l[0] : 0.f, i1f = l[1] > 0.f ? 1.f / l[1] : 0.f;
