@@ -47,7 +47,7 @@
 namespace {
 
 constexpr int kD = 128;
-constexpr int kThreads = 320;
+constexpr int kThreads = 352;
 constexpr uint32_t kTmemCols = 512;
 
 struct BwdParams {
@@ -75,7 +75,7 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, int
 // TMEM column of k-slice k (16 values) of a W-wide bf16 operand written by the softmax warps: column
 // half c packs its W/2 values into the first W/4 columns of its own half.
 template <int W>
-__device__ __forceinline__ uint32_t slice_col(int k)
+__host__ __device__ constexpr uint32_t slice_col(int k)
 {
     constexpr int per_half = W / 32;
     return (uint32_t)((k / per_half) * (W / 2) + (k % per_half) * 8);
@@ -169,8 +169,9 @@ enum {
     B_QEMPTY = 1 + kStages,       // [stage]
     B_SFULL = 1 + 2 * kStages,    // [step parity]
     B_PFULL = 3 + 2 * kStages,    // [step parity], 256 arrivals
-    B_FINAL = 5 + 2 * kStages,
-    B_COUNT = 6 + 2 * kStages
+    B_FINAL = 5 + 2 * kStages,    // [issuing warp]
+    B_ACC = 7 + 2 * kStages,      // [step parity]: the step's accumulating MMAs are done
+    B_COUNT = 9 + 2 * kStages
 };
 constexpr size_t kSmemBytes = 1024 + 2 * (size_t)kKTile + 2 * (size_t)kStages * kQTile + (size_t)kStages * kAuxBytes +
                               B_COUNT * 8 + 64;
@@ -262,71 +263,55 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
             for (int u = (issued > kStages ? issued - kStages : 0); u < issued; ++u)
                 mbar_wait_bounded(bar(B_QFULL + u % kStages), (u / kStages) & 1, prm.err, 52);
         }
-    } else if (warp == 9) {
-        // ---------------------------------------------------------------- MMA issuer (whole warp)
+    } else if (warp == 9 || warp == 10) {
+        // ---------------------------------------------------------------- MMA issuers (whole warps)
+        // Warp 9 issues the S^T and dP^T, warp 10 the accumulating MMAs, so that one's waits (each
+        // issued behind the MMAs before it) leave the tensor cores the other's MMAs; a step's S^T waits
+        // for the accumulating MMAs that read the buffer it overwrites.
         if (nu > 0) {
-            constexpr uint32_t idS = umma_idesc_bf16(128, kQT, false);
-            constexpr uint32_t idAcc = umma_idesc_bf16(128, kD, true);
-            const uint64_t dK = umma_desc_sw128(smem_u32(sk), 16, 1024);
-            const uint64_t dV = umma_desc_sw128(smem_u32(sv), 16, 1024);
             auto wait_w = [&](int b, uint32_t parity, int site) {
                 const bool r = wait_or_abort(bar(b), parity, prm.err, site, abort_flag);
-                return __all_sync(0xffffffffu, r);
+                return (bool)__all_sync(0xffffffffu, r);
             };
-            // S^T and dP^T of step u into the parity-(u & 1) columns
-            auto issue_s = [&](int u) {
-                const int s = u % kStages;
-                const uint32_t b = (uint32_t)(u & 1) * 64;
-                const uint64_t dq = umma_desc_sw128(smem_u32(sq + s * kQTile), 16, 1024);
-                const uint64_t dg = umma_desc_sw128(smem_u32(sg + s * kQTile), 16, 1024);
-#pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
-                    const uint32_t oa = ((ks >> 2) * kKPanel + (ks & 3) * 32) >> 4;
-                    const uint32_t ob = ((ks >> 2) * kQPanel + (ks & 3) * 32) >> 4;
-                    umma_bf16_ss_warp(tmem + kColS + b, dK + oa, dq + ob, idS, ks > 0);
-                }
-#pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
-                    const uint32_t oa = ((ks >> 2) * kKPanel + (ks & 3) * 32) >> 4;
-                    const uint32_t ob = ((ks >> 2) * kQPanel + (ks & 3) * 32) >> 4;
-                    umma_bf16_ss_warp(tmem + kColDP + b, dV + oa, dg + ob, idS, ks > 0);
-                }
-                umma_commit_warp(bar(B_SFULL + (u & 1)));
-            };
-            bool ok = wait_w(B_KV, 0, 60);
-            for (int u = 0; ok && u < 2 && u < nu; ++u) {
-                ok = wait_w(B_QFULL + u % kStages, (u / kStages) & 1, 61);
-                if (ok) {
+            if (warp == 9) {
+                constexpr uint32_t idS = umma_idesc_bf16(128, kQT, false);
+                const uint64_t dK = umma_desc_sw128(smem_u32(sk), 16, 1024);
+                const uint64_t dV = umma_desc_sw128(smem_u32(sv), 16, 1024);
+                bool ok = wait_w(B_KV, 0, 60);
+                for (int u = 0; ok && u < nu; ++u) {
+                    const int s = u % kStages;
+                    const uint32_t b = (uint32_t)(u & 1) * 64;
+                    ok = wait_w(B_QFULL + s, (u / kStages) & 1, 61) && (u < 2 || wait_w(B_ACC + (u & 1), ((u >> 1) - 1) & 1, 63));
+                    if (!ok) break;
                     tc_fence_after();
-                    issue_s(u);
+                    const uint64_t dq = umma_desc_sw128(smem_u32(sq + s * kQTile), 16, 1024);
+                    const uint64_t dg = umma_desc_sw128(smem_u32(sg + s * kQTile), 16, 1024);
+                    umma_bf16_ss_k128_warp<1, kKPanel, kQPanel>(tmem + kColS + b, dK, dq, idS);
+                    umma_bf16_ss_k128_warp<1, kKPanel, kQPanel>(tmem + kColDP + b, dV, dg, idS);
+                    umma_commit_warp(bar(B_SFULL + (u & 1)));
                 }
-            }
-            for (int u = 0; ok && u < nu; ++u) {
-                const int s = u % kStages;
-                const uint32_t b = (uint32_t)(u & 1) * 64;
-                if (!wait_w(B_PFULL + (u & 1), (u >> 1) & 1, 62)) { ok = false; break; }
-                tc_fence_after();
-                // the step's Q and dO as MN-major B operands (N = head dim, K = the 64 queries)
-                const uint64_t gmn = umma_desc_sw128(smem_u32(sg + s * kQTile), kQPanel, 1024);
-                const uint64_t qmn = umma_desc_sw128(smem_u32(sq + s * kQTile), kQPanel, 1024);
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    umma_bf16_ts_warp(tmem + kColAcc0, tmem + kColS + b + slice_col<kQT>(kk), gmn + kk * (2048 >> 4), idAcc,
-                                      (u > 0 || kk > 0));
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    umma_bf16_ts_warp(tmem + kColAcc1, tmem + kColDP + b + slice_col<kQT>(kk), qmn + kk * (2048 >> 4), idAcc,
-                                      (u > 0 || kk > 0));
-                umma_commit_warp(bar(B_QEMPTY + s));
-                if (u + 2 < nu) {
-                    if (!wait_w(B_QFULL + (u + 2) % kStages, ((u + 2) / kStages) & 1, 63)) { ok = false; break; }
+            } else {
+                constexpr uint32_t idAcc = umma_idesc_bf16(128, kD, true);
+                bool ok = true;
+                for (int u = 0; ok && u < nu; ++u) {
+                    const int s = u % kStages;
+                    const uint32_t b = (uint32_t)(u & 1) * 64;
+                    if (!(ok = wait_w(B_PFULL + (u & 1), (u >> 1) & 1, 62))) break;
                     tc_fence_after();
-                    issue_s(u + 2);
+                    // the step's Q and dO as MN-major B operands (N = head dim, K = the 64 queries)
+                    const uint64_t gmn = umma_desc_sw128(smem_u32(sg + s * kQTile), kQPanel, 1024);
+                    const uint64_t qmn = umma_desc_sw128(smem_u32(sq + s * kQTile), kQPanel, 1024);
+                    umma_bf16_ts_k64_mn_warp<1, slice_col<kQT>(1), slice_col<kQT>(2), slice_col<kQT>(3)>(
+                        tmem + kColAcc0, tmem + kColS + b, gmn, idAcc, u > 0);
+                    umma_bf16_ts_k64_mn_warp<1, slice_col<kQT>(1), slice_col<kQT>(2), slice_col<kQT>(3)>(
+                        tmem + kColAcc1, tmem + kColDP + b, qmn, idAcc, u > 0);
+                    umma_commit_warp(bar(B_ACC + (u & 1)));
+                    umma_commit_warp(bar(B_QEMPTY + s));
                 }
             }
             // every MMA issued above must complete before tensor memory is read or released
-            umma_commit_warp(bar(B_FINAL));
-            mbar_wait_bounded(bar(B_FINAL), 0, prm.err, 64);
+            umma_commit_warp(bar(B_FINAL + warp - 9));
+            mbar_wait_bounded(bar(B_FINAL + warp - 9), 0, prm.err, 64);
         }
     } else {
         // ---------------------------------------------------------------- softmax + epilogue
@@ -405,7 +390,7 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
             tc_fence_before();
             mbar_arrive(bar(B_PFULL + (u & 1)));
         }
-        sums = ok && (nu == 0 || wait_all(B_FINAL, 0, 72));
+        sums = ok && (nu == 0 || wait_all(B_FINAL + 1, 0, 72));
         tc_fence_after();
     }
     // Epilogue. The 256 columns of dV | dK are split over the cluster's CTAs: each one's softmax threads
@@ -501,8 +486,9 @@ struct DqCfg {
         B_KEMPTY = 1 + kStages,         // [stage]
         B_SFULL = 1 + 2 * kStages,      // [buffer]
         B_PFULL = 1 + 2 * kStages + kDepth,   // [buffer], 256 arrivals
-        B_FINAL = 1 + 2 * kStages + 2 * kDepth,
-        B_COUNT = 2 + 2 * kStages + 2 * kDepth
+        B_FINAL = 1 + 2 * kStages + 2 * kDepth,     // [issuing warp]
+        B_ACC = 3 + 2 * kStages + 2 * kDepth,       // [buffer]: the accumulating MMAs that read it are done
+        B_COUNT = 3 + 2 * kStages + 3 * kDepth
     };
     static constexpr size_t kSmemBytes = 1024 + (size_t)kStages * 2 * kTile + B_COUNT * 8 + 64 + 2 * kQT * 4;
     static_assert(kDepth >= 1 && W % 32 == 0, "step width");
@@ -569,53 +555,50 @@ prefill_bwd_dq_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
             for (int u = (issued > S ? issued - S : 0); u < issued; ++u)
                 mbar_wait_bounded(bar(C::B_KFULL + u % S), (u / S) & 1, prm.err, 82);
         }
-    } else if (warp == 9) {
-        // ---------------------------------------------------------------- MMA issuer (whole warp)
+    } else if (warp == 9 || warp == 10) {
+        // ---------------------------------------------------------------- MMA issuers (whole warps)
+        // warp 9 the S and dP, warp 10 the accumulating MMAs, as in the dK/dV pass
         if (nu > 0) {
-            constexpr uint32_t idS = umma_idesc_bf16(128, W, false);
-            constexpr uint32_t idAcc = umma_idesc_bf16(128, kD, true);
             auto wait_w = [&](int b, uint32_t parity, int site) {
                 const bool r = wait_or_abort(bar(b), parity, prm.err, site, abort_flag);
-                return __all_sync(0xffffffffu, r);
+                return (bool)__all_sync(0xffffffffu, r);
             };
-            // S = Q K^T and dP = dO V^T of step u into buffer u % DEPTH (A from tensor memory)
-            auto issue_s = [&](int u) {
-                const int s = u % S;
-                const uint32_t b = C::kColBuf + (uint32_t)(u % DEPTH) * 2 * W;
-                if (!wait_w(C::B_KFULL + s, (u / S) & 1, 91)) return false;
-                tc_fence_after();
-                const uint64_t dk = umma_desc_sw128(smem_u32(sk + s * C::kTile), 16, 1024);
-                const uint64_t dv = umma_desc_sw128(smem_u32(sv + s * C::kTile), 16, 1024);
-#pragma unroll
-                for (int ks = 0; ks < 8; ++ks)
-                    umma_bf16_ts_warp(tmem + b, tmem + C::kColQ + 8 * ks,
-                                      dk + (((ks >> 2) * C::kPanel + (ks & 3) * 32) >> 4), idS, ks > 0);
-#pragma unroll
-                for (int ks = 0; ks < 8; ++ks)
-                    umma_bf16_ts_warp(tmem + b + W, tmem + C::kColG + 8 * ks,
-                                      dv + (((ks >> 2) * C::kPanel + (ks & 3) * 32) >> 4), idS, ks > 0);
-                umma_commit_warp(bar(C::B_SFULL + u % DEPTH));
-                return true;
-            };
-            bool ok = wait_w(C::B_QG, 0, 90);
-            if (ok) tc_fence_after();
-            for (int u = 0; ok && u < DEPTH && u < nu; ++u) ok = issue_s(u);
-            for (int u = 0; ok && u < nu; ++u) {
-                const int s = u % S;
-                const uint32_t b = C::kColBuf + (uint32_t)(u % DEPTH) * 2 * W;
-                if (!wait_w(C::B_PFULL + u % DEPTH, (u / DEPTH) & 1, 92)) { ok = false; break; }
-                tc_fence_after();
-                // the step's K as an MN-major B operand (N = head dim, K = the W keys)
-                const uint64_t kmn = umma_desc_sw128(smem_u32(sk + s * C::kTile), C::kPanel, 1024);
-#pragma unroll
-                for (int k = 0; k < W / 16; ++k)
-                    umma_bf16_ts_warp(tmem + C::kColDQ, tmem + b + W + slice_col<W>(k), kmn + k * (2048 >> 4), idAcc,
-                                      (u > 0 || k > 0));
-                umma_commit_warp(bar(C::B_KEMPTY + s));
-                if (u + DEPTH < nu && !issue_s(u + DEPTH)) { ok = false; break; }
+            if (warp == 9) {
+                // S = Q K^T and dP = dO V^T of step u into buffer u % DEPTH (A from tensor memory)
+                constexpr uint32_t idS = umma_idesc_bf16(128, W, false);
+                bool ok = wait_w(C::B_QG, 0, 90);
+                for (int u = 0; ok && u < nu; ++u) {
+                    const int s = u % S;
+                    const uint32_t b = C::kColBuf + (uint32_t)(u % DEPTH) * 2 * W;
+                    ok = wait_w(C::B_KFULL + s, (u / S) & 1, 91) &&
+                         (u < DEPTH || wait_w(C::B_ACC + u % DEPTH, (u / DEPTH - 1) & 1, 93));
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint64_t dk = umma_desc_sw128(smem_u32(sk + s * C::kTile), 16, 1024);
+                    const uint64_t dv = umma_desc_sw128(smem_u32(sv + s * C::kTile), 16, 1024);
+                    umma_bf16_ts_k128_warp<C::kPanel>(tmem + b, tmem + C::kColQ, dk, idS);
+                    umma_bf16_ts_k128_warp<C::kPanel>(tmem + b + W, tmem + C::kColG, dv, idS);
+                    umma_commit_warp(bar(C::B_SFULL + u % DEPTH));
+                }
+            } else {
+                static_assert(W == 64, "the accumulating block takes four K-steps");
+                constexpr uint32_t idAcc = umma_idesc_bf16(128, kD, true);
+                bool ok = true;
+                for (int u = 0; ok && u < nu; ++u) {
+                    const int s = u % S;
+                    const uint32_t b = C::kColBuf + (uint32_t)(u % DEPTH) * 2 * W;
+                    if (!(ok = wait_w(C::B_PFULL + u % DEPTH, (u / DEPTH) & 1, 92))) break;
+                    tc_fence_after();
+                    // the step's K as an MN-major B operand (N = head dim, K = the W keys)
+                    const uint64_t kmn = umma_desc_sw128(smem_u32(sk + s * C::kTile), C::kPanel, 1024);
+                    umma_bf16_ts_k64_mn_warp<1, slice_col<W>(1), slice_col<W>(2), slice_col<W>(3)>(
+                        tmem + C::kColDQ, tmem + b + W, kmn, idAcc, u > 0);
+                    umma_commit_warp(bar(C::B_ACC + u % DEPTH));
+                    umma_commit_warp(bar(C::B_KEMPTY + s));
+                }
             }
-            umma_commit_warp(bar(C::B_FINAL));
-            mbar_wait_bounded(bar(C::B_FINAL), 0, prm.err, 94);
+            umma_commit_warp(bar(C::B_FINAL + warp - 9));
+            mbar_wait_bounded(bar(C::B_FINAL + warp - 9), 0, prm.err, 94);
         }
     } else {
         // ---------------------------------------------------------------- softmax + epilogue
@@ -725,7 +708,7 @@ prefill_bwd_dq_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
             mbar_arrive(bar(C::B_PFULL + u % DEPTH));
         }
         // epilogue: dQ times scale, columns 64 ch .. 64 ch + 63 of the thread's row
-        if (ok && (nu == 0 || wait_all(C::B_FINAL, 0, 96))) {
+        if (ok && (nu == 0 || wait_all(C::B_FINAL + 1, 0, 96))) {
             tc_fence_after();
             __nv_bfloat16 *dst = prm.out0 + ((size_t)(t < prm.T ? t : 0) * hq + h) * kD + 64 * ch;
 #pragma unroll

@@ -156,9 +156,9 @@ __device__ __forceinline__ void umma_bf16_ss_k128_warp(uint32_t d_tmem, uint64_t
             " add.s64 a, %1, %4+6;\n add.s64 b, %2, %5+6;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n}" ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "n"(PA >> 4), "n"(PB >> 4)
             : "memory");
 }
-// Four K-steps (64 elements) of D (+)= A[tmem] . B[smem], B MN-major (a step adds 16 rows, 2048 bytes)
-// and A 8 columns a step; `accumulate` 0: the first step overwrites D.
-template <int CG>
+// Four K-steps (64 elements) of D (+)= A[tmem] . B[smem], B MN-major (a step adds 16 rows, 2048 bytes);
+// A's steps start at columns 0, A1, A2 and A3; `accumulate` 0: the first step overwrites D.
+template <int CG, int A1 = 8, int A2 = 16, int A3 = 24>
 __device__ __forceinline__ void umma_bf16_ts_k64_mn_warp(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
                                                          uint32_t accumulate)
 {
@@ -167,19 +167,36 @@ __device__ __forceinline__ void umma_bf16_ts_k64_mn_warp(uint32_t d_tmem, uint32
             "{\n .reg .pred e, t, p;\n .reg .b64 b;\n .reg .b32 a;\n elect.sync _|e, 0xffffffff;\n"
             " setp.eq.u32 t, 0, 0;\n setp.ne.b32 p, %4, 0;\n"
             " @e tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n"
-            " add.s32 a, %1, 8;\n add.s64 b, %2, 128;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], [a], b, %3, t;\n"
-            " add.s32 a, %1, 16;\n add.s64 b, %2, 256;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], [a], b, %3, t;\n"
-            " add.s32 a, %1, 24;\n add.s64 b, %2, 384;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], [a], b, %3, t;\n}" ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+            " add.s32 a, %1, %5;\n add.s64 b, %2, 128;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], [a], b, %3, t;\n"
+            " add.s32 a, %1, %6;\n add.s64 b, %2, 256;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], [a], b, %3, t;\n"
+            " add.s32 a, %1, %7;\n add.s64 b, %2, 384;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], [a], b, %3, t;\n}" ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate), "n"(A1), "n"(A2), "n"(A3)
             : "memory");
     else
         asm volatile(
             "{\n .reg .pred e, t, p;\n .reg .b64 b;\n .reg .b32 a;\n elect.sync _|e, 0xffffffff;\n"
             " setp.eq.u32 t, 0, 0;\n setp.ne.b32 p, %4, 0;\n"
             " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n"
-            " add.s32 a, %1, 8;\n add.s64 b, %2, 128;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
-            " add.s32 a, %1, 16;\n add.s64 b, %2, 256;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
-            " add.s32 a, %1, 24;\n add.s64 b, %2, 384;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n}" ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+            " add.s32 a, %1, %5;\n add.s64 b, %2, 128;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
+            " add.s32 a, %1, %6;\n add.s64 b, %2, 256;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
+            " add.s32 a, %1, %7;\n add.s64 b, %2, 384;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n}" ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate), "n"(A1), "n"(A2), "n"(A3)
             : "memory");
+}
+// Eight K-steps (128 elements) of D = A[tmem] . B[smem]^T, B K-major (panels of 64 elements, PB bytes apart).
+template <int PB>
+__device__ __forceinline__ void umma_bf16_ts_k128_warp(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc)
+{
+    asm volatile(
+        "{\n .reg .pred e, t, f;\n .reg .b64 b;\n .reg .b32 a;\n elect.sync _|e, 0xffffffff;\n"
+        " setp.eq.u32 t, 0, 0;\n setp.ne.u32 f, 0, 0;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, f;\n"
+        " add.s32 a, %1, 8;\n add.s64 b, %2, 2;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
+        " add.s32 a, %1, 16;\n add.s64 b, %2, 4;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
+        " add.s32 a, %1, 24;\n add.s64 b, %2, 6;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
+        " add.s32 a, %1, 32;\n add.s64 b, %2, %4;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
+        " add.s32 a, %1, 40;\n add.s64 b, %2, %4+2;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
+        " add.s32 a, %1, 48;\n add.s64 b, %2, %4+4;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
+        " add.s32 a, %1, 56;\n add.s64 b, %2, %4+6;\n @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n}" ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "n"(PB >> 4)
+        : "memory");
 }
 // As umma_commit_warp for MMAs over a CTA pair: arrives on the barrier at this offset in both CTAs.
 __device__ __forceinline__ void umma_commit_pair_warp(uint32_t mbar)
@@ -238,46 +255,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16])
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
-}
-
-// 16 lanes (taddr's lane a multiple of 16 in the warp's quarter) in the layout of an MMA accumulator: of
-// each 8 columns thread i holds columns 2 (i % 4), + 1 of lane i / 4 in registers 0, 1 and of lane i / 4 + 8
-// in registers 2, 3. A row's columns so lie in four threads of one warp.
-__device__ __forceinline__ void tmem_ld_16x256b_x8(uint32_t taddr, uint32_t (&r)[32])   // 64 columns
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x256b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_ld_16x256b_x4(uint32_t taddr, uint32_t (&r)[16])   // 32 columns
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_st_16x256b_x4(uint32_t taddr, const uint32_t (&r)[16])   // 32 columns
-{
-    asm volatile(
-        "tcgen05.st.sync.aligned.16x256b.x4.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
-        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-        : "memory");
-}
-// 16 lanes, of each 4 columns thread i holds column i % 4 of lane i / 4 in register 0 and of lane i / 4 + 8
-// in register 1: where the packed pairs of the layout above go.
-__device__ __forceinline__ void tmem_st_16x128b_x8(uint32_t taddr, const uint32_t (&r)[16])   // 32 columns
-{
-    asm volatile(
-        "tcgen05.st.sync.aligned.16x128b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
-        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-        : "memory");
 }
 
 // 32 lanes x 8 consecutive 32-bit columns.
