@@ -287,8 +287,8 @@ def _stream_ptr(stream):
     """The cudaStream_t of ``stream`` (a torch stream or a raw handle); None: torch's current stream."""
     global _raw_stream
     if stream is None:
-        import torch
         if _raw_stream is None:
+            import torch
             get, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
             _raw_stream = (lambda: get(dev())) if get and dev else (lambda: torch.cuda.current_stream().cuda_stream)
         return _raw_stream()
@@ -802,8 +802,11 @@ class MpdRunner:
         self._up_ref = ctypes.byref(self._up)
         self._ids = np.zeros(64, np.int32)
         self._args.ids_capacity, self._args.stream_ids = self._ids.size, self._ids.ctypes.data
-        self._src = None
-        self._outs = {}
+        self._src = self._outs = None
+        import torch
+        self._elt = torch.bfloat16 if pool.dtype == PADOC_DTYPE_BF16 else torch.float32
+        self._f32 = torch.float32
+        self._hq, self._d = int(cfg.num_q_heads), int(cfg.head_dim)
 
     def close(self):
         if self._h:
@@ -819,17 +822,26 @@ class MpdRunner:
     def step(self, k_src, v_src, q_src, row_of_stream: np.ndarray, scale: float, out, lse, stream=None):
         """One step: returns (C, stream ids int32 [C], a view of the runner's array valid until the
         next step). out [rows >= C][Hq][d] and lse fp32 [rows][Hq] receive the outputs in step order;
-        row_of_stream: int32 [ids] (host), the source row of each live stream's input. Arrays are
-        checked the first time they are seen (the runner keeps the last few)."""
+        row_of_stream: int32 [ids] (host), the source row of each live stream's input. The sources
+        are checked when they change. The outputs, usually new slices of a longer buffer, are checked
+        on every step by plain attribute reads (the cached, general check was 5.8 us of a 56 us step
+        on a Grace core); the last pair is kept alive until the next step."""
         a = self._args
         src = self._src
         if src is None or src[0] is not k_src or src[1] is not v_src or src[2] is not q_src or \
                 src[3] is not row_of_stream:
             self._set_sources(k_src, v_src, q_src, row_of_stream)
-        o = self._outs.get((id(out), id(lse)))
-        if o is None or o[0] is not out or o[1] is not lse:
-            o = self._set_outputs(out, lse)
-        a.out, a.lse, a.out_rows = o[2], o[3], o[4]
+        osh, lsh = out.shape, lse.shape
+        if not (out.dtype is self._elt and lse.dtype is self._f32 and out.is_cuda and lse.is_cuda and
+                out.is_contiguous() and lse.is_contiguous() and len(osh) == 3 and len(lsh) == 2 and
+                osh[1] == self._hq and osh[2] == self._d and lsh[1] == self._hq):
+            self._refuse_outputs(out, lse)
+        cap = osh[0] if osh[0] < lsh[0] else lsh[0]
+        if self._ids.size < cap:
+            self._ids = np.zeros(cap, np.int32)
+            a.ids_capacity, a.stream_ids = self._ids.size, self._ids.ctypes.data
+        a.out, a.lse, a.out_rows = out.data_ptr(), lse.data_ptr(), cap
+        self._outs = (out, lse)
         a.scale = scale
         a.stream = _stream_ptr(stream)
         _check("padoc_mpd_runner_step", self._lib.padoc_mpd_runner_step(self._h, self._args_ref, self._n_ref,
@@ -862,26 +874,14 @@ class MpdRunner:
         a.num_stream_ids = row_of_stream.size
         self._src = (k_src, v_src, q_src, row_of_stream)
 
-    def _set_outputs(self, out, lse):
-        c = self._cfg
-        dt = PADOC_DTYPE_BF16 if self._pool.dtype == PADOC_DTYPE_BF16 else PADOC_DTYPE_F32
+    def _refuse_outputs(self, out, lse):
         _dev(out, "out")
         _dev(lse, "lse")
-        if _dtype_code(out) != dt:
+        if out.dtype is not self._elt:
             raise TypeError("out must have the pool's dtype")
-        if str(lse.dtype) != "torch.float32":
+        if lse.dtype is not self._f32:
             raise TypeError("lse must be float32")
-        if tuple(out.shape[1:]) != (c.num_q_heads, c.head_dim) or lse.dim() != 2 or lse.shape[1] != c.num_q_heads:
-            raise ValueError("out [rows][Hq][d], lse [rows][Hq]")
-        cap = min(int(out.shape[0]), int(lse.shape[0]))
-        if self._ids.size < cap:
-            self._ids = np.zeros(cap, np.int32)
-            self._args.ids_capacity, self._args.stream_ids = self._ids.size, self._ids.ctypes.data
-        if len(self._outs) >= 8:
-            self._outs.clear()
-        o = (out, lse, out.data_ptr(), lse.data_ptr(), cap)
-        self._outs[(id(out), id(lse))] = o
-        return o
+        raise ValueError("out [rows][Hq][d], lse [rows][Hq]")
 
     def last_step(self):
         """(padoc_mpd_step, its staging buffer as an int32 numpy array [total_words])."""
