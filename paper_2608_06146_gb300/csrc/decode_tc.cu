@@ -491,8 +491,7 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
         const uint64_t dv0 = umma_desc_sw128(smem_u32(sv), kPanel, 1024);
         const uint32_t tS = tmem + 128 * mi, tO = tmem + 256 + 128 * mi;
         auto wait_w = [&](int b, uint32_t parity, int site) {
-            const bool r = wait_or_abort(bar(b), parity, prm.err, site, abort_flag);
-            return __all_sync(0xffffffffu, r);
+            return mbar_wait_warp(bar(b), parity, prm.err, site, abort_flag);
         };
         auto issue_s = [&](int stage) {
             const uint64_t db = dk0 + (uint64_t)(stage * (kTile >> 4));
@@ -565,8 +564,7 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
         const float c = prm.scale_log2;
         const float cm = kE4M3 ? 1.f : c;   // E4M3: the row maxima are already scaled by the multipliers
         auto wait_all = [&](int bb, uint32_t parity, int site) {
-            const bool r = wait_or_abort(bar(bb), parity, prm.err, site, abort_flag);
-            return __all_sync(0xffffffffu, r);
+            return mbar_wait_warp(bar(bb), parity, prm.err, site, abort_flag);
         };
         // Warps w and w + 4 (the same TMEM lanes, the two column halves) meet at a named barrier of
         // their own (1 + w % 4) for every swap, so neither may leave the loops early: after a failed

@@ -270,8 +270,7 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
         // for the accumulating MMAs that read the buffer it overwrites.
         if (nu > 0) {
             auto wait_w = [&](int b, uint32_t parity, int site) {
-                const bool r = wait_or_abort(bar(b), parity, prm.err, site, abort_flag);
-                return (bool)__all_sync(0xffffffffu, r);
+                return mbar_wait_warp(bar(b), parity, prm.err, site, abort_flag);
             };
             if (warp == 9) {
                 constexpr uint32_t idS = umma_idesc_bf16(128, kQT, false);
@@ -317,8 +316,7 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
         // ---------------------------------------------------------------- softmax + epilogue
         const float c = prm.scale_log2;
         auto wait_all = [&](int b, uint32_t parity, int site) {
-            const bool r = wait_or_abort(bar(b), parity, prm.err, site, abort_flag);
-            return __all_sync(0xffffffffu, r);
+            return mbar_wait_warp(bar(b), parity, prm.err, site, abort_flag);
         };
         bool ok = true;
         for (int u = 0; u < nu; ++u) {
@@ -560,8 +558,7 @@ prefill_bwd_dq_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
         // warp 9 the S and dP, warp 10 the accumulating MMAs, as in the dK/dV pass
         if (nu > 0) {
             auto wait_w = [&](int b, uint32_t parity, int site) {
-                const bool r = wait_or_abort(bar(b), parity, prm.err, site, abort_flag);
-                return (bool)__all_sync(0xffffffffu, r);
+                return mbar_wait_warp(bar(b), parity, prm.err, site, abort_flag);
             };
             if (warp == 9) {
                 // S = Q K^T and dP = dO V^T of step u into buffer u % DEPTH (A from tensor memory)
@@ -615,8 +612,7 @@ prefill_bwd_dq_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
         }
         const uint64_t c2 = f2_pack(c, c);
         auto wait_all = [&](int b, uint32_t parity, int site) {
-            const bool r = wait_or_abort(bar(b), parity, prm.err, site, abort_flag);
-            return __all_sync(0xffffffffu, r);
+            return mbar_wait_warp(bar(b), parity, prm.err, site, abort_flag);
         };
         // Q and dO rows of this query into tensor memory (dims 64 ch .. 64 ch + 63), and the row's
         // statistics: D = dO . O (fp32, the two column halves added through shared memory) and

@@ -327,8 +327,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
             const uint64_t dk = umma_desc_sw128(smem_u32(sk), 16, 1024), dv = umma_desc_sw128(smem_u32(sv), kPanel, 1024);
             const uint32_t tS = tmem + 128 * i, tO = tmem + 256 + 128 * i;
             auto wait = [&](int b, uint32_t parity, int site) {
-                const bool r = wait_or_abort<false>(bar(b), parity, prm.err, site, abort_flag);
-                return (bool)__all_sync(0xffffffffu, r);
+                return mbar_wait_warp(bar(b), parity, prm.err, site, abort_flag);
             };
             auto commit = [&](int b) {
                 if (CG == 2) umma_commit_pair_warp(bar(b));
@@ -412,8 +411,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
         const float c = prm.scale_log2;
         // every decision below is warp-uniform: the TMEM loads and stores are warp-collective
         auto wait_all = [&](int b, uint32_t parity, int site) {
-            const bool r = wait_or_abort<false>(bar(b), parity, prm.err, site, abort_flag);
-            return (bool)__all_sync(0xffffffffu, r);
+            return mbar_wait_warp(bar(b), parity, prm.err, site, abort_flag);
         };
         bool ok = true;
         int t_tile = 0;   // tiles so far
