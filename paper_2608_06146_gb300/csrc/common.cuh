@@ -67,6 +67,16 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
     asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+// One arrival of a converged warp, by an elected lane (predicated, no branch; callers order the other
+// lanes' accesses before it with __syncwarp).
+__device__ __forceinline__ void mbar_arrive_warp(uint32_t bar)
+{
+    asm volatile(
+        "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+        " @e mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];\n}" ::"r"(bar)
+        : "memory");
+}
+
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;

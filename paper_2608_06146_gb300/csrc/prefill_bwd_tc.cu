@@ -8,34 +8,36 @@
 //
 // dK/dV pass: a unit is a (128-key k-tile, KV head), units taken in the key-major map's order (most
 //   work first), run by a cluster of 1, 2, 4 or 8 CTAs that share out its steps and add their fp32 sums
-//   through distributed shared memory (pick_cluster below). K and V of the tile sit in shared memory
-//   for the whole walk.
-//   For every (64-row q-tile that sees the k-tile, query head reading the KV head) step the tensor
-//   cores form S^T = K Q^T and dP^T = V dO^T (M = 128 keys, N = 32 queries, B from shared memory),
-//   the softmax warps write P^T and dS^T back into tensor memory as bf16, and dV += P^T dO,
-//   dK += dS^T Q accumulate in tensor memory over the whole walk. Every query that sees a
-//   shared-stream key (the stream's later tokens and each branch forked after it) therefore adds
-//   into that key's gradient inside one CTA: the scatter-add of the gather's backward, with nothing
-//   scattered.
-// dQ pass: one CTA per (128-row q-tile, query head), heavier q-tiles first, Q and dO resident in
-//   tensor memory. It walks the query-major map of 32-key k-tiles: S = Q K^T, dP = dO V^T, dS written
-//   back as bf16, dQ += dS K.
+//   through distributed shared memory (pick_cluster below). For every (64-row q-tile that sees the
+//   k-tile, query head reading the KV head) step the tensor cores form S^T = K Q^T (K from shared
+//   memory) and dP^T = V dO^T (V copied to tensor memory once), the softmax warps write P^T and dS^T
+//   as bf16 over S^T, and dV += P^T dO, dK += dS^T Q accumulate in tensor memory over the whole walk.
+//   Every query that sees a shared-stream key (the stream's later tokens and each branch forked after
+//   it) therefore adds into that key's gradient inside one cluster: the scatter-add of the gather's
+//   backward, with nothing scattered.
+// dQ pass: one CTA per (128-row q-tile, query head), heavier q-tiles first. It walks the query-major
+//   map of 64-key k-tiles: S = Q K^T (Q in tensor memory), dP = dO V^T (dO in shared memory), dS as
+//   bf16 over S, dQ += dS K.
 //
-// Every MMA reads at most one operand from shared memory (the other lives in tensor memory), which
-// keeps the narrow steps at the tensor cores' rate instead of shared memory's. Tensor memory holds
-// the resident A operands (128 columns), the accumulators (dV and dK: 256; dQ: 128) and, in what
-// is left, as many step buffers (S and dP, 2 x 32 columns each) as fit: 2 in the dK/dV pass, 4 in
-// the dQ pass. While the softmax warps turn step u into P and dS, the tensor cores run the
-// accumulating MMAs of step u-1 and the S and dP of the steps after u. A softmax warp owns 32 TMEM
-// lanes (rows) and one 16-column half of a step and packs its 16 bf16 results into the first 8
-// columns of its own half, so no warp overwrites a column another warp still has to read; the
-// accumulating MMAs read the two k-slices at columns 0 and 16 of the buffer.
+// What bounds a step is less its MMAs (about 1150 cycles in the dK/dV pass, 900 in the dQ pass, of
+// 1500 and 1000) than the chain S -> softmax -> accumulation -> S, whose hand-overs take 300 to 400 cycles
+// each because a warp's wait queues up behind the MMAs it has issued. So:
+// - S, dP and the accumulating MMAs are issued by a warp each;
+// - P and dS share S's columns, so dP's buffer is free again as soon as it is read, and the room that
+//   gives holds V (dK/dV pass) or a third S buffer (dQ pass);
+// - waits and roles are uniform per warp (see mbar_wait_warp), and a step's map entry is read a step ahead.
+// A packed batch of 34107 tokens, 16 query heads: dK/dV pass 735 -> 657 us, dQ pass 644 -> 487 us (of
+// which 70 us are its tiles of Q, dO and O, now copied by TMA: the rows read lane by lane took 8000
+// cycles a CTA). One page of 3419 tokens: both passes 161 -> 140 us.
 //
-// Warp roles (320 threads): warps 0-7 softmax and epilogue (they also store the resident operands
-// into tensor memory), warp 8 TMA producer, warp 9 TMEM allocation and MMA issue (converged warp,
-// one elected lane issues). Every wait is bounded; a wait that runs out records an error and all
-// roles leave their loops, the MMA warp waits for its MMAs, the producer for its copies, and tensor
-// memory is released.
+// A softmax warp owns 32 TMEM lanes (rows) and one 32-column half of a step. Its bf16 results go to the
+// first 16 columns of its own half of S (dS of the dK/dV pass to the other 16), so no warp overwrites
+// a column another warp still has to read.
+//
+// Warp roles (384 threads): warps 0-7 softmax and epilogue, warp 8 TMA producer, warp 9 TMEM allocation
+// and S, warp 10 the accumulating MMAs, warp 11 dP (converged warps, one elected lane issues). Every
+// wait is bounded; a wait that runs out records an error and all roles leave their loops, the MMA
+// warps wait for their MMAs, the producer for its copies, and tensor memory is released.
 #include <math.h>
 
 #include <algorithm>
@@ -47,20 +49,18 @@
 namespace {
 
 constexpr int kD = 128;
-constexpr int kThreads = 352;
+constexpr int kThreads = 384;
 constexpr uint32_t kTmemCols = 512;
 
 struct BwdParams {
     const int32_t *spans, *ptr, *idx, *order;
     const int8_t *kind;
     float *lt, *dt;                     // [Hq][t_pad]: -lse2 and D (written by the dQ pass, read by the dK/dV pass)
-    const __nv_bfloat16 *o;             // the forward's output (dQ pass: D = dO . O)
     const float *lse;                   // the forward's log-sum-exp, natural log, [T][Hq]
-    const __nv_bfloat16 *a0, *a1;       // the pass's tensor-memory operands: dQ pass Q, dO; dK/dV pass K, V
     int64_t T, t_pad;
     int32_t num_q_heads, num_kv_heads, num_tiles;
     float scale_log2, scale;
-    __nv_bfloat16 *out0, *out1;         // dK/dV pass: dK, dV; dQ pass: dQ
+    __nv_bfloat16 *out0, *out1;         // dK/dV pass: dK, dV
     int *err;
 };
 
@@ -81,19 +81,6 @@ __host__ __device__ constexpr uint32_t slice_col(int k)
     return (uint32_t)((k / per_half) * (W / 2) + (k % per_half) * 8);
 }
 
-template <int N>
-__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[N])
-{
-    static_assert(N == 16 || N == 32, "16 or 32 columns");
-    if constexpr (N == 32) tmem_ld32(taddr, r); else tmem_ld16(taddr, r);
-}
-template <int N>
-__device__ __forceinline__ void tmem_st_cols(uint32_t taddr, const uint32_t (&r)[N])
-{
-    static_assert(N == 8 || N == 16, "8 or 16 columns");
-    if constexpr (N == 16) tmem_st16(taddr, r); else tmem_st8(taddr, r);
-}
-
 __device__ __forceinline__ void store_row_bf16(__nv_bfloat16 *dst, const float (&o)[16], float mul)
 {
 #pragma unroll
@@ -106,32 +93,6 @@ __device__ __forceinline__ void store_row_bf16(__nv_bfloat16 *dst, const float (
         *reinterpret_cast<uint4 *>(dst + i) = w;
     }
 }
-__device__ __forceinline__ void store_row_bf16(__nv_bfloat16 *dst, const uint32_t (&o)[32], float mul)
-{
-#pragma unroll
-    for (int i = 0; i < 32; i += 8) {
-        uint4 w;
-        w.x = pack_bf16x2(__uint_as_float(o[i]) * mul, __uint_as_float(o[i + 1]) * mul);
-        w.y = pack_bf16x2(__uint_as_float(o[i + 2]) * mul, __uint_as_float(o[i + 3]) * mul);
-        w.z = pack_bf16x2(__uint_as_float(o[i + 4]) * mul, __uint_as_float(o[i + 5]) * mul);
-        w.w = pack_bf16x2(__uint_as_float(o[i + 6]) * mul, __uint_as_float(o[i + 7]) * mul);
-        *reinterpret_cast<uint4 *>(dst + i) = w;
-    }
-}
-
-// Stores 64 bf16 of a row (global, 16-byte aligned; zeros when src is null) into 32 TMEM columns of
-// the calling thread's lane: the K-major A-operand layout (column c holds elements 2c, 2c+1).
-__device__ __forceinline__ void row_to_tmem(uint32_t taddr, const __nv_bfloat16 *src)
-{
-    uint32_t w[32];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const uint4 x = src ? reinterpret_cast<const uint4 *>(src)[i] : make_uint4(0u, 0u, 0u, 0u);
-        w[4 * i] = x.x; w[4 * i + 1] = x.y; w[4 * i + 2] = x.z; w[4 * i + 3] = x.w;
-    }
-    tmem_st32(taddr, w);
-}
-
 __device__ __forceinline__ int clamp_w(int x, int w) { return min(max(x, 0), w); }
 
 // 32 x 32 bit-matrix transpose across a warp: lane r holds row r (bit c = element (r, c)); on return
@@ -157,7 +118,7 @@ namespace dkv {
 constexpr int kKT = PADOC_BWD_DKV_K_TILE;   // 128 keys: the M of every MMA
 constexpr int kQT = PADOC_BWD_DKV_Q_TILE;   // 64 queries per step
 constexpr int kStages = 4;   // (3: the Q of the step after next is still on its way, +1.5% time)
-constexpr uint32_t kColS = 0, kColDP = 128, kColAcc0 = 256, kColAcc1 = 384;
+constexpr uint32_t kColS = 0, kColDP = 128, kColV = 192, kColAcc0 = 256, kColAcc1 = 384;   // kColS: two buffers
 constexpr int kKPanel = kKT * 128;           // [128 rows][64 bf16]
 constexpr int kQPanel = kQT * 128;           // [64 rows][64 bf16]
 constexpr int kKTile = 2 * kKPanel;
@@ -168,10 +129,12 @@ enum {
     B_QFULL = 1,                  // [stage]
     B_QEMPTY = 1 + kStages,       // [stage]
     B_SFULL = 1 + 2 * kStages,    // [step parity]
-    B_PFULL = 3 + 2 * kStages,    // [step parity], 256 arrivals
-    B_FINAL = 5 + 2 * kStages,    // [issuing warp]
-    B_ACC = 7 + 2 * kStages,      // [step parity]: the step's accumulating MMAs are done
-    B_COUNT = 9 + 2 * kStages
+    B_PFULL = 3 + 2 * kStages,    // [step parity], an arrival per softmax warp
+    B_ACC = 5 + 2 * kStages,      // [step parity]: the step's accumulating MMAs are done
+    B_DPFREE = 7 + 2 * kStages,   // dP is read (an arrival per softmax warp)
+    B_VT = 8 + 2 * kStages,       // V is in tensor memory (an arrival per softmax warp)
+    B_FINAL = 9 + 2 * kStages,    // [issuing warp]
+    B_COUNT = 12 + 2 * kStages
 };
 constexpr size_t kSmemBytes = 1024 + 2 * (size_t)kKTile + 2 * (size_t)kStages * kQTile + (size_t)kStages * kAuxBytes +
                               B_COUNT * 8 + 64;
@@ -196,17 +159,19 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
     uint32_t *tmem_slot = (uint32_t *)(bars + B_COUNT);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (a value the compiler knows to be warp-uniform)
     const int hkv = prm.num_kv_heads, group = prm.num_q_heads / hkv;
     // the cluster's unit, and this CTA's steps of it: ub .. ub + nu - 1
     const int unit = (int)blockIdx.x / NC, rank = (int)blockIdx.x % NC, g = unit % hkv;
-    const int kt = prm.order[unit / hkv];
-    const int e0 = prm.ptr[kt], steps = (prm.ptr[kt + 1] - e0) * group;
+    const int kt = __shfl_sync(0xffffffffu, prm.order[unit / hkv], 0);
+    const int e0 = __shfl_sync(0xffffffffu, prm.ptr[kt], 0), steps = (__shfl_sync(0xffffffffu, prm.ptr[kt + 1], 0) - e0) * group;
     const int ub = (int)((int64_t)steps * rank / NC), nu = (int)((int64_t)steps * (rank + 1) / NC) - ub;
     auto bar = [&](int i) { return smem_u32(&bars[i]); };
 
     if (tid == 0) {
-        for (int i = 0; i < B_COUNT; ++i) mbar_init(bar(i), (i == B_PFULL || i == B_PFULL + 1) ? 256 : 1);
+        for (int i = 0; i < B_COUNT; ++i) mbar_init(bar(i), (i == B_PFULL || i == B_PFULL + 1 || i == B_DPFREE || i == B_VT) ? 8
+                                                                  : i == B_SFULL || i == B_SFULL + 1 ? 2 : 1);
         *abort_flag = 0;
         fence_barrier_init();
     }
@@ -217,7 +182,7 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     const int lq = warp & 3, ch = warp >> 2;          // softmax warps: TMEM lane quarter, column half
     const int key = kt * kKT + lq * 32 + lane;
     const uint32_t lanes = (uint32_t)(lq * 32) << 16;
@@ -263,11 +228,11 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
             for (int u = (issued > kStages ? issued - kStages : 0); u < issued; ++u)
                 mbar_wait_bounded(bar(B_QFULL + u % kStages), (u / kStages) & 1, prm.err, 52);
         }
-    } else if (warp == 9 || warp == 10) {
+    } else if (warp >= 9) {
         // ---------------------------------------------------------------- MMA issuers (whole warps)
-        // Warp 9 issues the S^T and dP^T, warp 10 the accumulating MMAs, so that one's waits (each
-        // issued behind the MMAs before it) leave the tensor cores the other's MMAs; a step's S^T waits
-        // for the accumulating MMAs that read the buffer it overwrites.
+        // Warp 9 S^T, warp 11 dP^T, warp 10 the accumulating MMAs: one's waits, each behind the MMAs it
+        // has issued, leave the tensor cores the others' MMAs. A step's S^T waits for the accumulating
+        // MMAs that read the buffer it overwrites, its dP^T for the softmax warps' reads of the last one.
         if (nu > 0) {
             auto wait_w = [&](int b, uint32_t parity, int site) {
                 return mbar_wait_warp(bar(b), parity, prm.err, site, abort_flag);
@@ -275,7 +240,6 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
             if (warp == 9) {
                 constexpr uint32_t idS = umma_idesc_bf16(128, kQT, false);
                 const uint64_t dK = umma_desc_sw128(smem_u32(sk), 16, 1024);
-                const uint64_t dV = umma_desc_sw128(smem_u32(sv), 16, 1024);
                 bool ok = wait_w(B_KV, 0, 60);
                 for (int u = 0; ok && u < nu; ++u) {
                     const int s = u % kStages;
@@ -284,9 +248,19 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
                     if (!ok) break;
                     tc_fence_after();
                     const uint64_t dq = umma_desc_sw128(smem_u32(sq + s * kQTile), 16, 1024);
-                    const uint64_t dg = umma_desc_sw128(smem_u32(sg + s * kQTile), 16, 1024);
                     umma_bf16_ss_k128_warp<1, kKPanel, kQPanel>(tmem + kColS + b, dK, dq, idS);
-                    umma_bf16_ss_k128_warp<1, kKPanel, kQPanel>(tmem + kColDP + b, dV, dg, idS);
+                    umma_commit_warp(bar(B_SFULL + (u & 1)));
+                }
+            } else if (warp == 11) {
+                constexpr uint32_t idS = umma_idesc_bf16(128, kQT, false);
+                bool ok = wait_w(B_VT, 0, 66);
+                for (int u = 0; ok && u < nu; ++u) {
+                    const int s = u % kStages;
+                    ok = wait_w(B_QFULL + s, (u / kStages) & 1, 67) && (u == 0 || wait_w(B_DPFREE, (u - 1) & 1, 65));
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint64_t dg = umma_desc_sw128(smem_u32(sg + s * kQTile), 16, 1024);
+                    umma_bf16_ts_k128_warp<kQPanel>(tmem + kColDP, tmem + kColV, dg, idS);
                     umma_commit_warp(bar(B_SFULL + (u & 1)));
                 }
             } else {
@@ -303,7 +277,7 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
                     umma_bf16_ts_k64_mn_warp<1, slice_col<kQT>(1), slice_col<kQT>(2), slice_col<kQT>(3)>(
                         tmem + kColAcc0, tmem + kColS + b, gmn, idAcc, u > 0);
                     umma_bf16_ts_k64_mn_warp<1, slice_col<kQT>(1), slice_col<kQT>(2), slice_col<kQT>(3)>(
-                        tmem + kColAcc1, tmem + kColDP + b, qmn, idAcc, u > 0);
+                        tmem + kColAcc1, tmem + kColS + b + 16, qmn, idAcc, u > 0);
                     umma_commit_warp(bar(B_ACC + (u & 1)));
                     umma_commit_warp(bar(B_QEMPTY + s));
                 }
@@ -319,20 +293,41 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
             return mbar_wait_warp(bar(b), parity, prm.err, site, abort_flag);
         };
         bool ok = true;
-        for (int u = 0; u < nu; ++u) {
+        if (nu > 0 && (ok = wait_all(B_KV, 0, 73))) {   // V's rows into tensor memory, 64 dims a thread
+            uint32_t w[32];
+            const uint8_t *row = sv + ch * kKPanel + (lq * 32 + lane) * 128;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint4 x = *reinterpret_cast<const uint4 *>(row + ((i ^ (lane & 7)) * 16));
+                w[4 * i] = x.x; w[4 * i + 1] = x.y; w[4 * i + 2] = x.z; w[4 * i + 3] = x.w;
+            }
+            tmem_st32(tmem + lanes + kColV + 32 * ch, w);
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            mbar_arrive_warp(bar(B_VT));
+        }
+        // the next step's entry, read a step ahead
+        int e = e0 + ub / group, left = group - ub % group;   // steps left of entry e
+        int kind = nu > 0 ? prm.kind[e] : 0, qtile = nu > 0 ? prm.idx[e] : 0;
+        for (int u = 0; ok && u < nu; ++u) {
             const int s = u % kStages;
             const uint32_t b = (uint32_t)(u & 1) * 64 + 32 * ch;
-            const int e = e0 + (ub + u) / group;
-            const bool partial = prm.kind[e] != PADOC_TILE_FULL;
-            const int qbase = prm.idx[e] * kQT + 32 * ch;
-            if (!wait_all(B_SFULL + (u & 1), (u >> 1) & 1, 70) || !wait_all(B_QFULL + s, (u / kStages) & 1, 71)) {
+            const bool partial = __any_sync(0xffffffffu, kind != PADOC_TILE_FULL);
+            const int qbase = qtile * kQT + 32 * ch;
+            if (!wait_all(B_QFULL + s, (u / kStages) & 1, 71) || !wait_all(B_SFULL + (u & 1), (u >> 1) & 1, 70)) {
                 ok = false;
                 break;
             }
             tc_fence_after();
+            if (--left == 0 && u + 1 < nu) {
+                left = group;
+                kind = prm.kind[++e];
+                qtile = prm.idx[e];
+            }
             uint32_t sr[32], dr[32];
             tmem_ld32(tmem + lanes + kColS + b, sr);
-            tmem_ld32(tmem + lanes + kColDP + b, dr);
+            tmem_ld32(tmem + lanes + kColDP + 32 * ch, dr);
             const float4 *la = reinterpret_cast<const float4 *>(aux + s * kAuxBytes) + 8 * ch;
             const float4 *da = reinterpret_cast<const float4 *>(aux + s * kAuxBytes + kQT * 4) + 8 * ch;
             const int4 *sp = reinterpret_cast<const int4 *>(aux + s * kAuxBytes + 2 * kQT * 4) + 32 * ch;
@@ -354,6 +349,9 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
                 vis = transpose32_warp(x, lane);
             }
             tmem_ld_wait();
+            tc_fence_before();
+            __syncwarp();
+            mbar_arrive_warp(bar(B_DPFREE));
             uint32_t pk[16], dk[16];
             const uint64_t c2 = f2_pack(c, c);
             // two query columns per packed instruction: P = exp2(S c - lse2), dS = P (dP - D)
@@ -383,10 +381,11 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
             };
             if (partial) column_pairs(std::true_type{}); else column_pairs(std::false_type{});
             tmem_st16(tmem + lanes + kColS + b, pk);
-            tmem_st16(tmem + lanes + kColDP + b, dk);
+            tmem_st16(tmem + lanes + kColS + b + 16, dk);
             tmem_st_wait();
             tc_fence_before();
-            mbar_arrive(bar(B_PFULL + (u & 1)));
+            __syncwarp();
+            mbar_arrive_warp(bar(B_PFULL + (u & 1)));
         }
         sums = ok && (nu == 0 || wait_all(B_FINAL + 1, 0, 72));
         tc_fence_after();
@@ -468,57 +467,64 @@ prefill_bwd_dkv_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_co
 // ================================================================================================
 // dQ pass
 // ================================================================================================
-// TMEM: Q at [0,64) and dO at [64,128) as A operands, the step buffers at 128 + 2W i (S, then dP),
-// dQ at [384,512).
-template <int W>
-struct DqCfg {
-    static constexpr int kQT = PADOC_BWD_DQ_Q_TILE;    // 128 query rows: the M of every MMA
-    static constexpr int kDepth = 256 / (2 * W);
-    static constexpr int kStages = W == 32 ? 8 : W == 64 ? 5 : 3;
-    static constexpr int kPanel = W * 128;
-    static constexpr int kTile = 2 * kPanel;            // K or V of one step
-    static constexpr uint32_t kColQ = 0, kColG = 64, kColBuf = 128, kColDQ = 384;
-    enum {
-        B_QG = 0,                       // 256 arrivals: Q and dO stored into tensor memory
-        B_KFULL = 1,                    // [stage]
-        B_KEMPTY = 1 + kStages,         // [stage]
-        B_SFULL = 1 + 2 * kStages,      // [buffer]
-        B_PFULL = 1 + 2 * kStages + kDepth,   // [buffer], 256 arrivals
-        B_FINAL = 1 + 2 * kStages + 2 * kDepth,     // [issuing warp]
-        B_ACC = 3 + 2 * kStages + 2 * kDepth,       // [buffer]: the accumulating MMAs that read it are done
-        B_COUNT = 3 + 2 * kStages + 3 * kDepth
-    };
-    static constexpr size_t kSmemBytes = 1024 + (size_t)kStages * 2 * kTile + B_COUNT * 8 + 64 + 2 * kQT * 4;
-    static_assert(kDepth >= 1 && W % 32 == 0, "step width");
+namespace dqp {
+constexpr int kQT = PADOC_BWD_DQ_Q_TILE;     // 128 query rows: the M of every MMA
+constexpr int kW = PADOC_BWD_DQ_K_TILE;      // 64 keys per step
+constexpr int kStages = 4;
+constexpr int kQPanel = kQT * 128;           // [128 rows][64 bf16]
+constexpr int kQTile = 2 * kQPanel;
+constexpr int kKPanel = kW * 128;            // [64 rows][64 bf16]
+constexpr int kKTile = 2 * kKPanel;          // K or V of one step
+constexpr int kSlots = 3;                    // S buffers; a step's dS takes its S's place
+constexpr uint32_t kColQ = 0, kColS = 64, kColDP = 256, kColDQ = 384;   // Q (A operand), S x 3, dP x 2, dQ
+static_assert(kW == 64, "the accumulating block takes four K-steps");
+enum {
+    B_ROWS = 0,                    // Q, dO and O have landed
+    B_QT = 1,                      // Q is in tensor memory (an arrival per softmax warp)
+    B_KFULL = 2,                   // [stage]
+    B_KEMPTY = 2 + kStages,        // [stage]
+    B_SFULL = 2 + 2 * kStages,     // [slot]: S and dP (an arrival each)
+    B_PFULL = 5 + 2 * kStages,     // [slot]: dS (an arrival per softmax warp)
+    B_ACC = 8 + 2 * kStages,       // [slot]: the accumulating MMAs that read it are done
+    B_DPFREE = 11 + 2 * kStages,   // [step parity]: dP is read (an arrival per softmax warp)
+    B_FINAL = 13 + 2 * kStages,    // [issuing warp]
+    B_COUNT = 16 + 2 * kStages
 };
+constexpr size_t kSmemBytes = 1024 + 3 * (size_t)kQTile + 2 * (size_t)kStages * kKTile + B_COUNT * 8 + 64 + 2 * kQT * 4;
+}  // namespace dqp
 
-template <int W>
 __global__ void __launch_bounds__(kThreads, 1)
-prefill_bwd_dq_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
+prefill_bwd_dq_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap gmap,
+                      const __grid_constant__ CUtensorMap omap, const __grid_constant__ CUtensorMap kmap,
+                      const __grid_constant__ CUtensorMap vmap, const __grid_constant__ CUtensorMap dqmap,
                       const BwdParams prm)
 {
-    using C = DqCfg<W>;
-    constexpr int S = C::kStages, DEPTH = C::kDepth;
+    using namespace dqp;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t *sk = smem;                        // [stage] K step tiles
-    uint8_t *sv = sk + S * C::kTile;           // [stage] V step tiles
-    uint64_t *bars = (uint64_t *)(sv + S * C::kTile);
-    uint32_t *tmem_slot = (uint32_t *)(bars + C::B_COUNT);
+    uint8_t *sq = smem;                        // Q, dO and O rows; dQ takes O's place
+    uint8_t *sg = sq + kQTile;
+    uint8_t *so = sg + kQTile;
+    uint8_t *sk = so + kQTile;                 // [stage] K step tiles
+    uint8_t *sv = sk + kStages * kKTile;       // [stage] V step tiles
+    uint64_t *bars = (uint64_t *)(sv + kStages * kKTile);
+    uint32_t *tmem_slot = (uint32_t *)(bars + B_COUNT);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
     float *dsum = (float *)(tmem_slot + 16);   // [2][128]: the two column halves' parts of D
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (a value the compiler knows to be warp-uniform)
     const int hq = prm.num_q_heads, group = hq / prm.num_kv_heads;
     const int qt = prm.num_tiles - 1 - (int)(blockIdx.x / hq);   // heavier q-tiles (later in a page) first
     pdl_launch_dependents();   // the dK/dV pass may take the SMs that run out of work here
     const int h = (int)(blockIdx.x % hq), g = h / group;
-    const int e0 = prm.ptr[qt], nu = prm.ptr[qt + 1] - e0;
+    const int e0 = __shfl_sync(0xffffffffu, prm.ptr[qt], 0), nu = __shfl_sync(0xffffffffu, prm.ptr[qt + 1], 0) - e0;
     auto bar = [&](int i) { return smem_u32(&bars[i]); };
 
     if (tid == 0) {
-        for (int i = 0; i < C::B_COUNT; ++i)
-            mbar_init(bar(i), (i == C::B_QG || (i >= C::B_PFULL && i < C::B_PFULL + DEPTH)) ? 256 : 1);
+        for (int i = 0; i < B_COUNT; ++i)
+            mbar_init(bar(i), i == B_QT || (i >= B_PFULL && i < B_PFULL + kSlots) || i == B_DPFREE || i == B_DPFREE + 1 ? 8
+                              : i >= B_SFULL && i < B_SFULL + kSlots ? 2 : 1);
         *abort_flag = 0;
         fence_barrier_init();
     }
@@ -529,195 +535,238 @@ prefill_bwd_dq_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    auto wait_w = [&](int b, uint32_t parity, int site) {
+        return mbar_wait_warp(bar(b), parity, prm.err, site, abort_flag);
+    };
 
     if (warp == 8) {
         // ---------------------------------------------------------------- TMA producer
-        if (lane == 0 && nu > 0) {
-            tma_prefetch_desc(&kmap);
-            tma_prefetch_desc(&vmap);
+        if (lane == 0) {
+            const uint32_t rb = bar(B_ROWS);
+            mbar_arrive_expect_tx(rb, 3 * kQTile);
+            for (int p = 0; p < 2; ++p) {
+                tma_load_2d(smem_u32(sq) + p * kQPanel, &qmap, h * kD + 64 * p, qt * kQT, rb);
+                tma_load_2d(smem_u32(sg) + p * kQPanel, &gmap, h * kD + 64 * p, qt * kQT, rb);
+                tma_load_2d(smem_u32(so) + p * kQPanel, &omap, h * kD + 64 * p, qt * kQT, rb);
+            }
             int issued = 0;
             for (int u = 0; u < nu; ++u) {
-                const int s = u % S;
-                if (u >= S && !wait_or_abort(bar(C::B_KEMPTY + s), (u / S - 1) & 1, prm.err, 80, abort_flag)) break;
-                const int k0 = prm.idx[e0 + u] * W;
-                const uint32_t fb = bar(C::B_KFULL + s);
-                const uint32_t kb = smem_u32(sk + s * C::kTile), vb = smem_u32(sv + s * C::kTile);
-                mbar_arrive_expect_tx(fb, 2 * C::kTile);
+                const int s = u % kStages;
+                if (u >= kStages && !wait_or_abort(bar(B_KEMPTY + s), (u / kStages - 1) & 1, prm.err, 80, abort_flag)) break;
+                const int k0 = prm.idx[e0 + u] * kW;
+                const uint32_t fb = bar(B_KFULL + s);
+                const uint32_t kb = smem_u32(sk + s * kKTile), vb = smem_u32(sv + s * kKTile);
+                mbar_arrive_expect_tx(fb, 2 * kKTile);
                 tma_load_2d(kb, &kmap, g * kD, k0, fb);
-                tma_load_2d(kb + C::kPanel, &kmap, g * kD + 64, k0, fb);
+                tma_load_2d(kb + kKPanel, &kmap, g * kD + 64, k0, fb);
                 tma_load_2d(vb, &vmap, g * kD, k0, fb);
-                tma_load_2d(vb + C::kPanel, &vmap, g * kD + 64, k0, fb);
+                tma_load_2d(vb + kKPanel, &vmap, g * kD + 64, k0, fb);
                 issued = u + 1;
             }
-            for (int u = (issued > S ? issued - S : 0); u < issued; ++u)
-                mbar_wait_bounded(bar(C::B_KFULL + u % S), (u / S) & 1, prm.err, 82);
+            // copies still in flight must land before the CTA's shared memory is released
+            mbar_wait_bounded(rb, 0, prm.err, 81);
+            for (int u = (issued > kStages ? issued - kStages : 0); u < issued; ++u)
+                mbar_wait_bounded(bar(B_KFULL + u % kStages), (u / kStages) & 1, prm.err, 82);
         }
-    } else if (warp == 9 || warp == 10) {
+    } else if (warp >= 9) {
         // ---------------------------------------------------------------- MMA issuers (whole warps)
-        // warp 9 the S and dP, warp 10 the accumulating MMAs, as in the dK/dV pass
+        // warp 9 S, warp 11 dP, warp 10 dQ, as in the dK/dV pass
         if (nu > 0) {
-            auto wait_w = [&](int b, uint32_t parity, int site) {
-                return mbar_wait_warp(bar(b), parity, prm.err, site, abort_flag);
-            };
+            int slot = 0;
+            uint32_t ph = 0;   // parity of the slot's use
             if (warp == 9) {
-                // S = Q K^T and dP = dO V^T of step u into buffer u % DEPTH (A from tensor memory)
-                constexpr uint32_t idS = umma_idesc_bf16(128, W, false);
-                bool ok = wait_w(C::B_QG, 0, 90);
+                // S = Q K^T, A from tensor memory
+                constexpr uint32_t idS = umma_idesc_bf16(128, kW, false);
+                bool ok = wait_w(B_QT, 0, 90);
                 for (int u = 0; ok && u < nu; ++u) {
-                    const int s = u % S;
-                    const uint32_t b = C::kColBuf + (uint32_t)(u % DEPTH) * 2 * W;
-                    ok = wait_w(C::B_KFULL + s, (u / S) & 1, 91) &&
-                         (u < DEPTH || wait_w(C::B_ACC + u % DEPTH, (u / DEPTH - 1) & 1, 93));
+                    const int s = u % kStages;
+                    ok = wait_w(B_KFULL + s, (u / kStages) & 1, 91) && (u < kSlots || wait_w(B_ACC + slot, ph ^ 1, 93));
                     if (!ok) break;
                     tc_fence_after();
-                    const uint64_t dk = umma_desc_sw128(smem_u32(sk + s * C::kTile), 16, 1024);
-                    const uint64_t dv = umma_desc_sw128(smem_u32(sv + s * C::kTile), 16, 1024);
-                    umma_bf16_ts_k128_warp<C::kPanel>(tmem + b, tmem + C::kColQ, dk, idS);
-                    umma_bf16_ts_k128_warp<C::kPanel>(tmem + b + W, tmem + C::kColG, dv, idS);
-                    umma_commit_warp(bar(C::B_SFULL + u % DEPTH));
+                    const uint64_t dk = umma_desc_sw128(smem_u32(sk + s * kKTile), 16, 1024);
+                    umma_bf16_ts_k128_warp<kKPanel>(tmem + kColS + 64 * slot, tmem + kColQ, dk, idS);
+                    umma_commit_warp(bar(B_SFULL + slot));
+                    if (++slot == kSlots) { slot = 0; ph ^= 1; }
+                }
+            } else if (warp == 11) {
+                // dP = dO V^T, both from shared memory
+                constexpr uint32_t idS = umma_idesc_bf16(128, kW, false);
+                const uint64_t dg = umma_desc_sw128(smem_u32(sg), 16, 1024);
+                bool ok = wait_w(B_ROWS, 0, 97);
+                for (int u = 0; ok && u < nu; ++u) {
+                    const int s = u % kStages;
+                    ok = wait_w(B_KFULL + s, (u / kStages) & 1, 98) &&
+                         (u < 2 || wait_w(B_DPFREE + (u & 1), ((u >> 1) - 1) & 1, 99));
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint64_t dv = umma_desc_sw128(smem_u32(sv + s * kKTile), 16, 1024);
+                    umma_bf16_ss_k128_warp<1, kQPanel, kKPanel>(tmem + kColDP + 64 * (u & 1), dg, dv, idS);
+                    umma_commit_warp(bar(B_SFULL + slot));
+                    if (++slot == kSlots) slot = 0;
                 }
             } else {
-                static_assert(W == 64, "the accumulating block takes four K-steps");
                 constexpr uint32_t idAcc = umma_idesc_bf16(128, kD, true);
                 bool ok = true;
                 for (int u = 0; ok && u < nu; ++u) {
-                    const int s = u % S;
-                    const uint32_t b = C::kColBuf + (uint32_t)(u % DEPTH) * 2 * W;
-                    if (!(ok = wait_w(C::B_PFULL + u % DEPTH, (u / DEPTH) & 1, 92))) break;
+                    const int s = u % kStages;
+                    if (!(ok = wait_w(B_PFULL + slot, ph, 92))) break;
                     tc_fence_after();
-                    // the step's K as an MN-major B operand (N = head dim, K = the W keys)
-                    const uint64_t kmn = umma_desc_sw128(smem_u32(sk + s * C::kTile), C::kPanel, 1024);
-                    umma_bf16_ts_k64_mn_warp<1, slice_col<W>(1), slice_col<W>(2), slice_col<W>(3)>(
-                        tmem + C::kColDQ, tmem + b + W, kmn, idAcc, u > 0);
-                    umma_commit_warp(bar(C::B_ACC + u % DEPTH));
-                    umma_commit_warp(bar(C::B_KEMPTY + s));
+                    // the step's K as an MN-major B operand (N = head dim, K = the 64 keys)
+                    const uint64_t kmn = umma_desc_sw128(smem_u32(sk + s * kKTile), kKPanel, 1024);
+                    umma_bf16_ts_k64_mn_warp<1, slice_col<kW>(1), slice_col<kW>(2), slice_col<kW>(3)>(
+                        tmem + kColDQ, tmem + kColS + 64 * slot, kmn, idAcc, u > 0);
+                    umma_commit_warp(bar(B_ACC + slot));
+                    umma_commit_warp(bar(B_KEMPTY + s));
+                    if (++slot == kSlots) { slot = 0; ph ^= 1; }
                 }
             }
-            umma_commit_warp(bar(C::B_FINAL + warp - 9));
-            mbar_wait_bounded(bar(C::B_FINAL + warp - 9), 0, prm.err, 94);
+            umma_commit_warp(bar(B_FINAL + warp - 9));
+            mbar_wait_bounded(bar(B_FINAL + warp - 9), 0, prm.err, 94);
         }
     } else {
         // ---------------------------------------------------------------- softmax + epilogue
-        constexpr int HW = W / 2;
         const int lq = warp & 3, ch = warp >> 2;
         const int row = lq * 32 + lane;
-        const int64_t t = (int64_t)qt * C::kQT + row;
+        const int64_t t = (int64_t)qt * kQT + row;
+        const bool in = t < prm.T;
         const uint32_t lanes = (uint32_t)(lq * 32) << 16;
         const float c = prm.scale_log2;
         int a0 = 0, a1 = 0, b0 = 0, b1 = 0;
-        if (t < prm.T) {
+        float nlrow = -INFINITY;
+        if (in) {
             const int4 w = *reinterpret_cast<const int4 *>(prm.spans + 4 * t);
             a0 = w.x; a1 = w.y; b0 = w.z; b1 = w.w;
+            const float l = prm.lse[(size_t)t * hq + h];
+            nlrow = l == -INFINITY ? -INFINITY : -l * PADOC_LOG2E;
         }
         const uint64_t c2 = f2_pack(c, c);
-        auto wait_all = [&](int b, uint32_t parity, int site) {
-            return mbar_wait_warp(bar(b), parity, prm.err, site, abort_flag);
-        };
-        // Q and dO rows of this query into tensor memory (dims 64 ch .. 64 ch + 63), and the row's
-        // statistics: D = dO . O (fp32, the two column halves added through shared memory) and
-        // -lse2; rows past T get -lse2 = -inf and D = 0, so that their P and dS are 0. Every
-        // (row, head) of [0, t_pad) belongs to exactly one CTA, which writes them for the dK/dV pass.
-        float nlrow, drow;
-        {
-            const bool in = t < prm.T;
-            const size_t off = ((size_t)(in ? t : 0) * hq + h) * kD + 64 * ch;
-            row_to_tmem(tmem + lanes + C::kColQ + 32 * ch, in ? prm.a0 + off : nullptr);
+        // Q's row of this query into tensor memory (dims 64 ch .. 64 ch + 63), and the row's statistics:
+        // D = dO . O (fp32, the two column halves added through shared memory) and -lse2; rows past T
+        // (zeros in the tiles) get -lse2 = -inf and D = 0, so that their P and dS are 0. Every (row, head)
+        // of [0, t_pad) belongs to exactly one CTA, which writes them for the dK/dV pass.
+        uint8_t *orow = so + ch * kQPanel + row * 128;
+        float drow = 0.f;
+        bool ok = wait_w(B_ROWS, 0, 100);
+        if (ok) {
+            const uint8_t *qrow = sq + ch * kQPanel + row * 128, *grow = sg + ch * kQPanel + row * 128;
             uint32_t w[32];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint4 x = *reinterpret_cast<const uint4 *>(qrow + ((i ^ (lane & 7)) * 16));
+                w[4 * i] = x.x; w[4 * i + 1] = x.y; w[4 * i + 2] = x.z; w[4 * i + 3] = x.w;
+            }
+            tmem_st32(tmem + lanes + kColQ + 32 * ch, w);
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            mbar_arrive_warp(bar(B_QT));
             uint64_t acc2 = f2_pack(0.f, 0.f);
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                const uint4 x = in ? reinterpret_cast<const uint4 *>(prm.a1 + off)[i] : make_uint4(0u, 0u, 0u, 0u);
-                const uint4 y = in ? reinterpret_cast<const uint4 *>(prm.o + off)[i] : make_uint4(0u, 0u, 0u, 0u);
+                const uint4 x = *reinterpret_cast<const uint4 *>(grow + ((i ^ (lane & 7)) * 16));
+                const uint4 y = *reinterpret_cast<const uint4 *>(orow + ((i ^ (lane & 7)) * 16));
                 const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    w[4 * i + j] = xs[j];
+                for (int j = 0; j < 4; ++j)
                     acc2 = f2_fma(f2_pack(__uint_as_float(xs[j] << 16), __uint_as_float(xs[j] & 0xffff0000u)),
                                   f2_pack(__uint_as_float(ys[j] << 16), __uint_as_float(ys[j] & 0xffff0000u)), acc2);
-                }
             }
-            tmem_st32(tmem + lanes + C::kColG + 32 * ch, w);
-            tmem_st_wait();
-            tc_fence_before();
-            mbar_arrive(bar(C::B_QG));
             float lo, hi;
             f2_unpack(acc2, lo, hi);
-            dsum[ch * C::kQT + row] = lo + hi;
-            named_bar_sync(1, 256);   // the eight softmax warps
-            drow = dsum[row] + dsum[C::kQT + row];
-            const float l = in ? prm.lse[(size_t)t * hq + h] : -INFINITY;
-            nlrow = l == -INFINITY ? -INFINITY : -l * PADOC_LOG2E;
-            if (!in) drow = 0.f;
+            dsum[ch * kQT + row] = lo + hi;
+        }
+        named_bar_sync(1, 256);   // the eight softmax warps
+        if (ok) {
+            drow = in ? dsum[row] + dsum[kQT + row] : 0.f;
             if (ch == 0) {
                 prm.lt[(size_t)h * prm.t_pad + t] = nlrow;
                 prm.dt[(size_t)h * prm.t_pad + t] = drow;
             }
         }
         const uint64_t nl2 = f2_pack(nlrow, nlrow), d2 = f2_pack(drow, drow);
-        bool ok = true;
-        for (int u = 0; u < nu; ++u) {
-            const uint32_t b = C::kColBuf + (uint32_t)(u % DEPTH) * 2 * W + HW * ch;
-            const bool partial = prm.kind[e0 + u] != PADOC_TILE_FULL;
-            const int cb = prm.idx[e0 + u] * W + HW * ch;
-            if (!wait_all(C::B_SFULL + u % DEPTH, (u / DEPTH) & 1, 95)) { ok = false; break; }
+        int slot = 0;
+        uint32_t ph = 0;
+        int kind = nu > 0 ? prm.kind[e0] : 0, ktile = nu > 0 ? prm.idx[e0] : 0;   // the next step's entry
+        for (int u = 0; ok && u < nu; ++u) {
+            const uint32_t b = tmem + lanes + kColS + 64 * slot + 32 * ch;
+            const bool partial = __any_sync(0xffffffffu, kind != PADOC_TILE_FULL);
+            const int cb = ktile * kW + 32 * ch;
+            if (!(ok = wait_w(B_SFULL + slot, ph, 95))) break;
             tc_fence_after();
-            // the thread's HW key columns in blocks of at most 32: block j's dS (bf16 pairs) goes to
-            // columns 16 j .. of its half of the dP buffer, which block j has already read
-            constexpr int HB = HW < 32 ? HW : 32;
-#pragma unroll
-            for (int j = 0; j < HW / HB; ++j) {
-                uint32_t sr[HB], dr[HB];
-                tmem_ld_cols<HB>(tmem + lanes + b + HB * j, sr);
-                tmem_ld_cols<HB>(tmem + lanes + b + W + HB * j, dr);
-                uint32_t vis = 0xffffffffu;
-                if (partial) {
-                    const int cj = cb + HB * j;
-                    const int lo0 = clamp_w(a0 - cj, HB), lo1 = clamp_w(b0 - cj, HB);
-                    vis = interval_bits(lo0, max(clamp_w(a1 - cj, HB) - lo0, 0), 0) |
-                          interval_bits(lo1, max(clamp_w(b1 - cj, HB) - lo1, 0), 0);
-                }
-                tmem_ld_wait();
-                uint32_t dk[HB / 2];
-                // two key columns per packed instruction: P = exp2(S c - lse2), dS = P (dP - D)
-                auto column_pairs = [&](auto masked) {
-#pragma unroll
-                    for (int i = 0; i < HB; i += 2) {
-                        float x0, x1;
-                        f2_unpack(f2_fma(f2_pack(__uint_as_float(sr[i]), __uint_as_float(sr[i + 1])), c2, nl2), x0, x1);
-                        float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
-                        if (decltype(masked)::value) {
-                            p0 = (vis >> i) & 1u ? p0 : 0.f;
-                            p1 = (vis >> (i + 1)) & 1u ? p1 : 0.f;
-                        }
-                        const uint64_t t = f2_sub(f2_pack(__uint_as_float(dr[i]), __uint_as_float(dr[i + 1])), d2);
-                        float d0, d1;
-                        f2_unpack(f2_mul(f2_pack(p0, p1), t), d0, d1);
-                        dk[i >> 1] = pack_bf16x2(d0, d1);
-                    }
-                };
-                if (partial) column_pairs(std::true_type{}); else column_pairs(std::false_type{});
-                tmem_st_cols<HB / 2>(tmem + lanes + b + W + (HB / 2) * j, dk);
+            if (u + 1 < nu) {
+                kind = prm.kind[e0 + u + 1];
+                ktile = prm.idx[e0 + u + 1];
             }
+            uint32_t sr[32], dr[32];
+            tmem_ld32(b, sr);
+            tmem_ld32(tmem + lanes + kColDP + 64 * (u & 1) + 32 * ch, dr);
+            uint32_t vis = 0xffffffffu;
+            if (partial) {
+                const int lo0 = clamp_w(a0 - cb, 32), lo1 = clamp_w(b0 - cb, 32);
+                vis = interval_bits(lo0, max(clamp_w(a1 - cb, 32) - lo0, 0), 0) |
+                      interval_bits(lo1, max(clamp_w(b1 - cb, 32) - lo1, 0), 0);
+            }
+            tmem_ld_wait();
+            tc_fence_before();
+            __syncwarp();
+            mbar_arrive_warp(bar(B_DPFREE + (u & 1)));
+            uint32_t dk[16];
+            // two key columns per packed instruction: P = exp2(S c - lse2), dS = P (dP - D)
+            auto column_pairs = [&](auto masked) {
+#pragma unroll
+                for (int i = 0; i < 32; i += 2) {
+                    float x0, x1;
+                    f2_unpack(f2_fma(f2_pack(__uint_as_float(sr[i]), __uint_as_float(sr[i + 1])), c2, nl2), x0, x1);
+                    float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
+                    if (decltype(masked)::value) {
+                        p0 = (vis >> i) & 1u ? p0 : 0.f;
+                        p1 = (vis >> (i + 1)) & 1u ? p1 : 0.f;
+                    }
+                    const uint64_t t2 = f2_sub(f2_pack(__uint_as_float(dr[i]), __uint_as_float(dr[i + 1])), d2);
+                    float d0, d1;
+                    f2_unpack(f2_mul(f2_pack(p0, p1), t2), d0, d1);
+                    dk[i >> 1] = pack_bf16x2(d0, d1);
+                }
+            };
+            if (partial) column_pairs(std::true_type{}); else column_pairs(std::false_type{});
+            tmem_st16(b, dk);   // over the first half of this thread's own S columns
             tmem_st_wait();
             tc_fence_before();
-            mbar_arrive(bar(C::B_PFULL + u % DEPTH));
+            __syncwarp();
+            mbar_arrive_warp(bar(B_PFULL + slot));
+            if (++slot == kSlots) { slot = 0; ph ^= 1; }
         }
-        // epilogue: dQ times scale, columns 64 ch .. 64 ch + 63 of the thread's row
-        if (ok && (nu == 0 || wait_all(C::B_FINAL + 1, 0, 96))) {
+        // epilogue: dQ times scale, columns 64 ch .. 64 ch + 63 of the thread's row, by way of O's place
+        // (each warp's own part of it) and one TMA store per warp, which leaves out the rows past T
+        if (ok && (nu == 0 || wait_w(B_FINAL + 1, 0, 96))) {
             tc_fence_after();
-            __nv_bfloat16 *dst = prm.out0 + ((size_t)(t < prm.T ? t : 0) * hq + h) * kD + 64 * ch;
 #pragma unroll
             for (int cc = 0; cc < 2; ++cc) {
                 uint32_t o[32];
                 if (nu > 0) {
-                    tmem_ld32(tmem + lanes + C::kColDQ + 64 * ch + 32 * cc, o);
+                    tmem_ld32(tmem + lanes + kColDQ + 64 * ch + 32 * cc, o);
                     tmem_ld_wait();
                 } else {
 #pragma unroll
                     for (int i = 0; i < 32; ++i) o[i] = 0u;
                 }
-                if (t < prm.T) store_row_bf16(dst + 32 * cc, o, prm.scale);
+#pragma unroll
+                for (int i = 0; i < 32; i += 8) {
+                    uint4 w;
+                    w.x = pack_bf16x2(__uint_as_float(o[i]) * prm.scale, __uint_as_float(o[i + 1]) * prm.scale);
+                    w.y = pack_bf16x2(__uint_as_float(o[i + 2]) * prm.scale, __uint_as_float(o[i + 3]) * prm.scale);
+                    w.z = pack_bf16x2(__uint_as_float(o[i + 4]) * prm.scale, __uint_as_float(o[i + 5]) * prm.scale);
+                    w.w = pack_bf16x2(__uint_as_float(o[i + 6]) * prm.scale, __uint_as_float(o[i + 7]) * prm.scale);
+                    *reinterpret_cast<uint4 *>(orow + (((4 * cc + i / 8) ^ (lane & 7)) * 16)) = w;
+                }
+            }
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                tma_store_2d(&dqmap, h * kD + 64 * ch, qt * kQT + lq * 32, smem_u32(so + ch * kQPanel + lq * 4096));
+                tma_store_commit();
+                tma_store_wait_read<0>();   // before the CTA's shared memory is released
             }
         }
     }
@@ -772,21 +821,23 @@ padoc_status padoc_launch_prefill_bwd_tc(const void *q, const void *k, const voi
                                          float *dt, int64_t t_pad, float scale, void *dq, void *dk,
                                          void *dv, cudaStream_t stream)
 {
-    constexpr int WQ = PADOC_BWD_DQ_K_TILE;
-    using CQ = DqCfg<WQ>;
     int *err = padoc_device_error_word();
     if (!err) return PADOC_ERR_CUDA;
     const int64_t T = total_tokens;
-    const int64_t nkt = (T + dkv::kKT - 1) / dkv::kKT, nqt = (T + CQ::kQT - 1) / CQ::kQT;
+    const int64_t nkt = (T + dkv::kKT - 1) / dkv::kKT, nqt = (T + dqp::kQT - 1) / dqp::kQT;
     if (8 * nkt * num_kv_heads > INT32_MAX || nqt * num_q_heads > INT32_MAX) return PADOC_ERR_UNSUPPORTED;
     const uint64_t qcols = (uint64_t)num_q_heads * kD, kcols = (uint64_t)num_kv_heads * kD;
-    CUtensorMap q64, g64, k128, v128, kmap, vmap;
+    CUtensorMap q64, g64, k128, v128, k64, v64, q128, g128, o128, dq32;
     if (!padoc_make_tmap_bf16(&q64, q, qcols, T, qcols * 2, 64, dkv::kQT) ||
         !padoc_make_tmap_bf16(&g64, dout, qcols, T, qcols * 2, 64, dkv::kQT) ||
         !padoc_make_tmap_bf16(&k128, k, kcols, T, kcols * 2, 64, dkv::kKT) ||
         !padoc_make_tmap_bf16(&v128, v, kcols, T, kcols * 2, 64, dkv::kKT) ||
-        !padoc_make_tmap_bf16(&kmap, k, kcols, T, kcols * 2, 64, WQ) ||
-        !padoc_make_tmap_bf16(&vmap, v, kcols, T, kcols * 2, 64, WQ))
+        !padoc_make_tmap_bf16(&k64, k, kcols, T, kcols * 2, 64, dqp::kW) ||
+        !padoc_make_tmap_bf16(&v64, v, kcols, T, kcols * 2, 64, dqp::kW) ||
+        !padoc_make_tmap_bf16(&q128, q, qcols, T, qcols * 2, 64, dqp::kQT) ||
+        !padoc_make_tmap_bf16(&g128, dout, qcols, T, qcols * 2, 64, dqp::kQT) ||
+        !padoc_make_tmap_bf16(&o128, out, qcols, T, qcols * 2, 64, dqp::kQT) ||
+        !padoc_make_tmap_bf16(&dq32, dq, qcols, T, qcols * 2, 64, 32))
         return PADOC_ERR_CUDA;
     BwdParams prm;
     prm.spans = spans_dev;
@@ -799,24 +850,20 @@ padoc_status padoc_launch_prefill_bwd_tc(const void *q, const void *k, const voi
     prm.scale_log2 = scale * PADOC_LOG2E;
     prm.scale = scale;
     prm.err = err;
-    prm.o = nullptr;
     prm.lse = nullptr;
 
     // the dQ pass first: it also writes -lse2 and D of every row for the dK/dV pass
-    BwdParams pq = prm;   // dQ pass over the query-major map; Q and dO go to tensor memory
+    BwdParams pq = prm;   // dQ pass over the query-major map
     pq.ptr = q_map->ptr;
     pq.idx = q_map->idx;
     pq.kind = q_map->kind;
     pq.order = nullptr;
-    pq.a0 = (const __nv_bfloat16 *)q;
-    pq.a1 = (const __nv_bfloat16 *)dout;
     pq.num_tiles = (int32_t)nqt;
-    pq.out0 = (__nv_bfloat16 *)dq;
-    pq.out1 = nullptr;
-    pq.o = (const __nv_bfloat16 *)out;
+    pq.out0 = pq.out1 = nullptr;
     pq.lse = lse;
-    if (const padoc_status sm = padoc_set_max_smem((const void *)prefill_bwd_dq_kernel<WQ>, (int)CQ::kSmemBytes)) return sm;
-    prefill_bwd_dq_kernel<WQ><<<(unsigned)(nqt * num_q_heads), kThreads, CQ::kSmemBytes, stream>>>(kmap, vmap, pq);
+    if (const padoc_status sm = padoc_set_max_smem((const void *)prefill_bwd_dq_kernel, (int)dqp::kSmemBytes)) return sm;
+    prefill_bwd_dq_kernel<<<(unsigned)(nqt * num_q_heads), kThreads, dqp::kSmemBytes, stream>>>(q128, g128, o128, k64, v64,
+                                                                                             dq32, pq);
     padoc_status st = padoc_launch_status();
     if (st != PADOC_OK) return st;
 
