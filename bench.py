@@ -46,13 +46,12 @@ FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustain
 # of each kernel as it stands; None where no capture of the current kernel exists. Decode: one step =
 # its kernels' counters added up (bf16: the decode grid and the merge, captured with the caches left
 # as the pipeline leaves them, so that the merge reads its partials from L2 as it does in the timed
-# step, the mean of two consecutive steps; E4M3: the tensor-core grid, the warp grid and the merge,
-# cold caches). Prefill: cold caches. Prefill backward: both passes and the merge of the split key
-# tiles, cold caches.
+# step, the mean of two consecutive steps; E4M3: the decode grid and the merge, cold caches, the mean
+# of two consecutive steps). Prefill: cold caches. Prefill backward: both passes, cold caches.
 TRAFFIC_BYTES = {"decode": 201_274_880,
-                 "decode_e4m3": 114_668_800,
-                 "prefill": 260_600_000,
-                 "prefill_bwd": 1_670_324_480}
+                 "decode_e4m3": 113_394_432,
+                 "prefill": 263_395_840,
+                 "prefill_bwd": 1_616_259_840}
 
 
 def load_peaks():
@@ -420,8 +419,7 @@ def bench_decode_e4m3(args, torch, dev, rank, world):
 
     timing = time_steps(args, torch, world, stream, step, steady=False)
     info = plan.info
-    # the tensor-core grid, the warp grid (the E4M3 pool runs them apart) and the merge
-    launches = (1 if info.num_tc_items > 0 else 0) + (1 if info.num_warps > 0 else 0) + 1
+    launches = (1 if info.num_tc_items > 0 or info.num_warps > 0 else 0) + 1   # the decode grid + the merge
     return dict(ms=timing["ms"], streams=S, bytes=decode_bytes(wl, kv_bytes=1, scale_bytes=4), launches=launches,
                 clocks=timing["clocks"], replicas=R)
 

@@ -519,8 +519,7 @@ struct DecodeParams;
 }
 // The decode grid (decode_tc.cu): the plan's tensor-core items, then its warp lists (wprm, the
 // warp path's arguments). k_scales / v_scales non-null: an E4M3 pool (kmap / vmap are
-// padoc_make_tmap_u8 maps of the codes), whose grid runs the tensor-core items only (the caller
-// launches decode_warp_kernel after it).
+// padoc_make_tmap_u8 maps of the codes).
 padoc_status padoc_launch_decode_tc(const CUtensorMap *kmap, const CUtensorMap *vmap, const CUtensorMap *qmap, const int32_t *plan,
                                     const padoc_decode_plan *info, const int32_t *page_table, int32_t page_stride,
                                     const int32_t *stream_table, int32_t stream_stride, int32_t num_blocks,

@@ -544,9 +544,8 @@ padoc_status build_work(int32_t num_pages, const padoc_decode_config *cfg, PlanP
         ctas = (int32_t)walk(lo, true);
         pp.cta_ptr.push_back((int32_t)tc_items.size());
         // The CTAs in order of planned load, lightest first, so that they are predicted to end in
-        // index order: warp CTA early + j then follows tensor-core CTA j's pieces in the decode grid,
-        // and takes the SM of the j-th CTA to end in a warp grid of its own (the E4M3 pool), both
-        // with the start the warp planning below gives it.
+        // index order: warp CTA early + j then follows tensor-core CTA j's pieces in the decode grid with
+        // the start the warp planning below gives it.
         std::vector<int32_t> &perm = sc.perm;
         perm.resize((size_t)ctas);
         std::iota(perm.begin(), perm.end(), 0);

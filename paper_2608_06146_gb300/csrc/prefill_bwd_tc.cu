@@ -825,7 +825,7 @@ padoc_status padoc_launch_prefill_bwd_tc(const void *q, const void *k, const voi
     if (!err) return PADOC_ERR_CUDA;
     const int64_t T = total_tokens;
     const int64_t nkt = (T + dkv::kKT - 1) / dkv::kKT, nqt = (T + dqp::kQT - 1) / dqp::kQT;
-    if (8 * nkt * num_kv_heads > INT32_MAX || nqt * num_q_heads > INT32_MAX) return PADOC_ERR_UNSUPPORTED;
+    if (2 * nkt * num_kv_heads > INT32_MAX || nqt * num_q_heads > INT32_MAX) return PADOC_ERR_UNSUPPORTED;   // (8 CTAs a unit: few units)
     const uint64_t qcols = (uint64_t)num_q_heads * kD, kcols = (uint64_t)num_kv_heads * kD;
     CUtensorMap q64, g64, k128, v128, k64, v64, q128, g128, o128, dq32;
     if (!padoc_make_tmap_bf16(&q64, q, qcols, T, qcols * 2, 64, dkv::kQT) ||

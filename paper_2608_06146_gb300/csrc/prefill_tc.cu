@@ -21,8 +21,9 @@
 //   index handed over). Every SM runs one CTA for the whole call, the next unit's queries, first K/V
 //   tiles and first S come under the softmax warps' output, which leaves through shared memory and the
 //   TMA (16-byte stores of a row per thread cost 30 us of the call's 400).
-// Together 400 -> 338 us (1.03 -> 1.23 PFLOP/s of visible entries); what is left is the tensor cores'
-// 1152 cycles a half of both heads (of ~1450) and the units' ends (~4000 cycles).
+// Together 400 -> 332 us (1.03 -> 1.25 PFLOP/s of visible entries; 338 before the waits of
+// mbar_wait_warp); what is left is the tensor cores' 1152 cycles a half of both heads (of ~1450) and the
+// units' ends (~4000 cycles).
 //
 // Warp roles (384 threads):
 //   warps 0-3 / 4-7  softmax + epilogue of head 0 / head 1; thread t owns query row t (TMEM lane
