@@ -246,6 +246,32 @@ __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk
 template <int N>
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
 
+// Asks for a CTA of this grid that has not been launched; the 16-byte answer arrives on `bar`.
+__device__ __forceinline__ void launch_control_ask(uint32_t answer, uint32_t bar)
+{
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(answer),
+                 "r"(bar)
+                 : "memory");
+}
+// Whether the answer names a CTA, now this one's to run, and its index.
+__device__ __forceinline__ bool launch_control_answer(uint32_t answer, int &x, int &y)
+{
+    uint32_t got, cx = 0, cy = 0;
+    asm volatile(
+        "{\n .reg .pred p;\n .reg .b128 a;\n"
+        " ld.shared.b128 a, [%3];\n"
+        " clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, a;\n"
+        " selp.u32 %0, 1, 0, p;\n"
+        " mov.u32 %1, 0;\n mov.u32 %2, 0;\n"
+        " @p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%1, %2, _, _}, a;\n}"
+        : "=&r"(got), "=&r"(cx), "=&r"(cy)
+        : "r"(answer)
+        : "memory");
+    x = (int)cx;
+    y = (int)cy;
+    return got != 0;
+}
+
 // L2 policy for data read once per call (the paged K/V): such lines are the first evicted, so the
 // split-K partials written in the same call stay in L2 for the merge that reads them.
 __device__ __forceinline__ uint64_t l2_evict_first_policy()

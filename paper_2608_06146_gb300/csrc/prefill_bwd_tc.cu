@@ -479,18 +479,34 @@ constexpr int kSlots = 3;                    // S buffers; a step's dS takes its
 constexpr uint32_t kColQ = 0, kColS = 64, kColDP = 256, kColDQ = 384;   // Q (A operand), S x 3, dP x 2, dQ
 static_assert(kW == 64, "the accumulating block takes four K-steps");
 enum {
-    B_ROWS = 0,                    // Q, dO and O have landed
-    B_QT = 1,                      // Q is in tensor memory (an arrival per softmax warp)
-    B_KFULL = 2,                   // [stage]
-    B_KEMPTY = 2 + kStages,        // [stage]
-    B_SFULL = 2 + 2 * kStages,     // [slot]: S and dP (an arrival each)
-    B_PFULL = 5 + 2 * kStages,     // [slot]: dS (an arrival per softmax warp)
-    B_ACC = 8 + 2 * kStages,       // [slot]: the accumulating MMAs that read it are done
-    B_DPFREE = 11 + 2 * kStages,   // [step parity]: dP is read (an arrival per softmax warp)
-    B_FINAL = 13 + 2 * kStages,    // [issuing warp]
-    B_COUNT = 16 + 2 * kStages
+    B_QROWS = 0,                   // the unit's Q has landed
+    B_GROWS = 1,                   // its dO and O have landed
+    B_QT = 2,                      // its Q is in tensor memory (an arrival per softmax warp)
+    B_D = 3,                       // its rows' halves of D are in shared memory (an arrival per softmax warp)
+    B_DREAD = 4,                   // ... and have been read, as dO and O (an arrival per softmax warp)
+    B_QFREE = 5,                   // Q's place is free for the next unit's (an arrival per softmax warp)
+    B_GFREE = 6,                   // the unit's last dP is done
+    B_DQFULL = 7,                  // the unit's dQ is complete
+    B_DQFREE = 8,                  // ... and read (an arrival per softmax warp)
+    B_NEXT = 9,                    // the launch control's answer
+    B_UFULL = 10,                  // [unit parity]
+    B_UEMPTY = 12,                 // [unit parity], an arrival per reading warp
+    B_KFULL = 14,                  // [stage]
+    B_KEMPTY = 14 + kStages,       // [stage]
+    B_SFULL = 14 + 2 * kStages,    // [slot]: S and dP (an arrival each)
+    B_PFULL = 17 + 2 * kStages,    // [slot]: dS (an arrival per softmax warp)
+    B_ACC = 20 + 2 * kStages,      // [slot]: the accumulating MMAs that read it are done
+    B_DPFREE = 23 + 2 * kStages,   // [step parity]: dP is read (an arrival per softmax warp)
+    B_FINAL = 25 + 2 * kStages,    // [issuing warp]
+    B_COUNT = 28 + 2 * kStages
 };
-constexpr size_t kSmemBytes = 1024 + 3 * (size_t)kQTile + 2 * (size_t)kStages * kKTile + B_COUNT * 8 + 64 + 2 * kQT * 4;
+struct Unit {   // nu < 0: no more units
+    int h, qt, e0, nu;
+};
+constexpr int kReaders = 11;       // softmax and issuing warps
+constexpr size_t kSmemBytes = 1024 + 3 * (size_t)kQTile + 2 * (size_t)kStages * kKTile + B_COUNT * 8 + 2 * sizeof(Unit) + 48 +
+                              2 * kQT * 4;
+static_assert(kSmemBytes <= 232448, "shared memory per CTA");
 }  // namespace dqp
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -502,29 +518,30 @@ prefill_bwd_dq_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
     using namespace dqp;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t *sq = smem;                        // Q, dO and O rows; dQ takes O's place
+    uint8_t *sq = smem;                        // Q, dO and O rows; dQ leaves by way of Q's place
     uint8_t *sg = sq + kQTile;
     uint8_t *so = sg + kQTile;
     uint8_t *sk = so + kQTile;                 // [stage] K step tiles
     uint8_t *sv = sk + kStages * kKTile;       // [stage] V step tiles
-    uint64_t *bars = (uint64_t *)(sv + kStages * kKTile);
+    Unit *units = (Unit *)(sv + kStages * kKTile);   // [2]
+    uint8_t *answer = (uint8_t *)(units + 2);  // 16 bytes
+    uint64_t *bars = (uint64_t *)(answer + 16);
     uint32_t *tmem_slot = (uint32_t *)(bars + B_COUNT);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
-    float *dsum = (float *)(tmem_slot + 16);   // [2][128]: the two column halves' parts of D
+    float *dsum = (float *)(tmem_slot + 8);    // [2][128]: the two column halves' parts of D
 
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (a value the compiler knows to be warp-uniform)
     const int hq = prm.num_q_heads, group = hq / prm.num_kv_heads;
-    const int qt = prm.num_tiles - 1 - (int)(blockIdx.x / hq);   // heavier q-tiles (later in a page) first
     pdl_launch_dependents();   // the dK/dV pass may take the SMs that run out of work here
-    const int h = (int)(blockIdx.x % hq), g = h / group;
-    const int e0 = __shfl_sync(0xffffffffu, prm.ptr[qt], 0), nu = __shfl_sync(0xffffffffu, prm.ptr[qt + 1], 0) - e0;
     auto bar = [&](int i) { return smem_u32(&bars[i]); };
 
     if (tid == 0) {
-        for (int i = 0; i < B_COUNT; ++i)
-            mbar_init(bar(i), i == B_QT || (i >= B_PFULL && i < B_PFULL + kSlots) || i == B_DPFREE || i == B_DPFREE + 1 ? 8
-                              : i >= B_SFULL && i < B_SFULL + kSlots ? 2 : 1);
+        for (int i = 0; i < B_COUNT; ++i) {
+            const bool soft = i == B_QT || i == B_D || i == B_DREAD || i == B_QFREE || i == B_DQFREE ||
+                              (i >= B_PFULL && i < B_PFULL + kSlots) || i == B_DPFREE || i == B_DPFREE + 1;
+            mbar_init(bar(i), soft ? 8 : i == B_UEMPTY || i == B_UEMPTY + 1 ? kReaders : i >= B_SFULL && i < B_SFULL + kSlots ? 2 : 1);
+        }
         *abort_flag = 0;
         fence_barrier_init();
     }
@@ -539,78 +556,144 @@ prefill_bwd_dq_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
     auto wait_w = [&](int b, uint32_t parity, int site) {
         return mbar_wait_warp(bar(b), parity, prm.err, site, abort_flag);
     };
+    // the n-th unit, as every lane of a reading warp sees it
+    auto read_unit = [&](int n, Unit &u, int site) {
+        if (!wait_w(B_UFULL + (n & 1), (n >> 1) & 1, site)) return false;
+        const Unit v = units[n & 1];
+        u.h = __shfl_sync(0xffffffffu, v.h, 0);
+        u.qt = __shfl_sync(0xffffffffu, v.qt, 0);
+        u.e0 = __shfl_sync(0xffffffffu, v.e0, 0);
+        u.nu = __shfl_sync(0xffffffffu, v.nu, 0);
+        __syncwarp();   // (every lane's read has returned before the slot may be written again)
+        mbar_arrive_warp(bar(B_UEMPTY + (n & 1)));
+        return true;
+    };
 
     if (warp == 8) {
         // ---------------------------------------------------------------- TMA producer
         if (lane == 0) {
-            const uint32_t rb = bar(B_ROWS);
-            mbar_arrive_expect_tx(rb, 3 * kQTile);
-            for (int p = 0; p < 2; ++p) {
-                tma_load_2d(smem_u32(sq) + p * kQPanel, &qmap, h * kD + 64 * p, qt * kQT, rb);
-                tma_load_2d(smem_u32(sg) + p * kQPanel, &gmap, h * kD + 64 * p, qt * kQT, rb);
-                tma_load_2d(smem_u32(so) + p * kQPanel, &omap, h * kD + 64 * p, qt * kQT, rb);
-            }
-            int issued = 0;
-            for (int u = 0; u < nu; ++u) {
-                const int s = u % kStages;
-                if (u >= kStages && !wait_or_abort(bar(B_KEMPTY + s), (u / kStages - 1) & 1, prm.err, 80, abort_flag)) break;
-                const int k0 = prm.idx[e0 + u] * kW;
-                const uint32_t fb = bar(B_KFULL + s);
-                const uint32_t kb = smem_u32(sk + s * kKTile), vb = smem_u32(sv + s * kKTile);
-                mbar_arrive_expect_tx(fb, 2 * kKTile);
-                tma_load_2d(kb, &kmap, g * kD, k0, fb);
-                tma_load_2d(kb + kKPanel, &kmap, g * kD + 64, k0, fb);
-                tma_load_2d(vb, &vmap, g * kD, k0, fb);
-                tma_load_2d(vb + kKPanel, &vmap, g * kD + 64, k0, fb);
-                issued = u + 1;
+            auto wait = [&](int b, uint32_t parity, int site) {
+                return wait_or_abort(bar(b), parity, prm.err, site, abort_flag);
+            };
+            int x = blockIdx.x, y = 0;
+            int tk = 0, nq = 0, ng = 0;   // K/V tiles, Q tiles, dO and O tiles issued so far
+            bool ok = true, more = true, asked = false;
+            // asked with the unit's last tile: early enough for the answer, and late enough that no CTA
+            // holds a second unit while others run out of work
+            auto ask = [&]() {
+                mbar_arrive_expect_tx(bar(B_NEXT), 16);
+                launch_control_ask(smem_u32(answer), bar(B_NEXT));
+                asked = true;
+            };
+            int n = 0;
+            for (;; ++n) {
+                if (n >= 2 && !wait(B_UEMPTY + (n & 1), ((n >> 1) - 1) & 1, 83)) break;
+                Unit u = {0, 0, 0, -1};
+                if (more) {
+                    u.h = x % hq;
+                    u.qt = prm.num_tiles - 1 - x / hq;   // heavier q-tiles (later in a page) first
+                    u.e0 = prm.ptr[u.qt];
+                    u.nu = max(prm.ptr[u.qt + 1] - u.e0, 0);
+                }
+                units[n & 1] = u;
+                mbar_arrive(bar(B_UFULL + (n & 1)));
+                if (u.nu < 0) break;
+                if (n > 0 && !wait(B_QFREE, (n - 1) & 1, 84)) break;
+                mbar_arrive_expect_tx(bar(B_QROWS), kQTile);
+                for (int p = 0; p < 2; ++p)
+                    tma_load_2d(smem_u32(sq) + p * kQPanel, &qmap, u.h * kD + 64 * p, u.qt * kQT, bar(B_QROWS));
+                ++nq;
+                // the first K and V tiles go before dO, whose place is free later
+                auto load_rows = [&]() {
+                    if (n > 0 && (!wait(B_DREAD, (n - 1) & 1, 85) || !wait(B_GFREE, (n - 1) & 1, 86))) return false;
+                    mbar_arrive_expect_tx(bar(B_GROWS), 2 * kQTile);
+                    for (int p = 0; p < 2; ++p) {
+                        tma_load_2d(smem_u32(sg) + p * kQPanel, &gmap, u.h * kD + 64 * p, u.qt * kQT, bar(B_GROWS));
+                        tma_load_2d(smem_u32(so) + p * kQPanel, &omap, u.h * kD + 64 * p, u.qt * kQT, bar(B_GROWS));
+                    }
+                    ++ng;
+                    return true;
+                };
+                const int g = u.h / group;
+                for (int j = 0; j < u.nu; ++j, ++tk) {
+                    if (j + 1 == u.nu) ask();
+                    const int s = tk % kStages;
+                    if (tk >= kStages && !(ok = wait(B_KEMPTY + s, (tk / kStages - 1) & 1, 80))) break;
+                    const int k0 = prm.idx[u.e0 + j] * kW;
+                    const uint32_t fb = bar(B_KFULL + s);
+                    const uint32_t kb = smem_u32(sk + s * kKTile), vb = smem_u32(sv + s * kKTile);
+                    mbar_arrive_expect_tx(fb, 2 * kKTile);
+                    tma_load_2d(kb, &kmap, g * kD, k0, fb);
+                    tma_load_2d(kb + kKPanel, &kmap, g * kD + 64, k0, fb);
+                    tma_load_2d(vb, &vmap, g * kD, k0, fb);
+                    tma_load_2d(vb + kKPanel, &vmap, g * kD + 64, k0, fb);
+                    if (j == 0 && !(ok = load_rows())) { ++tk; break; }
+                }
+                if (!ok) break;
+                if (u.nu == 0) {
+                    ask();
+                    if (!load_rows()) break;
+                }
+                if (!wait(B_NEXT, n & 1, 87)) break;
+                asked = false;
+                more = launch_control_answer(smem_u32(answer), x, y);
+                fence_proxy_async_smem();   // the answer is read before the next one may be written
             }
             // copies still in flight must land before the CTA's shared memory is released
-            mbar_wait_bounded(rb, 0, prm.err, 81);
-            for (int u = (issued > kStages ? issued - kStages : 0); u < issued; ++u)
-                mbar_wait_bounded(bar(B_KFULL + u % kStages), (u / kStages) & 1, prm.err, 82);
+            if (asked) mbar_wait_bounded(bar(B_NEXT), n & 1, prm.err, 88);
+            if (nq) mbar_wait_bounded(bar(B_QROWS), (nq - 1) & 1, prm.err, 81);
+            if (ng) mbar_wait_bounded(bar(B_GROWS), (ng - 1) & 1, prm.err, 81);
+            for (int i = max(tk - kStages, 0); i < tk; ++i)
+                mbar_wait_bounded(bar(B_KFULL + i % kStages), (i / kStages) & 1, prm.err, 82);
         }
     } else if (warp >= 9) {
         // ---------------------------------------------------------------- MMA issuers (whole warps)
-        // warp 9 S, warp 11 dP, warp 10 dQ, as in the dK/dV pass
-        if (nu > 0) {
-            int slot = 0;
-            uint32_t ph = 0;   // parity of the slot's use
+        // warp 9 S, warp 11 dP, warp 10 dQ, as in the dK/dV pass; c counts the steps of all units
+        int c = 0, slot = 0;
+        uint32_t ph = 0;   // parity of the slot's use
+        bool ok = true;
+        auto next_step = [&]() {
+            ++c;
+            if (++slot == kSlots) { slot = 0; ph ^= 1; }
+        };
+        Unit un;
+        for (int n = 0; ok && (ok = read_unit(n, un, 101)) && un.nu >= 0; ++n) {
             if (warp == 9) {
                 // S = Q K^T, A from tensor memory
                 constexpr uint32_t idS = umma_idesc_bf16(128, kW, false);
-                bool ok = wait_w(B_QT, 0, 90);
-                for (int u = 0; ok && u < nu; ++u) {
-                    const int s = u % kStages;
-                    ok = wait_w(B_KFULL + s, (u / kStages) & 1, 91) && (u < kSlots || wait_w(B_ACC + slot, ph ^ 1, 93));
+                ok = wait_w(B_QT, n & 1, 90);
+                for (int u = 0; ok && u < un.nu; ++u, next_step()) {
+                    const int s = c % kStages;
+                    ok = wait_w(B_KFULL + s, (c / kStages) & 1, 91) && (c < kSlots || wait_w(B_ACC + slot, ph ^ 1, 93));
                     if (!ok) break;
                     tc_fence_after();
                     const uint64_t dk = umma_desc_sw128(smem_u32(sk + s * kKTile), 16, 1024);
                     umma_bf16_ts_k128_warp<kKPanel>(tmem + kColS + 64 * slot, tmem + kColQ, dk, idS);
                     umma_commit_warp(bar(B_SFULL + slot));
-                    if (++slot == kSlots) { slot = 0; ph ^= 1; }
                 }
             } else if (warp == 11) {
                 // dP = dO V^T, both from shared memory
                 constexpr uint32_t idS = umma_idesc_bf16(128, kW, false);
                 const uint64_t dg = umma_desc_sw128(smem_u32(sg), 16, 1024);
-                bool ok = wait_w(B_ROWS, 0, 97);
-                for (int u = 0; ok && u < nu; ++u) {
-                    const int s = u % kStages;
-                    ok = wait_w(B_KFULL + s, (u / kStages) & 1, 98) &&
-                         (u < 2 || wait_w(B_DPFREE + (u & 1), ((u >> 1) - 1) & 1, 99));
+                ok = wait_w(B_GROWS, n & 1, 97);
+                for (int u = 0; ok && u < un.nu; ++u, next_step()) {
+                    const int s = c % kStages;
+                    ok = wait_w(B_KFULL + s, (c / kStages) & 1, 98) &&
+                         (c < 2 || wait_w(B_DPFREE + (c & 1), ((c >> 1) - 1) & 1, 99));
                     if (!ok) break;
                     tc_fence_after();
                     const uint64_t dv = umma_desc_sw128(smem_u32(sv + s * kKTile), 16, 1024);
-                    umma_bf16_ss_k128_warp<1, kQPanel, kKPanel>(tmem + kColDP + 64 * (u & 1), dg, dv, idS);
+                    umma_bf16_ss_k128_warp<1, kQPanel, kKPanel>(tmem + kColDP + 64 * (c & 1), dg, dv, idS);
                     umma_commit_warp(bar(B_SFULL + slot));
-                    if (++slot == kSlots) slot = 0;
                 }
+                umma_commit_warp(bar(B_GFREE));
             } else {
                 constexpr uint32_t idAcc = umma_idesc_bf16(128, kD, true);
-                bool ok = true;
-                for (int u = 0; ok && u < nu; ++u) {
-                    const int s = u % kStages;
-                    if (!(ok = wait_w(B_PFULL + slot, ph, 92))) break;
+                for (int u = 0; ok && u < un.nu; ++u, next_step()) {
+                    const int s = c % kStages;
+                    // (the dQ of the unit before is read before this one's first product overwrites it)
+                    ok = wait_w(B_PFULL + slot, ph, 92) && (u > 0 || n == 0 || wait_w(B_DQFREE, (n - 1) & 1, 102));
+                    if (!ok) break;
                     tc_fence_after();
                     // the step's K as an MN-major B operand (N = head dim, K = the 64 keys)
                     const uint64_t kmn = umma_desc_sw128(smem_u32(sk + s * kKTile), kKPanel, 1024);
@@ -618,49 +701,95 @@ prefill_bwd_dq_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
                         tmem + kColDQ, tmem + kColS + 64 * slot, kmn, idAcc, u > 0);
                     umma_commit_warp(bar(B_ACC + slot));
                     umma_commit_warp(bar(B_KEMPTY + s));
-                    if (++slot == kSlots) { slot = 0; ph ^= 1; }
                 }
+                umma_commit_warp(bar(B_DQFULL));
             }
-            umma_commit_warp(bar(B_FINAL + warp - 9));
-            mbar_wait_bounded(bar(B_FINAL + warp - 9), 0, prm.err, 94);
         }
+        umma_commit_warp(bar(B_FINAL + warp - 9));
+        mbar_wait_bounded(bar(B_FINAL + warp - 9), 0, prm.err, 94);
     } else {
         // ---------------------------------------------------------------- softmax + epilogue
         const int lq = warp & 3, ch = warp >> 2;
         const int row = lq * 32 + lane;
-        const int64_t t = (int64_t)qt * kQT + row;
-        const bool in = t < prm.T;
         const uint32_t lanes = (uint32_t)(lq * 32) << 16;
-        const float c = prm.scale_log2;
-        int a0 = 0, a1 = 0, b0 = 0, b1 = 0;
-        float nlrow = -INFINITY;
-        if (in) {
-            const int4 w = *reinterpret_cast<const int4 *>(prm.spans + 4 * t);
-            a0 = w.x; a1 = w.y; b0 = w.z; b1 = w.w;
-            const float l = prm.lse[(size_t)t * hq + h];
-            nlrow = l == -INFINITY ? -INFINITY : -l * PADOC_LOG2E;
-        }
-        const uint64_t c2 = f2_pack(c, c);
-        // Q's row of this query into tensor memory (dims 64 ch .. 64 ch + 63), and the row's statistics:
-        // D = dO . O (fp32, the two column halves added through shared memory) and -lse2; rows past T
-        // (zeros in the tiles) get -lse2 = -inf and D = 0, so that their P and dS are 0. Every (row, head)
-        // of [0, t_pad) belongs to exactly one CTA, which writes them for the dK/dV pass.
-        uint8_t *orow = so + ch * kQPanel + row * 128;
-        float drow = 0.f;
-        bool ok = wait_w(B_ROWS, 0, 100);
-        if (ok) {
-            const uint8_t *qrow = sq + ch * kQPanel + row * 128, *grow = sg + ch * kQPanel + row * 128;
-            uint32_t w[32];
+        const uint64_t c2 = f2_pack(prm.scale_log2, prm.scale_log2);
+        uint8_t *qrow = sq + ch * kQPanel + row * 128;
+        const uint8_t *grow = sg + ch * kQPanel + row * 128, *orow = so + ch * kQPanel + row * 128;
+        int c = 0, slot = 0;   // steps of all units
+        uint32_t ph = 0;
+        Unit un, last = {0, 0, 0, 0};
+        bool ok = true;
+        for (int n = 0; ok && (ok = read_unit(n, un, 103)); ++n) {
+            const int64_t t = (int64_t)un.qt * kQT + row;
+            const bool in = un.nu >= 0 && t < prm.T;
+            int a0 = 0, a1 = 0, b0 = 0, b1 = 0, kind = 0, ktile = 0;   // kind, ktile: the next step's entry
+            float nlrow = -INFINITY;
+            if (un.nu >= 0) {
+                if (in) {
+                    const int4 w = *reinterpret_cast<const int4 *>(prm.spans + 4 * t);
+                    a0 = w.x; a1 = w.y; b0 = w.z; b1 = w.w;
+                    const float l = prm.lse[(size_t)t * hq + un.h];
+                    nlrow = l == -INFINITY ? -INFINITY : -l * PADOC_LOG2E;
+                }
+                if (un.nu > 0) {
+                    kind = prm.kind[un.e0];
+                    ktile = prm.idx[un.e0];
+                }
+                // Q's row of this query into tensor memory (dims 64 ch .. 64 ch + 63); the S of the unit before
+                // that read the last one are done, as their steps are
+                if (!(ok = wait_w(B_QROWS, n & 1, 100))) break;
+                uint32_t w[32];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const uint4 x = *reinterpret_cast<const uint4 *>(qrow + ((i ^ (lane & 7)) * 16));
-                w[4 * i] = x.x; w[4 * i + 1] = x.y; w[4 * i + 2] = x.z; w[4 * i + 3] = x.w;
+                for (int i = 0; i < 8; ++i) {
+                    const uint4 x = *reinterpret_cast<const uint4 *>(qrow + ((i ^ (lane & 7)) * 16));
+                    w[4 * i] = x.x; w[4 * i + 1] = x.y; w[4 * i + 2] = x.z; w[4 * i + 3] = x.w;
+                }
+                tmem_st32(tmem + lanes + kColQ + 32 * ch, w);
+                tmem_st_wait();
+                tc_fence_before();
+                __syncwarp();
+                mbar_arrive_warp(bar(B_QT));
             }
-            tmem_st32(tmem + lanes + kColQ + 32 * ch, w);
-            tmem_st_wait();
-            tc_fence_before();
-            __syncwarp();
-            mbar_arrive_warp(bar(B_QT));
+            // the unit before's dQ times scale, columns 64 ch .. 64 ch + 63 of the thread's row, by way of this
+            // warp's part of Q's place and one TMA store per warp, which leaves out the rows past T
+            if (n > 0) {
+                if (!(ok = wait_w(B_DQFULL, (n - 1) & 1, 96))) break;
+                tc_fence_after();
+                uint32_t o[2][32];
+                if (last.nu > 0) {
+                    tmem_ld32(tmem + lanes + kColDQ + 64 * ch, o[0]);
+                    tmem_ld32(tmem + lanes + kColDQ + 64 * ch + 32, o[1]);
+                    tmem_ld_wait();
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) o[0][i] = o[1][i] = 0u;
+                }
+                tc_fence_before();
+                __syncwarp();
+                mbar_arrive_warp(bar(B_DQFREE));
+#pragma unroll
+                for (int i = 0; i < 64; i += 8) {
+                    auto v = [&](int k) { return __uint_as_float(o[i >> 5][(i & 31) + k]) * prm.scale; };
+                    *reinterpret_cast<uint4 *>(qrow + (((i / 8) ^ (lane & 7)) * 16)) =
+                        make_uint4(pack_bf16x2(v(0), v(1)), pack_bf16x2(v(2), v(3)), pack_bf16x2(v(4), v(5)), pack_bf16x2(v(6), v(7)));
+                }
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    tma_store_2d(&dqmap, last.h * kD + 64 * ch, last.qt * kQT + lq * 32, smem_u32(sq + ch * kQPanel + lq * 4096));
+                    tma_store_commit();
+                    tma_store_wait_read<0>();   // before the next unit's Q, or the release of shared memory
+                }
+                __syncwarp();
+            }
+            if (un.nu < 0) break;
+            if (lane == 0) mbar_arrive(bar(B_QFREE));
+            last = un;
+            // the row's statistics: D = dO . O (fp32, the two column halves added through shared memory)
+            // and -lse2; rows past T (zeros in the tiles) get -lse2 = -inf and D = 0, so that their P and dS
+            // are 0. Every (row, head) of [0, t_pad) belongs to exactly one unit, which writes them for the
+            // dK/dV pass.
+            if (!(ok = wait_w(B_GROWS, n & 1, 104) && (n == 0 || wait_w(B_DREAD, (n - 1) & 1, 105)))) break;
             uint64_t acc2 = f2_pack(0.f, 0.f);
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
@@ -675,98 +804,65 @@ prefill_bwd_dq_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
             float lo, hi;
             f2_unpack(acc2, lo, hi);
             dsum[ch * kQT + row] = lo + hi;
-        }
-        named_bar_sync(1, 256);   // the eight softmax warps
-        if (ok) {
-            drow = in ? dsum[row] + dsum[kQT + row] : 0.f;
+            __syncwarp();
+            mbar_arrive_warp(bar(B_D));
+            if (!(ok = wait_w(B_D, n & 1, 106))) break;
+            const float drow = in ? dsum[row] + dsum[kQT + row] : 0.f;
+            __syncwarp();
+            mbar_arrive_warp(bar(B_DREAD));
             if (ch == 0) {
-                prm.lt[(size_t)h * prm.t_pad + t] = nlrow;
-                prm.dt[(size_t)h * prm.t_pad + t] = drow;
+                prm.lt[(size_t)un.h * prm.t_pad + t] = nlrow;
+                prm.dt[(size_t)un.h * prm.t_pad + t] = drow;
             }
-        }
-        const uint64_t nl2 = f2_pack(nlrow, nlrow), d2 = f2_pack(drow, drow);
-        int slot = 0;
-        uint32_t ph = 0;
-        int kind = nu > 0 ? prm.kind[e0] : 0, ktile = nu > 0 ? prm.idx[e0] : 0;   // the next step's entry
-        for (int u = 0; ok && u < nu; ++u) {
-            const uint32_t b = tmem + lanes + kColS + 64 * slot + 32 * ch;
-            const bool partial = __any_sync(0xffffffffu, kind != PADOC_TILE_FULL);
-            const int cb = ktile * kW + 32 * ch;
-            if (!(ok = wait_w(B_SFULL + slot, ph, 95))) break;
-            tc_fence_after();
-            if (u + 1 < nu) {
-                kind = prm.kind[e0 + u + 1];
-                ktile = prm.idx[e0 + u + 1];
-            }
-            uint32_t sr[32], dr[32];
-            tmem_ld32(b, sr);
-            tmem_ld32(tmem + lanes + kColDP + 64 * (u & 1) + 32 * ch, dr);
-            uint32_t vis = 0xffffffffu;
-            if (partial) {
-                const int lo0 = clamp_w(a0 - cb, 32), lo1 = clamp_w(b0 - cb, 32);
-                vis = interval_bits(lo0, max(clamp_w(a1 - cb, 32) - lo0, 0), 0) |
-                      interval_bits(lo1, max(clamp_w(b1 - cb, 32) - lo1, 0), 0);
-            }
-            tmem_ld_wait();
-            tc_fence_before();
-            __syncwarp();
-            mbar_arrive_warp(bar(B_DPFREE + (u & 1)));
-            uint32_t dk[16];
-            // two key columns per packed instruction: P = exp2(S c - lse2), dS = P (dP - D)
-            auto column_pairs = [&](auto masked) {
+            const uint64_t nl2 = f2_pack(nlrow, nlrow), d2 = f2_pack(drow, drow);
+            for (int u = 0; ok && u < un.nu; ++u, ++c) {
+                const uint32_t b = tmem + lanes + kColS + 64 * slot + 32 * ch;
+                const bool partial = __any_sync(0xffffffffu, kind != PADOC_TILE_FULL);
+                const int cb = ktile * kW + 32 * ch;
+                if (!(ok = wait_w(B_SFULL + slot, ph, 95))) break;
+                tc_fence_after();
+                if (u + 1 < un.nu) {
+                    kind = prm.kind[un.e0 + u + 1];
+                    ktile = prm.idx[un.e0 + u + 1];
+                }
+                uint32_t sr[32], dr[32];
+                tmem_ld32(b, sr);
+                tmem_ld32(tmem + lanes + kColDP + 64 * (c & 1) + 32 * ch, dr);
+                uint32_t vis = 0xffffffffu;
+                if (partial) {
+                    const int lo0 = clamp_w(a0 - cb, 32), lo1 = clamp_w(b0 - cb, 32);
+                    vis = interval_bits(lo0, max(clamp_w(a1 - cb, 32) - lo0, 0), 0) |
+                          interval_bits(lo1, max(clamp_w(b1 - cb, 32) - lo1, 0), 0);
+                }
+                tmem_ld_wait();
+                tc_fence_before();
+                __syncwarp();
+                mbar_arrive_warp(bar(B_DPFREE + (c & 1)));
+                uint32_t dk[16];
+                // two key columns per packed instruction: P = exp2(S c - lse2), dS = P (dP - D)
+                auto column_pairs = [&](auto masked) {
 #pragma unroll
-                for (int i = 0; i < 32; i += 2) {
-                    float x0, x1;
-                    f2_unpack(f2_fma(f2_pack(__uint_as_float(sr[i]), __uint_as_float(sr[i + 1])), c2, nl2), x0, x1);
-                    float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
-                    if (decltype(masked)::value) {
-                        p0 = (vis >> i) & 1u ? p0 : 0.f;
-                        p1 = (vis >> (i + 1)) & 1u ? p1 : 0.f;
+                    for (int i = 0; i < 32; i += 2) {
+                        float x0, x1;
+                        f2_unpack(f2_fma(f2_pack(__uint_as_float(sr[i]), __uint_as_float(sr[i + 1])), c2, nl2), x0, x1);
+                        float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
+                        if (decltype(masked)::value) {
+                            p0 = (vis >> i) & 1u ? p0 : 0.f;
+                            p1 = (vis >> (i + 1)) & 1u ? p1 : 0.f;
+                        }
+                        const uint64_t t2 = f2_sub(f2_pack(__uint_as_float(dr[i]), __uint_as_float(dr[i + 1])), d2);
+                        float d0, d1;
+                        f2_unpack(f2_mul(f2_pack(p0, p1), t2), d0, d1);
+                        dk[i >> 1] = pack_bf16x2(d0, d1);
                     }
-                    const uint64_t t2 = f2_sub(f2_pack(__uint_as_float(dr[i]), __uint_as_float(dr[i + 1])), d2);
-                    float d0, d1;
-                    f2_unpack(f2_mul(f2_pack(p0, p1), t2), d0, d1);
-                    dk[i >> 1] = pack_bf16x2(d0, d1);
-                }
-            };
-            if (partial) column_pairs(std::true_type{}); else column_pairs(std::false_type{});
-            tmem_st16(b, dk);   // over the first half of this thread's own S columns
-            tmem_st_wait();
-            tc_fence_before();
-            __syncwarp();
-            mbar_arrive_warp(bar(B_PFULL + slot));
-            if (++slot == kSlots) { slot = 0; ph ^= 1; }
-        }
-        // epilogue: dQ times scale, columns 64 ch .. 64 ch + 63 of the thread's row, by way of O's place
-        // (each warp's own part of it) and one TMA store per warp, which leaves out the rows past T
-        if (ok && (nu == 0 || wait_w(B_FINAL + 1, 0, 96))) {
-            tc_fence_after();
-#pragma unroll
-            for (int cc = 0; cc < 2; ++cc) {
-                uint32_t o[32];
-                if (nu > 0) {
-                    tmem_ld32(tmem + lanes + kColDQ + 64 * ch + 32 * cc, o);
-                    tmem_ld_wait();
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) o[i] = 0u;
-                }
-#pragma unroll
-                for (int i = 0; i < 32; i += 8) {
-                    uint4 w;
-                    w.x = pack_bf16x2(__uint_as_float(o[i]) * prm.scale, __uint_as_float(o[i + 1]) * prm.scale);
-                    w.y = pack_bf16x2(__uint_as_float(o[i + 2]) * prm.scale, __uint_as_float(o[i + 3]) * prm.scale);
-                    w.z = pack_bf16x2(__uint_as_float(o[i + 4]) * prm.scale, __uint_as_float(o[i + 5]) * prm.scale);
-                    w.w = pack_bf16x2(__uint_as_float(o[i + 6]) * prm.scale, __uint_as_float(o[i + 7]) * prm.scale);
-                    *reinterpret_cast<uint4 *>(orow + (((4 * cc + i / 8) ^ (lane & 7)) * 16)) = w;
-                }
-            }
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) {
-                tma_store_2d(&dqmap, h * kD + 64 * ch, qt * kQT + lq * 32, smem_u32(so + ch * kQPanel + lq * 4096));
-                tma_store_commit();
-                tma_store_wait_read<0>();   // before the CTA's shared memory is released
+                };
+                if (partial) column_pairs(std::true_type{}); else column_pairs(std::false_type{});
+                tmem_st16(b, dk);   // over the first half of this thread's own S columns
+                tmem_st_wait();
+                tc_fence_before();
+                __syncwarp();
+                mbar_arrive_warp(bar(B_PFULL + slot));
+                if (++slot == kSlots) { slot = 0; ph ^= 1; }
             }
         }
     }
