@@ -51,7 +51,7 @@ FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustain
 TRAFFIC_BYTES = {"decode": 201_274_880,
                  "decode_e4m3": 113_394_432,
                  "prefill": 263_395_840,
-                 "prefill_bwd": 1_616_259_840}
+                 "prefill_bwd": 1_612_553_728}
 
 
 def load_peaks():

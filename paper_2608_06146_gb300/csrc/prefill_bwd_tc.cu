@@ -15,9 +15,10 @@
 //   Every query that sees a shared-stream key (the stream's later tokens and each branch forked after
 //   it) therefore adds into that key's gradient inside one cluster: the scatter-add of the gather's
 //   backward, with nothing scattered.
-// dQ pass: one CTA per (128-row q-tile, query head), heavier q-tiles first. It walks the query-major
-//   map of 64-key k-tiles: S = Q K^T (Q in tensor memory), dP = dO V^T (dO in shared memory), dS as
-//   bf16 over S, dQ += dS K.
+// dQ pass: a unit is a (128-row q-tile, query head), heavier q-tiles first; a running CTA takes over units
+//   not yet launched (cluster launch control), and the next unit's loads and first scores come under the
+//   last one's output. It walks the query-major map of 64-key k-tiles: S = Q K^T (Q in tensor memory),
+//   dP = dO V^T (dO in shared memory), dS as bf16 over S, dQ += dS K.
 //
 // What bounds a step is less its MMAs (about 1150 cycles in the dK/dV pass, 900 in the dQ pass, of
 // 1500 and 1000) than the chain S -> softmax -> accumulation -> S, whose hand-overs take 300 to 400 cycles
@@ -26,9 +27,10 @@
 // - P and dS share S's columns, so dP's buffer is free again as soon as it is read, and the room that
 //   gives holds V (dK/dV pass) or a third S buffer (dQ pass);
 // - waits and roles are uniform per warp (see mbar_wait_warp), and a step's map entry is read a step ahead.
-// A packed batch of 34107 tokens, 16 query heads: dK/dV pass 735 -> 657 us, dQ pass 644 -> 487 us (of
-// which 70 us are its tiles of Q, dO and O, now copied by TMA: the rows read lane by lane took 8000
-// cycles a CTA). One page of 3419 tokens: both passes 161 -> 140 us.
+// A packed batch of 34107 tokens, 16 query heads: dK/dV pass 735 -> 657 us; dQ pass 644 -> 490 us (of which
+// 70 us are its tiles of Q, dO and O, copied by TMA: the rows read lane by lane took 8000 cycles a
+// CTA), -> 440 us with units taken over (a unit's start and end were 8000 of its 35000 cycles). One page
+// of 3419 tokens: both passes 161 -> 140 -> 137 us.
 //
 // A softmax warp owns 32 TMEM lanes (rows) and one 32-column half of a step. Its bf16 results go to the
 // first 16 columns of its own half of S (dS of the dK/dV pass to the other 16), so no warp overwrites
