@@ -877,11 +877,11 @@ prefill_bwd_dq_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
 }
 
 // The CTAs that share a dK/dV unit. A page's first k-tiles are seen by all of its later queries, so the
-// largest unit is about twice the mean and a few units leave most of the chip idle: one page of 3419
-// tokens (54 units, 432 steps of 0.9 us the largest) takes 225 us with the largest units on two CTAs,
-// 105 on four, and no merge kernel follows (24 us). With more units than this the sharing's own cost (~8 us a CTA) is the larger: a
-// list-scheduling model over 60 page sets drawn from 1 to 6 pages puts the lines where they are (within
-// 10% of the best choice of the four on all of them).
+// largest unit is about twice the mean and a few units leave most of the chip idle; with many units the
+// sharing's own cost (~8 us a CTA) is the larger. Measured, both passes, with 1 / 2 / 4 / 8 CTAs a unit:
+// one page of 3419 tokens (54 units, 432 steps of 0.9 us the largest) 368 / 215 / 137 / 156 us, 34107
+// packed tokens (534 units) 1179 / 1159 / 1249 / 1517 us. A list-scheduling model over 60 page sets drawn
+// from 1 to 6 pages puts the lines where they are (within 10% of the best choice on all of them).
 int pick_cluster(int64_t units)
 {
     return units <= 45 ? 8 : units <= 160 ? 4 : units <= 560 ? 2 : 1;
