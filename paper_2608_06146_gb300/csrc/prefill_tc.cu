@@ -3,9 +3,9 @@
 // [K_{M<=f_k}; K_{Y_k}], computed in packed order without a gather).
 //
 // A work unit is a 128-row q-tile of four query heads sharing a KV head, run by a CTA pair (two heads
-// per CTA); when the GQA group is no multiple of four it is the q-tile of two heads or of one, run by
-// one CTA. It walks the q-tile's entries of the tile map: fully masked k-tiles are never visited, FULL
-// tiles skip masking, PARTIAL tiles mask each row with its two spans.
+// per CTA); in small calls, and when the GQA group is no multiple of four, it is the q-tile of one head or
+// of two, run by one CTA. It walks the q-tile's entries of the tile map: fully masked k-tiles are never
+// visited, FULL tiles skip masking, PARTIAL tiles mask each row with its two spans.
 //
 // What bounds it and why this split (8 pages, 34107 packed tokens, 16 / 2 heads; clock64 timelines):
 // - Shared-memory bandwidth. A 128 x 128 x 16 MMA with both operands in shared memory reads 8 KB in its
@@ -586,10 +586,14 @@ padoc_status padoc_launch_prefill_tc(const void *q, const void *k, const void *v
     if (!err) return PADOC_ERR_CUDA;
     const int64_t nqt = (total_tokens + kQT - 1) / kQT;
     if (nqt > 65535) return PADOC_ERR_UNSUPPORTED;
-    // CTA pairs when the heads of a KV head come in fours (at 16 / 2 heads 338 us against 400 without),
-    // else a CTA alone with two heads or one
+    // Up to two (q-tile, head) units an SM, a CTA per unit: a call then lasts as long as its longest units,
+    // and a head alone takes ~1000 cycles a half where two share the tensor cores (1450). At 16 / 2 heads, one
+    // page of 500 / 1000 / 2048 tokens takes 12.4 / 16.5 / 27.0 us against 16.5 / 21.5 / 32.9 in pairs; 3000
+    // tokens (384 units) 44.7 against 42.6. Above that, CTA pairs when the heads of a KV head come in fours
+    // (34107 tokens: 332 us against 400 with two heads on a CTA), else a CTA with two heads or one.
     const int group = num_q_heads / num_kv_heads;
-    const int cg = group % 4 == 0 ? 2 : 1;
+    const bool small = nqt * num_q_heads <= 2 * padoc_default_ctas();
+    const int cg = !small && group % 4 == 0 ? 2 : 1;
     CUtensorMap qmap, kmap, vmap, omap;
     if (!padoc_make_tmap_bf16(&qmap, q, (uint64_t)num_q_heads * kD, total_tokens, (uint64_t)num_q_heads * kD * 2, 64, kQT) ||
         !padoc_make_tmap_bf16(&kmap, k, (uint64_t)num_kv_heads * kD, total_tokens, (uint64_t)num_kv_heads * kD * 2, 64, 64 / cg) ||
@@ -609,6 +613,6 @@ padoc_status padoc_launch_prefill_tc(const void *q, const void *k, const void *v
     prm.lse = lse;
     prm.err = err;
     if (cg == 2) return launch<2, 2>(qmap, kmap, vmap, omap, prm, (unsigned)nqt, stream);
-    if (group % 2 == 0) return launch<2, 1>(qmap, kmap, vmap, omap, prm, (unsigned)nqt, stream);
+    if (!small && group % 2 == 0) return launch<2, 1>(qmap, kmap, vmap, omap, prm, (unsigned)nqt, stream);
     return launch<1, 1>(qmap, kmap, vmap, omap, prm, (unsigned)nqt, stream);
 }
