@@ -47,7 +47,8 @@ int *padoc_device_error_word()
 namespace {
 
 // The last few 2-D maps this thread encoded, by their arguments: a decoding loop encodes the same
-// pool's maps every step, and an encoding is a pure function of its arguments.
+// pool's maps every step, and an encoding is a pure function of its arguments. A backward takes ten.
+constexpr int kTmaps = 16;
 struct TmapKey {
     int dtype;
     const void *base;
@@ -60,16 +61,16 @@ struct TmapKey {
     }
 };
 struct TmapCache {
-    TmapKey key[4];
-    CUtensorMap map[4];
-    bool used[4] = {false, false, false, false};
+    TmapKey key[kTmaps];
+    CUtensorMap map[kTmaps];
+    bool used[kTmaps] = {};
     int next = 0;
 };
 thread_local TmapCache t_tmaps;
 
 bool tmap_cached(const TmapKey &k, CUtensorMap *map)
 {
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < kTmaps; ++i)
         if (t_tmaps.used[i] && t_tmaps.key[i] == k) {
             *map = t_tmaps.map[i];
             return true;
@@ -80,7 +81,7 @@ bool tmap_cached(const TmapKey &k, CUtensorMap *map)
 void tmap_remember(const TmapKey &k, const CUtensorMap &map)
 {
     const int i = t_tmaps.next;
-    t_tmaps.next = (i + 1) & 3;
+    t_tmaps.next = (i + 1) % kTmaps;
     t_tmaps.key[i] = k;
     t_tmaps.map[i] = map;
     t_tmaps.used[i] = true;
