@@ -348,7 +348,8 @@ __global__ void __launch_bounds__(128) decode_f32_kernel(const float *__restrict
 }
 
 // The bf16 path's split-K decode over either pool: the tensor-core grid for the shared streams of
-// dense pages, the warp grid for the rest, and the merge; arguments validated by the caller.
+// dense pages and the warp lists for the rest in one decode grid, then the merge; arguments validated by
+// the caller.
 struct DecodePool {
     bool e4m3;
     const void *k, *v;                    // bf16 pools or E4M3 codes

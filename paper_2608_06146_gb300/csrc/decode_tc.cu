@@ -284,7 +284,7 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
     // Nothing above touches global memory, so under a programmatic launch it overlaps the end of
     // the previous kernel in the stream. From here on the grid reads its inputs and writes partials
     // (which the previous step's merge may still be reading), so it first waits for that kernel, and
-    // only then lets the warp kernel (which writes partials too) launch.
+    // only then lets the next one launch.
     pdl_wait_prerequisite();
     pdl_launch_dependents();
     const int u0 = __shfl_sync(0xffffffffu, prm.cta_ptr[blockIdx.x], 0), u1 = __shfl_sync(0xffffffffu, prm.cta_ptr[blockIdx.x + 1], 0);
