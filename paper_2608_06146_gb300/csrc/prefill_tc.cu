@@ -240,7 +240,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
                 } else {
                     if (!wait_or_abort<true>(bar(C::B_UFULL + (n & 1)), (n >> 1) & 1, prm.err, 25, abort_flag)) break;
                     u = units[n & 1];
-                    arrive_lead(C::B_UEMPTY + (n & 1));
                 }
                 if (u.ne < 0) break;
                 const int g = u.h0 / group, h = u.h0 + NH * (int)rank;
@@ -269,7 +268,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
                     kt = kt_next;
                 }
                 if (!ok) break;
-                if (rank == 0) {
+                if (rank != 0) {
+                    // Only now may the first CTA write this slot of ours again (it does two units on): with
+                    // cluster scope, so that its stores come after the reads above, which an arrival of
+                    // CTA scope straight behind them did not order. The unit's loads are issued: nothing waits.
+                    mbar_arrive_cluster<true>(lead_bar(C::B_UEMPTY + (n & 1)));
+                } else {
                     if (u.ne == 0) ask();
                     if (!wait(C::B_NEXT, n & 1, 26)) break;
                     asked = false;
