@@ -704,6 +704,9 @@ prefill_bwd_dq_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
                     umma_commit_warp(bar(B_ACC + slot));
                     umma_commit_warp(bar(B_KEMPTY + s));
                 }
+                // A unit without entries issued nothing above and waited for nothing: its commit would complete the
+                // phase right behind the unit before's, whose parity the softmax warps may not have seen yet.
+                if (ok && un.nu == 0 && n > 0) ok = wait_w(B_DQFREE, (n - 1) & 1, 102);
                 umma_commit_warp(bar(B_DQFULL));
             }
         }
