@@ -721,7 +721,11 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                             }
                         const float qk = mi ? qk1 : qk0;
                         vl4[0] = vlb.x; vl4[1] = vlb.y; vl4[2] = vlb.z; vl4[3] = vlb.w;
-                        mul[0] = kcb.x * qk; mul[1] = kcb.y * qk; mul[2] = kcb.z * qk; mul[3] = kcb.w * qk;
+                        // a zero query row (its scale comes off as 2^-126) and a small K scale could multiply to 0, and
+                        // -inf, a masked column, times 0 is NaN: 2^-126 more, which no finite score (below 2^32 here) shows
+                        constexpr float kLeast = 0x1p-126f;
+                        mul[0] = fmaf(kcb.x, qk, kLeast); mul[1] = fmaf(kcb.y, qk, kLeast);
+                        mul[2] = fmaf(kcb.z, qk, kLeast); mul[3] = fmaf(kcb.w, qk, kLeast);
                         mx = fmaxf(fmax3f(fmaf(mx4[0], mul[0], vlb.x), fmaf(mx4[1], mul[1], vlb.y), fmaf(mx4[2], mul[2], vlb.z)),
                                    fmaf(mx4[3], mul[3], vlb.w));
                     } else {
