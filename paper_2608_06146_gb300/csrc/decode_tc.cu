@@ -180,6 +180,30 @@ __device__ __forceinline__ void expand_tile(uint8_t *slot, int lane)
     fence_proxy_async_smem();   // the MMAs read the panels through the async proxy
 }
 
+// E4M3: makes NaN codes in rows first .. end - 1 of a landed tile the format's largest magnitudes (whole warp,
+// before the tile's expansion; there the check would be paid by every tile).
+__device__ __forceinline__ void clean_tile(uint8_t *slot, int lane, int first, int end)
+{
+    uint4 *codes = reinterpret_cast<uint4 *>(slot + kPanel);
+    auto top = [](uint32_t w) { return (w & 0x7F7F7F7Fu) + 0x01010101u; };   // a byte's top bit: it is a NaN code
+    uint32_t any = 0u;
+#pragma unroll 8
+    for (int q = first * 8 + lane; q < end * 8; q += 32) {
+        const uint4 x = codes[q];
+        any |= top(x.x) | top(x.y);
+        any |= top(x.z) | top(x.w);
+    }
+    if (__any_sync(0xffffffffu, (any & 0x80808080u) != 0u)) {
+        auto finite = [&](uint32_t w) { return w - ((top(w) & 0x80808080u) >> 7); };
+#pragma unroll 1
+        for (int q = first * 8 + lane; q < end * 8; q += 32) {
+            const uint4 x = codes[q];
+            codes[q] = make_uint4(finite(x.x), finite(x.y), finite(x.z), finite(x.w));
+        }
+        __syncwarp();
+    }
+}
+
 // Pulls into L2 the first paged blocks (up to 4) of the first item of each of warp CTA wc's warp
 // lists, which this CTA runs once its pieces end, so that they land from L2 rather than from a
 // memory system under full load. Lane l takes block l % 4 of warp l / 4's first item; it reads the
@@ -338,10 +362,25 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
         // the next one to be (expanding tile n - 1 before issuing tile n kept one V load in flight).
         int nc = 0;
         float vl_last = -90.f;   // (K producer) log2 of the last nonzero V scale
+        // E4M3: V rows from a piece's least cutoff on (read an item ahead) are multiplied by probabilities of 0
+        // for some stream or all, and a NaN code there (a former owner's row, or one that only later branches
+        // see) would reach them; lane s holds slot s's first such row and (times 256) the end of its blocks.
+        int cut_next = 0, tile_clean = kKT;
+        auto fetch_low = [&](int uu) {
+            if (!kE4M3 || is_k) return;
+            const padoc_item &p = prm.items[uu];
+            const int32_t *cut = PADOC_ITEM_KIND(p.kind) == PADOC_ITEM_PRIVATE_TC ? prm.private_len : prm.shared_len;
+            cut_next = lane < p.num_streams ? cut[p.first_stream + lane] : INT32_MAX;
+        };
+        if (u0 < u1) fetch_low(u0);
         const int b_stg = is_k ? B_KSTG : B_VSTG;
         auto expand_next = [&]() {   // whole warp; nc counts only tiles whose codes have landed
             const int st = nc % nst;
             ++nc;
+            if (!is_k) {
+                const int rows = __shfl_sync(0xffffffffu, tile_clean, st), first = rows & 255;
+                if (first < kKT) clean_tile(ring + st * kTile, lane, first, rows >> 8);
+            }
             expand_tile(ring + st * kTile, lane);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(b_full + st));
@@ -402,15 +441,16 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
             const int ne = piece_tiles(it);
             // an item that continues the previous one keeps its queries
             const bool cont_in = u > u0 && (prm.items[u - 1].kind & PADOC_ITEM_CONT);
+            const int low = kE4M3 && !is_k ? __reduce_min_sync(0xffffffffu, min(cut_next, it.tok_end)) : 0;
             if (ne == 0) {
-                if (u + 1 < u1) fetch_id(u + 1, 0);
+                if (u + 1 < u1) { fetch_id(u + 1, 0); fetch_low(u + 1); }
                 continue;
             }
             for (int j = 0; j < ne; ++j) {
                 const int32_t id = id_next;
                 const bool in = in_next;
                 if (j + 1 < ne) fetch_id(u, j + 1);
-                else if (u + 1 < u1) fetch_id(u + 1, 0);
+                else if (u + 1 < u1) { fetch_id(u + 1, 0); fetch_low(u + 1); }
                 int32_t row = prm.pool_rows;
                 if (in) {
                     if (id >= 0 && id < prm.num_blocks) row = (id * prm.num_kv_heads + it.kv_head) * kBlk;
@@ -424,6 +464,10 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                     // the block's codes (16 rows x 128 bytes) into the slot's upper half; the K warp also
                     // copies the block's two scales into the tile's scale entry (zeros past the piece
                     // or for a bad id, whose codes are zeros too)
+                    if (!is_k && lane == s) {
+                        const int t0 = it.tok_begin + j * kKT;
+                        tile_clean = min(max(low - t0, 0), kKT) + 256 * min((it.tok_end - t0 + kBlk - 1) / kBlk * kBlk, kKT);
+                    }
                     if (lane == 0) mbar_arrive_expect_tx(bar(b_stg + s), kTile / 2);
                     __syncwarp();
                     if (lane < kKT / kBlk) {

@@ -86,6 +86,7 @@ __device__ __forceinline__ void decode_warp_role(const DecodeParams &prm, uint8_
     struct Walk {   // what the producer needs of an item
         const int32_t *table;
         int blk0, nblk, g;
+        int rows;   // E4M3: from blk0's first on, those the item sees
     };
     auto walk_of = [&](const padoc_item &it) {
         Walk w;
@@ -94,6 +95,7 @@ __device__ __forceinline__ void decode_warp_role(const DecodeParams &prm, uint8_
         w.blk0 = it.tok_begin / kBlk;
         w.nblk = it.tok_end > it.tok_begin ? (it.tok_end - it.tok_begin + kBlk - 1) / kBlk : 0;
         w.g = it.kv_head;
+        w.rows = it.tok_end - w.blk0 * kBlk;
         return w;
     };
     auto ids_of = [&](const Walk &w) { return lane < w.nblk ? w.table[w.blk0 + lane] : 0; };
@@ -106,7 +108,7 @@ __device__ __forceinline__ void decode_warp_role(const DecodeParams &prm, uint8_
     const bool have_fb = kPreWait && prm.first_blocks != nullptr;
     const int32_t fb = have_fb && lane < 4 ? prm.first_blocks[(size_t)wi * 4 + lane] : -1;
     int pu = i0, pb = 0;
-    Walk pc{prm.page_table, 0, 0, 0}, pn{prm.page_table, 0, 0, 0};
+    Walk pc{prm.page_table, 0, 0, 0, 0}, pn{prm.page_table, 0, 0, 0, 0};
     int32_t ids_c = 0, ids_n = 0;
     padoc_item hn2 = {};
     if (i0 < i1) { pc = walk_of(load_item(i0)); ids_c = ids_of(pc); }
@@ -134,15 +136,17 @@ __device__ __forceinline__ void decode_warp_role(const DecodeParams &prm, uint8_
             if constexpr (kE4M3) {
                 // chunk q = lane + 32k of the block's 256 16-byte chunks of codes: tensor q / 128,
                 // row (q / 8) % 16, chunk q % 8 (swizzled by row); lanes 0 and 1 also copy the K and
-                // V scales of the (block, KV head) (zeros for a bad id, whose codes are zeros too)
+                // V scales of the (block, KV head) (zeros for a bad id, whose codes are zeros too). V rows
+                // past the item's end land as zeros: a former owner's may hold NaN codes, against P = 0.
                 const uint32_t base = smem_u32(wbuf + (ring % kStages) * kE8StageBytes);
+                const int left = pc.rows - pb * kBlk;
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     const int q = lane + 32 * k;
                     const int tn = q >> 7, r = (q >> 3) & 15, cc = q & 7;
                     const uint8_t *src = (tn == 0 ? prm.k_codes : prm.v_codes) + (rowbase + r) * kD + cc * 16;
-                    cp_async_16_hint(base + tn * kE8Rows + r * 128 + ((cc ^ (r & 7)) << 4), src, okid ? 16u : 0u,
-                                     kv_policy);
+                    cp_async_16_hint(base + tn * kE8Rows + r * 128 + ((cc ^ (r & 7)) << 4), src,
+                                     okid && (tn == 0 || r < left) ? 16u : 0u, kv_policy);
                 }
                 if (lane < 2) {
                     const size_t si = okid ? (size_t)id * prm.num_kv_heads + pc.g : 0;

@@ -73,3 +73,20 @@ def test_multiplier_of_masked_columns(q_exp, k_exp):
     ks = (2.0 ** k_exp * rng.uniform(0.5, 1, (di.num_blocks, 2))).astype(np.float32)
     vs = rng.uniform(0.5, 2, (di.num_blocks, 2)).astype(np.float32)
     check(di, codes, ks, vs, q)
+
+
+def test_nan_codes_in_rows_no_stream_sees():
+    # Rows past a stream's end keep whatever a former owner left there, NaN codes too, and a row that
+    # only later branches see is nothing to the earlier ones.
+    di, codes, rng = cache(92)
+    for p, pg in enumerate(PAGES):
+        first = pg.prefix_len + (9 if p == 0 else max(pg.fork_offset))   # page 0: row 409 is seen from fork 16 on
+        for t in range(first, 16 * math.ceil((pg.prefix_len + pg.layout_len) / 16)):
+            for c in codes:
+                c[di.page_table[p, t // 16], :, t % 16] = rng.choice([0x7F, 0xFF], (2, 128))
+    for s, n in enumerate(di.priv_len):
+        for c in codes:
+            c[di.stream_table[s, (n - 1) // 16], :, (n - 1) % 16 + 1:] = 0x7F
+    ks, vs = (rng.uniform(0.2, 0.5, (di.num_blocks, 2)).astype(np.float32) for _ in range(2))
+    check(di, codes, ks, vs, di.q)
+    check(di, codes, ks, vs, di.q, tc_ctas=2, warp_ctas=2)
