@@ -41,9 +41,10 @@
 // landed whenever it would wait. The softmax warps turn each
 // piece's queries into f16, every row scaled by a power of two. The K producer also copies each block's
 // K and V scales into a ring of 4 entries, one per tile; the softmax applies the K scale to the block's
-// scores and folds the V scale into the block's probabilities before they are rounded to f16, and
-// removes it again from their row sum. The running maximum is that of score + log2(V scale), so that the
-// probabilities, times 2^6, fill f16's range whatever the scales.
+// scores and folds the V scale into the block's probabilities before they are rounded to f16. Their running
+// maximum is that of score + log2(V scale), so that they, times 2^6, fill f16's range whatever the scales; the
+// row sum is of the probabilities alone.
+#include <float.h>
 #include <math.h>
 
 #include <type_traits>
@@ -85,13 +86,13 @@ enum {
 };
 // scale ring: entry n % 4 for tile n (tile n is issued after the QK^T of tile n - 3, which follows the
 // softmax of tile n - 4): the K and V scales of the tile's 8 blocks as they land (16 floats), then what
-// the softmax reads: K factors, log2 of the V scales, and their inverses (8 floats each)
-constexpr int kSclEntries = 4, kSclFloats = 40;
+// the softmax reads: K factors and log2 of the V scales (8 floats each)
+constexpr int kSclEntries = 4, kSclFloats = 32;
 
 constexpr int kSoftmaxWarps = 8;
 constexpr int kXchBytes = 2 * 2 * 128 * 4;   // row max / sum swap: [buffer][column half][row] floats
 // Q (two M-tiles), the K and V rings, then barriers, the TMEM address and abort flag,
-// the scale ring (E4M3: [4 entries][40 floats]) and the swap buffer: 232,448 bytes,
+// the scale ring (E4M3: [4 entries][32 floats]) and the swap buffer: 232,448 bytes,
 // the most a CTA may have, so there is no room to align the start by hand; the kernel checks that
 // the driver placed it on a 1024-byte boundary (the base of a CTA's dynamic shared memory is) and
 // refuses to run otherwise.
@@ -361,7 +362,6 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
         // codes have landed, so that a slot is refilled as soon as it is free and no expansion waits for
         // the next one to be (expanding tile n - 1 before issuing tile n kept one V load in flight).
         int nc = 0;
-        float vl_last = -90.f;   // (K producer) log2 of the last nonzero V scale
         // E4M3: V rows from a piece's least cutoff on (read an item ahead) are multiplied by probabilities of 0
         // for some stream or all, and a NaN code there (a former owner's row, or one that only later branches
         // see) would reach them; lane s holds slot s's first such row and (times 256) the end of its blocks.
@@ -385,26 +385,17 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(b_full + st));
             if (is_k) {
-                // the tile's factors for the softmax, block l by lane l. A zero scale marks a block without
-                // a nonzero value (its codes are zeros): any positive factor gives the same result there,
-                // and the last nonzero V scale keeps the range.
+                // the tile's factors for the softmax, block l by lane l. A zero scale marks a block without a nonzero
+                // value (its codes are zeros): any K factor gives its scores, and no V factor is needed. A scale
+                // that is no finite number makes the block's scores NaN.
                 const int t = nc - 1, e = t % kSclEntries;
                 mbar_wait_bounded(bar(B_SCLRAW + e), (t / kSclEntries) & 1, prm.err, 58);
                 float *f = scl + e * kSclFloats;
                 const int b = lane & 7;
                 const float ks = f[b], vs = f[8 + b];
-                float vl = vs > 0.f ? fmaxf(__log2f(vs), -100.f) : INFINITY;
-#pragma unroll
-                for (int d = 1; d < 8; ++d) {   // a zero scale takes the nearest block's before it
-                    const float o = __shfl_up_sync(0xffffffffu, vl, 1, 8);
-                    if (vl == INFINITY && b > 0) vl = o;
-                }
-                if (vl == INFINITY) vl = vl_last;
-                vl_last = __shfl_sync(0xffffffffu, vl, 7, 8);
                 if (lane < 8) {
-                    f[16 + b] = ks > 0.f ? ks : 1.f;
-                    f[24 + b] = vl;
-                    f[32 + b] = fast_exp2(-vl);
+                    f[16 + b] = !(vs <= FLT_MAX) ? NAN : ks > 0.f ? ks : 1.f;
+                    f[24 + b] = vs > 0.f ? __log2f(vs) : -INFINITY;
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(B_SCL + e));
@@ -658,6 +649,10 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
             fetch_cut();
         }
         float m0 = -INFINITY, l0 = 0.f, m1 = -INFINITY, l1 = 0.f;   // running softmax state of the piece
+        // E4M3: m0, m1 are the maxima of score + log2 of the V scale, which P is taken against; the row sums have a
+        // reference of their own, the scores' alone in this column half: a token's weight in the denominator is
+        // its probability, however far its block's V scale lies from the others'
+        float a0 = -INFINITY, a1 = -INFINITY;
         // E4M3: the queries of a piece of mt M-tiles into f16, and what takes their rows' scales off again;
         // done for the next piece before this one's output, which then overlaps its first QK^T
         float qk0 = 1.f, qk1 = 1.f;
@@ -705,6 +700,7 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
             };
             if (!cont_in) {   // a new piece (an item continuing the previous one keeps the state)
                 m0 = -INFINITY; l0 = 0.f; m1 = -INFINITY; l1 = 0.f;
+                a0 = -INFINITY; a1 = -INFINITY;
                 if (kE4M3 && ne > 0) {
                     if (!q_done) convert_q(mt);
                     q_done = false;
@@ -713,19 +709,18 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
             for (int j = 0; j < ne; ++j) {
                 if (j == 1 && u + 1 < u1) fetch_cut();
                 if (j == ne - 1) fetch_slots();
-                // E4M3: for the 16-column blocks 4 hc .. 4 hc + 3 of this thread's column half, the K factor,
-                // the V scale's log2 (an offset of the exponent) and its inverse for the row sum
-                float4 kcb = {}, vlb = {}, vib = {};
+                // E4M3: for the 16-column blocks 4 hc .. 4 hc + 3 of this thread's column half, the K factor and
+                // the V scale's log2 (an offset of the exponent)
+                float4 kcb = {}, vlb = {};
                 if constexpr (kE4M3) {
                     const int e = cnt0 % kSclEntries;   // cnt0: tiles so far (every piece has M-tile 0)
                     ok = ok && wait_all(B_SCL + e, (cnt0 / kSclEntries) & 1, 72);
                     const float4 *f = reinterpret_cast<const float4 *>(scl + e * kSclFloats + 16) + hc;
                     kcb = f[0];
                     vlb = f[2];
-                    vib = f[4];
                 }
                 // one M-tile's turn
-                auto turn = [&](auto mi_, float &m_ref, float &l) {
+                auto turn = [&](auto mi_, float &m_ref, float &l, float &a_ref) {
                     const int mi = mi_;
                     const uint32_t tS = tmem + lanes + 128 * mi, tO = tS + 256;
                     const int cnt = mi ? cnt1 : cnt0;
@@ -752,7 +747,7 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                         }
                     }
                     float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-                    float mx, mul[4], vl4[4];   // E4M3: a block's score multiplier in log2 units, log2 of its V scale
+                    float mx, mul[4];   // E4M3: a block's score multiplier in log2 units
                     if constexpr (kE4M3) {
                         // block b = columns 16b .. 16b + 15 of the half: its max, then times its multiplier
 #pragma unroll
@@ -764,14 +759,24 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                                 mx4[b] = fmax3f(mx4[b], __uint_as_float(sr[uu][i + 2]), __uint_as_float(sr[uu][i + 3]));
                             }
                         const float qk = mi ? qk1 : qk0;
-                        vl4[0] = vlb.x; vl4[1] = vlb.y; vl4[2] = vlb.z; vl4[3] = vlb.w;
                         // a zero query row (its scale comes off as 2^-126) and a small K scale could multiply to 0, and
                         // -inf, a masked column, times 0 is NaN: 2^-126 more, which no finite score (below 2^32 here) shows
-                        constexpr float kLeast = 0x1p-126f;
-                        mul[0] = fmaf(kcb.x, qk, kLeast); mul[1] = fmaf(kcb.y, qk, kLeast);
-                        mul[2] = fmaf(kcb.z, qk, kLeast); mul[3] = fmaf(kcb.w, qk, kLeast);
-                        mx = fmaxf(fmax3f(fmaf(mx4[0], mul[0], vlb.x), fmaf(mx4[1], mul[1], vlb.y), fmaf(mx4[2], mul[2], vlb.z)),
-                                   fmaf(mx4[3], mul[3], vlb.w));
+                        const uint64_t qk2 = f2_pack(qk, qk), least = f2_pack(0x1p-126f, 0x1p-126f);
+                        const uint64_t u01 = f2_fma(f2_pack(kcb.x, kcb.y), qk2, least), u23 = f2_fma(f2_pack(kcb.z, kcb.w), qk2, least);
+                        const uint64_t s01 = f2_mul(f2_pack(mx4[0], mx4[1]), u01), s23 = f2_mul(f2_pack(mx4[2], mx4[3]), u23);
+                        float s0, s1, s2, s3, v0, v1, v2, v3;
+                        f2_unpack(u01, mul[0], mul[1]);
+                        f2_unpack(u23, mul[2], mul[3]);
+                        f2_unpack(s01, s0, s1);
+                        f2_unpack(s23, s2, s3);
+                        f2_unpack(f2_add(s01, f2_pack(vlb.x, vlb.y)), v0, v1);
+                        f2_unpack(f2_add(s23, f2_pack(vlb.z, vlb.w)), v2, v3);
+                        mx = fmaxf(fmax3f(v0, v1, v2), v3);
+                        const float am = fmaxf(fmax3f(s0, s1, s2), s3);
+                        if (am - a_ref > 8.f) {   // (the first time from -inf, with l still 0)
+                            l *= fast_exp2(a_ref - am);
+                            a_ref = am;
+                        }
                     } else {
 #pragma unroll
                         for (int uu = 0; uu < 2; ++uu)
@@ -794,18 +799,29 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                     float alpha = 1.f;
                     if (rescale) {
                         alpha = fast_exp2((m_ref - m_new) * cm);
-                        l *= alpha;
+                        if (!kE4M3) l *= alpha;
                         m_ref = m_new;
                     }
-                    // (E4M3: P times 2^6)
-                    const float moff = m_ref == -INFINITY ? 0.f : kE4M3 ? m_ref - 6.f : m_ref * cm;
-                    // two columns per packed instruction; E4M3: P of block b carries its V factor (the
-                    // exponent's log2 offset), which comes off again in the row sum
+                    const float moff = m_ref == -INFINITY ? 0.f : m_ref * cm;
+                    // two columns per packed instruction. E4M3: P of block b is the probability (against aoff) times
+                    // 2^(off + aoff), its V scale over the largest weighted one times 2^6: at most 2^14. Where that
+                    // power would be below -54 (0 in f16 either way) it is -54, so that the block's sum of P, divided
+                    // by it, stays the block's part of the row sum.
                     uint64_t rs2[4] = {0ull, 0ull, 0ull, 0ull};
                     uint32_t pk[32];
+                    float off4[4], aoff = 0.f;
+                    if constexpr (kE4M3) {
+                        aoff = a_ref == -INFINITY ? 0.f : a_ref;
+                        const float up = m_ref == -INFINITY ? -INFINITY : 6.f - m_ref, low = -54.f - aoff;
+                        const uint64_t up2 = f2_pack(up, up);
+                        f2_unpack(f2_add(f2_pack(vlb.x, vlb.y), up2), off4[0], off4[1]);
+                        f2_unpack(f2_add(f2_pack(vlb.z, vlb.w), up2), off4[2], off4[3]);
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) off4[b] = fmaxf(off4[b], low);
+                    }
 #pragma unroll
                     for (int b = 0; b < 4; ++b) {
-                        const float mb = kE4M3 ? mul[b] : c, ob = kE4M3 ? vl4[b] - moff : -moff;
+                        const float mb = kE4M3 ? mul[b] : c, ob = kE4M3 ? off4[b] : -moff;
                         const uint64_t m2 = f2_pack(mb, mb), o2 = f2_pack(ob, ob);
 #pragma unroll
                         for (int i = 16 * (b & 1); i < 16 * (b & 1) + 16; i += 2) {
@@ -820,8 +836,13 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                     tmem_st32(tS + 32 * hc, pk);   // P (pairs) of columns [64 hc, 64 hc + 64)
                     if constexpr (kE4M3) {
                         float a, b;
-                        f2_unpack(f2_fma(rs2[0], f2_pack(vib.x, vib.x), f2_fma(rs2[1], f2_pack(vib.y, vib.y),
-                                         f2_fma(rs2[2], f2_pack(vib.z, vib.z), f2_mul(rs2[3], f2_pack(vib.w, vib.w))))), a, b);
+                        uint64_t i2[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const float x = fast_exp2(-aoff - off4[k]);
+                            i2[k] = f2_pack(x, x);
+                        }
+                        f2_unpack(f2_fma(rs2[0], i2[0], f2_fma(rs2[1], i2[1], f2_fma(rs2[2], i2[2], f2_mul(rs2[3], i2[3])))), a, b);
                         l += a + b;
                     } else {
                         float a, b;
@@ -849,14 +870,14 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                 if constexpr (kE4M3) {   // one copy of the longer code (53.7 -> 51.5 us for the serving batch)
 #pragma unroll 1
                     for (int mi = 0; mi < mt; ++mi) {
-                        float m = mi ? m1 : m0, ll = mi ? l1 : l0;
-                        turn(mi, m, ll);
-                        if (mi) { m1 = m; l1 = ll; }
-                        else { m0 = m; l0 = ll; }
+                        float m = mi ? m1 : m0, ll = mi ? l1 : l0, aa = mi ? a1 : a0;
+                        turn(mi, m, ll, aa);
+                        if (mi) { m1 = m; l1 = ll; a1 = aa; }
+                        else { m0 = m; l0 = ll; a0 = aa; }
                     }
                 } else {                 // (one copy of the bf16 code spills: chunks 680 against 640 us)
-                    turn(std::integral_constant<int, 0>{}, m0, l0);
-                    if (mt == 2) turn(std::integral_constant<int, 1>{}, m1, l1);
+                    turn(std::integral_constant<int, 0>{}, m0, l0, a0);
+                    if (mt == 2) turn(std::integral_constant<int, 1>{}, m1, l1, a1);
                 }
             }
             if (ne < 2 && u + 1 < u1) fetch_cut();
@@ -876,6 +897,13 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                 if (ne > 0) {
                     ok = ok && wait_all(B_PVDONE + mi, (mi ? pd1 : pd0) & 1, 71);
                     if (mi) ++pd1; else ++pd0;
+                }
+                float lref = m_ref * cm, omul = 1.f;   // the row sum's reference; what O takes beside 1 / l
+                if constexpr (kE4M3) {                 // the halves' sums against the larger of their references
+                    const float a = mi ? a1 : a0;
+                    lref = fmaxf(a, swap_row(a));
+                    if (a != lref) l *= fast_exp2(a - lref);
+                    omul = m_ref == -INFINITY ? 0.f : exp2f(m_ref - 6.f - lref);
                 }
                 l += swap_row(l);   // plus the other column half's sum
                 if (!ok) continue;
@@ -901,7 +929,10 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                     if (valid) {
 #pragma unroll
                         for (int i = 0; i < 32; i += 8) {
-                            auto v = [&](int k) { return empty ? 0.f : __uint_as_float(o[i + k]) * inv; };
+                            auto v = [&](int k) {
+                                const float x = __uint_as_float(o[i + k]) * inv;
+                                return empty ? 0.f : kE4M3 ? x * omul : x;
+                            };
                             uint4 w;
                             w.x = pack_bf16x2(v(0), v(1));
                             w.y = pack_bf16x2(v(2), v(3));
@@ -917,7 +948,7 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                     }
                 }
                 if (valid && hc == 0) {
-                    const float lv = empty ? -INFINITY : (m_ref * cm - (kE4M3 ? 6.f : 0.f) + log2f(l)) * PADOC_LN2;
+                    const float lv = empty ? -INFINITY : (lref + log2f(l)) * PADOC_LN2;
                     if (sole) prm.lse[orow] = lv; else prm.part_lse[prow] = lv;
                 }
             }

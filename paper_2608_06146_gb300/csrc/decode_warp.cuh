@@ -14,9 +14,11 @@
 // movmatrix; the online softmax runs per head over the token axis with shuffles.
 #pragma once
 
+#include <float.h>
 #include <math.h>
 
 #include "common.cuh"
+#include "tc.cuh"
 
 namespace padoc_warp {
 
@@ -250,10 +252,10 @@ __device__ __forceinline__ void decode_warp_role(const DecodeParams &prm, uint8_
         const int blk0 = it.tok_begin / kBlk;
         const int nblk = cutoff > it.tok_begin ? (cutoff - it.tok_begin + kBlk - 1) / kBlk : 0;
         float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};   // heads h0 = 2*(lane%4), h0+1
-        // E4M3: the queries as f16, their scale off again in the score multipliers of heads h0, h0 + 1;
-        // the exponent of the last nonzero V scale
+        // E4M3: the queries as f16, their scale off again in the score multipliers of heads h0, h0 + 1; mv: the
+        // maxima of score + log2 of the V scale, which P is taken against (m: of the scores, for the row sums)
         float qk0 = prm.scale_log2, qk1 = prm.scale_log2;
-        int ev = -90;
+        float mv[2] = {-INFINITY, -INFINITY};
         if constexpr (kE4M3) {
             float amax = 0.f, qs, qi;
 #pragma unroll
@@ -279,121 +281,100 @@ __device__ __forceinline__ void decode_warp_role(const DecodeParams &prm, uint8_
             // j = lane % 4 (its rows' 32 contiguous bytes), and M row (m, half) of m-tile mt of O^T is dim
             // 16 m + 2 mt + half (16 contiguous bytes of each of its four tokens, two tokens' bytes
             // interleaved into pairs): one conversion instruction per two values, exact in f16, and no
-            // expanded copy in shared memory. The serving batch's lists alone: 52 us with the copy, 36 us so;
-            // kStep blocks share one turn of the softmax (2 and 3 are no faster: 38 and 41 us).
+            // expanded copy in shared memory. The serving batch's lists alone: 52 us with the copy, 36 us so
+            // (with two or three blocks to a turn of the softmax 38 and 41 us).
             const int r = lane >> 2, j = lane & 3;
             auto word = [](const uint4 &v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; };
-            constexpr int kStep = 1;
-            for (int bi = 0; bi < nblk; bi += kStep) {
-                const int nb = min(kStep, nblk - bi);
-                cp_async_wait<kStages - kStep>();   // the step's blocks have landed (one group per block)
+            for (int bi = 0; bi < nblk; ++bi, ++gc) {
+                cp_async_wait<kStages - 1>();   // block gc has landed (one group per block)
                 __syncwarp();
-                uint4 kc[kStep][2][2], vc[kStep][4];
-                float km0[kStep], km1[kStep], evf[kStep], lf[kStep], pf[kStep];
+                const uint8_t *stg = wbuf + (gc % kStages) * kE8StageBytes;
+                const float ks = *reinterpret_cast<const float *>(stg + 2 * kE8Rows);
+                const float vs = *reinterpret_cast<const float *>(stg + 2 * kE8Rows + 4);
+                uint4 kc[2][2], vc[4];
 #pragma unroll
-                for (int b = 0; b < kStep; ++b) {
-                    km0[b] = km1[b] = evf[b] = lf[b] = pf[b] = 0.f;
-                    if (b >= nb) {
+                for (int c = 0; c < 2; ++c)
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) kc[b][c >> 1][c & 1] = vc[b][c] = make_uint4(0u, 0u, 0u, 0u);
-                        continue;
-                    }
-                    const uint8_t *stg = wbuf + ((gc + b) % kStages) * kE8StageBytes;
-                    const float ks = *reinterpret_cast<const float *>(stg + 2 * kE8Rows);
-                    const float vs = *reinterpret_cast<const float *>(stg + 2 * kE8Rows + 4);
+                    for (int hh = 0; hh < 2; ++hh)
+                        kc[c][hh] = *reinterpret_cast<const uint4 *>(stg + (r + 8 * hh) * 128 + (((2 * j + c) ^ r) << 4));
 #pragma unroll
-                    for (int c = 0; c < 2; ++c)
-#pragma unroll
-                        for (int hh = 0; hh < 2; ++hh)
-                            kc[b][c][hh] = *reinterpret_cast<const uint4 *>(stg + (r + 8 * hh) * 128 + (((2 * j + c) ^ r) << 4));
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const int t = 2 * j + (c & 1) + 8 * (c >> 1);
-                        vc[b][c] = *reinterpret_cast<const uint4 *>(stg + kE8Rows + t * 128 + ((r ^ (t & 7)) << 4));
-                    }
-                    // A zero scale marks a block without a nonzero value (its codes are zeros): any positive
-                    // factor gives the same result. The V scale 2^ev x pf rides on P: the running maximum is
-                    // that of score + ev, so that P (times 2^6) fills the f16 range whatever the scales, and
-                    // the row sum takes the factor off again.
-                    if (vs > 0.f) ev = max((int)(__float_as_uint(vs) >> 23) - 127, -100);
-                    lf[b] = __uint_as_float((uint32_t)(127 - ev) << 23);
-                    pf[b] = vs * lf[b] * 64.f;
-                    evf[b] = (float)ev;
-                    km0[b] = qk0 * (ks > 0.f ? ks : 1.f);
-                    km1[b] = qk1 * (ks > 0.f ? ks : 1.f);
+                for (int c = 0; c < 4; ++c) {
+                    const int t = 2 * j + (c & 1) + 8 * (c >> 1);
+                    vc[c] = *reinterpret_cast<const uint4 *>(stg + kE8Rows + t * 128 + ((r ^ (t & 7)) << 4));
                 }
-                __syncwarp();   // every lane has its part: the stages may be refilled
-                for (int b = 0; b < nb; ++b) issue_next();
-                // S^T = K . Q^T, two independent MMA chains a block
-                float acc[kStep][2][4];
+                // A zero scale marks a block without a nonzero value (its codes are zeros): any K factor gives its
+                // scores, and its V counts nowhere. The V scale is 2^ev times a mantissa (NaN for none that is a
+                // finite number), which with 2^6 rides on P.
+                const bool tiny = vs < 0x1p-60f;
+                const uint32_t vb = __float_as_uint(tiny ? vs * 0x1p64f : vs);
+                const float ev = vs > 0.f ? (float)((int)(vb >> 23) - (tiny ? 127 + 64 : 127)) : -INFINITY;
+                const float pf = !(vs <= FLT_MAX) ? NAN : vs > 0.f ? __uint_as_float((vb & 0x007FFFFFu) | 0x42800000u) : 0.f;
+                const float kf = ks > 0.f ? ks : 1.f;
+                const uint64_t km = f2_mul(f2_pack(qk0, qk1), f2_pack(kf, kf));
+                __syncwarp();   // every lane has its part: the stage may be refilled
+                issue_next();
+                // S^T = K . Q^T, two independent MMA chains
+                float acc[2][4];
 #pragma unroll
-                for (int b = 0; b < kStep; ++b)
+                for (int c = 0; c < 2; ++c) acc[c][0] = acc[c][1] = acc[c][2] = acc[c][3] = 0.f;
 #pragma unroll
-                    for (int c = 0; c < 2; ++c) acc[b][c][0] = acc[b][c][1] = acc[b][c][2] = acc[b][c][3] = 0.f;
-#pragma unroll
-                for (int ks = 0; ks < 8; ++ks)
-#pragma unroll
-                    for (int b = 0; b < kStep; ++b) {
-                        const uint32_t x0 = word(kc[b][ks >> 2][0], ks & 3), x1 = word(kc[b][ks >> 2][1], ks & 3);
-                        const uint32_t a[4] = {e4m3x2_to_f16x2((uint16_t)x0), e4m3x2_to_f16x2((uint16_t)x1),
-                                               e4m3x2_to_f16x2((uint16_t)(x0 >> 16)), e4m3x2_to_f16x2((uint16_t)(x1 >> 16))};
-                        mma_f16_16816(acc[b][ks & 1], a, qb[ks][0], qb[ks][1]);
-                    }
-                float sc[kStep][4], mx0 = -INFINITY, mx1 = -INFINITY;
-#pragma unroll
-                for (int b = 0; b < kStep; ++b) {
-                    const int t0 = (blk0 + bi + b) * kBlk + r, t1 = t0 + 8;
-                    sc[b][0] = t0 < cutoff ? fmaf(acc[b][0][0] + acc[b][1][0], km0[b], evf[b]) : -INFINITY;
-                    sc[b][1] = t0 < cutoff ? fmaf(acc[b][0][1] + acc[b][1][1], km1[b], evf[b]) : -INFINITY;
-                    sc[b][2] = t1 < cutoff ? fmaf(acc[b][0][2] + acc[b][1][2], km0[b], evf[b]) : -INFINITY;
-                    sc[b][3] = t1 < cutoff ? fmaf(acc[b][0][3] + acc[b][1][3], km1[b], evf[b]) : -INFINITY;
-                    mx0 = fmaxf(mx0, fmaxf(sc[b][0], sc[b][2]));
-                    mx1 = fmaxf(mx1, fmaxf(sc[b][1], sc[b][3]));
+                for (int ks8 = 0; ks8 < 8; ++ks8) {
+                    const uint32_t x0 = word(kc[ks8 >> 2][0], ks8 & 3), x1 = word(kc[ks8 >> 2][1], ks8 & 3);
+                    const uint32_t a[4] = {e4m3x2_to_f16x2((uint16_t)x0), e4m3x2_to_f16x2((uint16_t)x1),
+                                           e4m3x2_to_f16x2((uint16_t)(x0 >> 16)), e4m3x2_to_f16x2((uint16_t)(x1 >> 16))};
+                    mma_f16_16816(acc[ks8 & 1], a, qb[ks8][0], qb[ks8][1]);
                 }
+                const int t0 = (blk0 + bi) * kBlk + r, t1 = t0 + 8;
+                float s0, s1, s2, s3;
+                f2_unpack(f2_mul(f2_add(f2_pack(acc[0][0], acc[0][1]), f2_pack(acc[1][0], acc[1][1])), km), s0, s1);
+                f2_unpack(f2_mul(f2_add(f2_pack(acc[0][2], acc[0][3]), f2_pack(acc[1][2], acc[1][3])), km), s2, s3);
+                if (t0 >= cutoff) s0 = s1 = -INFINITY;
+                if (t1 >= cutoff) s2 = s3 = -INFINITY;
+                float mx0 = fmaxf(s0, s2), mx1 = fmaxf(s1, s3);
 #pragma unroll
                 for (int sh = 4; sh < 32; sh <<= 1) {
                     mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, sh));
                     mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, sh));
                 }
                 const float mn0 = fmaxf(m[0], mx0), mn1 = fmaxf(m[1], mx1);
-                // a head whose columns are all masked so far keeps m = -inf and contributes 0
-                const float al0 = mn0 == -INFINITY ? 1.f : fast_exp2(m[0] - mn0);
-                const float al1 = mn1 == -INFINITY ? 1.f : fast_exp2(m[1] - mn1);
-                const float r0 = mn0 == -INFINITY ? 0.f : mn0, r1 = mn1 == -INFINITY ? 0.f : mn1;
-                m[0] = mn0; m[1] = mn1;
-                l[0] *= al0;
-                l[1] *= al1;
-                uint32_t bf[kStep][2];
-#pragma unroll
-                for (int b = 0; b < kStep; ++b) {
-                    const float p0 = fast_exp2(sc[b][0] - r0), p1 = fast_exp2(sc[b][1] - r1);
-                    const float p2 = fast_exp2(sc[b][2] - r0), p3 = fast_exp2(sc[b][3] - r1);
-                    l[0] = fmaf(p0 + p2, lf[b], l[0]);
-                    l[1] = fmaf(p1 + p3, lf[b], l[1]);
-                    bf[b][0] = movmatrix_trans(pack_f16x2(p0 * pf[b], p1 * pf[b]));
-                    bf[b][1] = movmatrix_trans(pack_f16x2(p2 * pf[b], p3 * pf[b]));
-                }
-                if (__any_sync(0xffffffffu, al0 != 1.f || al1 != 1.f)) {   // a head's running max moved
+                const float vn0 = fmaxf(mv[0], mx0 + ev), vn1 = fmaxf(mv[1], mx1 + ev);
+                if (__any_sync(0xffffffffu, mn0 != m[0] || mn1 != m[1] || vn0 != mv[0] || vn1 != mv[1])) {   // a maximum moved
+                    // (what has only been masked, or weighed by zero scales, keeps -inf and holds zeros)
+                    l[0] *= mn0 == -INFINITY ? 1.f : fast_exp2(m[0] - mn0);
+                    l[1] *= mn1 == -INFINITY ? 1.f : fast_exp2(m[1] - mn1);
+                    const float al0 = vn0 == -INFINITY ? 1.f : fast_exp2(mv[0] - vn0);
+                    const float al1 = vn1 == -INFINITY ? 1.f : fast_exp2(mv[1] - vn1);
 #pragma unroll
                     for (int mt = 0; mt < 8; ++mt) {
                         o[mt][0] *= al0; o[mt][1] *= al1; o[mt][2] *= al0; o[mt][3] *= al1;
                     }
+                    m[0] = mn0; m[1] = mn1;
+                    mv[0] = vn0; mv[1] = vn1;
                 }
+                // P is the probability times 2^f, f = V scale over the largest weighted one, at most 1; where f would
+                // be below -60 (0 in f16 either way) it is -60, and P times 2^-f is the probability for the row sum
+                const float r0 = mn0 == -INFINITY ? 0.f : mn0, r1 = mn1 == -INFINITY ? 0.f : mn1;
+                const float f0 = fmaxf(ev + (r0 - (vn0 == -INFINITY ? INFINITY : vn0)), -60.f);
+                const float f1 = fmaxf(ev + (r1 - (vn1 == -INFINITY ? INFINITY : vn1)), -60.f);
+                const uint64_t fr = f2_sub(f2_pack(f0, f1), f2_pack(r0, r1)), pf2 = f2_pack(pf, pf);
+                float x0, x1, x2, x3, y0, y1, y2, y3;
+                f2_unpack(f2_add(f2_pack(s0, s1), fr), x0, x1);
+                f2_unpack(f2_add(f2_pack(s2, s3), fr), x2, x3);
+                const uint64_t p01 = f2_pack(fast_exp2(x0), fast_exp2(x1)), p23 = f2_pack(fast_exp2(x2), fast_exp2(x3));
+                f2_unpack(f2_fma(f2_add(p01, p23), f2_pack(fast_exp2(-f0), fast_exp2(-f1)), f2_pack(l[0], l[1])), l[0], l[1]);
+                f2_unpack(f2_mul(p01, pf2), y0, y1);
+                f2_unpack(f2_mul(p23, pf2), y2, y3);
+                const uint32_t b0 = movmatrix_trans(pack_f16x2(y0, y1)), b1 = movmatrix_trans(pack_f16x2(y2, y3));
 #pragma unroll
-                for (int b = 0; b < kStep; ++b) {
-                    if (b >= nb) break;
+                for (int w = 0; w < 4; ++w)
 #pragma unroll
-                    for (int w = 0; w < 4; ++w)
-#pragma unroll
-                        for (int hh = 0; hh < 2; ++hh) {   // dims 4 w + 2 hh, + 1 of the lane's 16
-                            const uint32_t lo = __byte_perm(word(vc[b][0], w), word(vc[b][1], w), hh ? 0x7362 : 0x5140);
-                            const uint32_t hi = __byte_perm(word(vc[b][2], w), word(vc[b][3], w), hh ? 0x7362 : 0x5140);
-                            const uint32_t a[4] = {e4m3x2_to_f16x2((uint16_t)lo), e4m3x2_to_f16x2((uint16_t)(lo >> 16)),
-                                                   e4m3x2_to_f16x2((uint16_t)hi), e4m3x2_to_f16x2((uint16_t)(hi >> 16))};
-                            mma_f16_16816(o[2 * w + hh], a, bf[b][0], bf[b][1]);
-                        }
-                }
-                gc += nb;
+                    for (int hh = 0; hh < 2; ++hh) {   // dims 4 w + 2 hh, + 1 of the lane's 16
+                        const uint32_t lo = __byte_perm(word(vc[0], w), word(vc[1], w), hh ? 0x7362 : 0x5140);
+                        const uint32_t hi = __byte_perm(word(vc[2], w), word(vc[3], w), hh ? 0x7362 : 0x5140);
+                        const uint32_t a[4] = {e4m3x2_to_f16x2((uint16_t)lo), e4m3x2_to_f16x2((uint16_t)(lo >> 16)),
+                                               e4m3x2_to_f16x2((uint16_t)hi), e4m3x2_to_f16x2((uint16_t)(hi >> 16))};
+                        mma_f16_16816(o[2 * w + hh], a, b0, b1);
+                    }
             }
         } else {
             for (int bi = 0; bi < nblk; ++bi, ++gc) {
@@ -469,16 +450,24 @@ __device__ __forceinline__ void decode_warp_role(const DecodeParams &prm, uint8_
         if constexpr (kE4M3) {
             // a lane holds dims 16 (l / 4) .. + 15 of both heads: two 16-byte pieces of each
             const int h0 = (lane & 3) * 2;
-            const float i0f = l[0] > 0.f ? 0x1p-6f / l[0] : 0.f, i1f = l[1] > 0.f ? 0x1p-6f / l[1] : 0.f;
+            // (in two factors: with V scales near the ends of fp32's range their product leaves it)
+            const float i0f = l[0] > 0.f ? 1.f / l[0] : 0.f, i1f = l[1] > 0.f ? 1.f / l[1] : 0.f;
+            const float e0f = mv[0] == -INFINITY ? 0.f : exp2f(mv[0] - 6.f - m[0]);
+            const float e1f = mv[1] == -INFINITY ? 0.f : exp2f(mv[1] - 6.f - m[1]);
+#pragma unroll
+            for (int mt = 0; mt < 8; ++mt) {
+                o[mt][0] = o[mt][0] * i0f * e0f; o[mt][1] = o[mt][1] * i1f * e1f;
+                o[mt][2] = o[mt][2] * i0f * e0f; o[mt][3] = o[mt][3] * i1f * e1f;
+            }
             __nv_bfloat16 *p = prm.part_o + row0 * kD + (lane >> 2) * 128 + h0 * 8;   // chunk 2 (l / 4)
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 *reinterpret_cast<uint4 *>(p + 64 * c) =
-                    make_uint4(pack_bf16x2(o[4 * c][0] * i0f, o[4 * c][2] * i0f), pack_bf16x2(o[4 * c + 1][0] * i0f, o[4 * c + 1][2] * i0f),
-                               pack_bf16x2(o[4 * c + 2][0] * i0f, o[4 * c + 2][2] * i0f), pack_bf16x2(o[4 * c + 3][0] * i0f, o[4 * c + 3][2] * i0f));
+                    make_uint4(pack_bf16x2(o[4 * c][0], o[4 * c][2]), pack_bf16x2(o[4 * c + 1][0], o[4 * c + 1][2]),
+                               pack_bf16x2(o[4 * c + 2][0], o[4 * c + 2][2]), pack_bf16x2(o[4 * c + 3][0], o[4 * c + 3][2]));
                 *reinterpret_cast<uint4 *>(p + 64 * c + 8) =
-                    make_uint4(pack_bf16x2(o[4 * c][1] * i1f, o[4 * c][3] * i1f), pack_bf16x2(o[4 * c + 1][1] * i1f, o[4 * c + 1][3] * i1f),
-                               pack_bf16x2(o[4 * c + 2][1] * i1f, o[4 * c + 2][3] * i1f), pack_bf16x2(o[4 * c + 3][1] * i1f, o[4 * c + 3][3] * i1f));
+                    make_uint4(pack_bf16x2(o[4 * c][1], o[4 * c][3]), pack_bf16x2(o[4 * c + 1][1], o[4 * c + 1][3]),
+                               pack_bf16x2(o[4 * c + 2][1], o[4 * c + 2][3]), pack_bf16x2(o[4 * c + 3][1], o[4 * c + 3][3]));
             }
         } else {
             const int h0 = (lane & 3) * 2, dm = lane >> 2;

@@ -90,3 +90,28 @@ def test_nan_codes_in_rows_no_stream_sees():
     ks, vs = (rng.uniform(0.2, 0.5, (di.num_blocks, 2)).astype(np.float32) for _ in range(2))
     check(di, codes, ks, vs, di.q)
     check(di, codes, ks, vs, di.q, tc_ctas=2, warp_ctas=2)
+
+
+@pytest.mark.parametrize("first,then", [(None, 40), (None, 15), (-100, 30), (-125, 15), (30, -100), (15, None)])
+def test_row_sums_do_not_depend_on_v_scales(first, then):
+    # A history's blocks with V scales of 2^first up to a point and 2^then from there (None: zero blocks, whose
+    # codes are zeros), all at like scores: each token counts in the row sum whatever its V scale.
+    di, codes, rng = cache(93)
+    vs = np.zeros((di.num_blocks, 2), np.float32)
+    for table in list(di.page_table) + list(di.stream_table):
+        blocks = table[table >= 0]
+        cut = max(len(blocks) * 2 // 3, 1)
+        for part, e in ((blocks[:cut], first), (blocks[cut:], then)):
+            vs[part] = 0.0 if e is None else 2.0 ** e * rng.uniform(0.5, 1, (len(part), 2))
+    codes[1][vs == 0.0] = 0
+    ks = rng.uniform(0.2, 0.5, (di.num_blocks, 2)).astype(np.float32)
+    check(di, codes, ks, vs, di.q)
+    check(di, codes, ks, vs, di.q, tc_ctas=2, warp_ctas=2)
+
+
+@pytest.mark.parametrize("v_exp", [-98, -104, -112, -116])
+def test_v_scales_below_2_to_the_minus_100(v_exp):
+    # tensor-core and warp items alike carry the scale's own value
+    di, codes, rng = cache(94)
+    vs = (2.0 ** v_exp * rng.uniform(0.25, 1, (di.num_blocks, 2))).astype(np.float32)
+    check(di, codes, rng.uniform(0.2, 0.5, (di.num_blocks, 2)).astype(np.float32), vs, di.q)
