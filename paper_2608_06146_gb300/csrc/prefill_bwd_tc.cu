@@ -880,14 +880,25 @@ prefill_bwd_dq_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
 }
 
 // The CTAs that share a dK/dV unit. A page's first k-tiles are seen by all of its later queries, so the
-// largest unit is about twice the mean and a few units leave most of the chip idle; with many units the
-// sharing's own cost (~8 us a CTA) is the larger. Measured, both passes, with 1 / 2 / 4 / 8 CTAs a unit:
-// one page of 3419 tokens (54 units, 432 steps of 0.9 us the largest) 368 / 215 / 137 / 156 us, 34107
-// packed tokens (534 units) 1179 / 1159 / 1249 / 1517 us. A list-scheduling model over 60 page sets drawn
-// from 1 to 6 pages puts the lines where they are (within 10% of the best choice on all of them).
-int pick_cluster(int64_t units)
+// largest unit is about twice the mean and a few units leave most of the chip idle; with many units, or units
+// of few steps, the sharing's own cost (~8 us a CTA) is the larger. The host knows the number of units, the
+// query heads of a KV head (`group`: a unit's steps per q-tile) and a bound on the steps (every q-tile of the
+// call), not the page lengths, so the lines suit batches of short pages too. Measured on 152 SMs over 258
+// calls (13 head shapes, 40 to 20k tokens, pages of 60 to 6000), both passes, with 1 / 2 / 4 / 8 CTAs a unit:
+//   group 8: one page of 3419 tokens (54 units) 368 / 215 / 137 / 156 us, 34107 packed tokens (534 units)
+//            1179 / 1159 / 1249 / 1517 us, 40 pages of 60 tokens (38 units) 40 / 29 / 34 / 44 us;
+//   group 4: 16 pages of 140 tokens (144 units) 47 / 49 / 66 / 121 us, one page of 2500 tokens (80) 152 / 96 / 83 / 119 us;
+//   group 1: 8 pages of 140 tokens (144 units) 18.9 / 27 / 44 / 99 us, one page of 2500 tokens (20) 52 / 39 / 32 / 35 us.
+// On none of the 258 calls is the choice slower (by more than the spread) than the kernel before the clusters.
+int pick_cluster(int64_t units, int group, int64_t total_tokens)
 {
-    return units <= 45 ? 8 : units <= 160 ? 4 : units <= 560 ? 2 : 1;
+    const int64_t u = units * 152 / padoc_default_ctas(), steps = (total_tokens + dkv::kQT - 1) / dkv::kQT * group;
+    if (group >= 6) return u <= 45 ? 8 : u <= 160 ? 4 : u <= 560 ? 2 : 1;
+    int nc;
+    if (group >= 3) nc = u <= 12 ? 8 : u <= (steps >= 280 ? 160 : 72) ? 4 : u <= 560 ? 2 : 1;
+    else nc = u <= 12 ? 8 : u <= 36 ? 4 : u <= (steps >= 40 ? 100 : 76) ? 2 : 1;
+    while (nc > 1 && nc >= steps) nc /= 2;   // a step or more for each
+    return nc;
 }
 
 template <int NC>
@@ -977,7 +988,7 @@ padoc_status padoc_launch_prefill_bwd_tc(const void *q, const void *k, const voi
     pk.out0 = (__nv_bfloat16 *)dk;
     pk.out1 = (__nv_bfloat16 *)dv;
     const int64_t units = nkt * num_kv_heads;
-    switch (pick_cluster(units)) {
+    switch (pick_cluster(units, num_q_heads / num_kv_heads, T)) {
         case 8: return launch_dkv<8>(q64, g64, k128, v128, pk, units, stream);
         case 4: return launch_dkv<4>(q64, g64, k128, v128, pk, units, stream);
         case 2: return launch_dkv<2>(q64, g64, k128, v128, pk, units, stream);
