@@ -4,7 +4,7 @@
 //
 // A work unit is a 128-row q-tile of four query heads sharing a KV head, run by a CTA pair (two heads
 // per CTA); in small calls, and when the GQA group is no multiple of four, it is the q-tile of one head or
-// of two, run by one CTA. It walks the q-tile's entries of the tile map: fully masked k-tiles are never
+// of two, run by one CTA (in calls between, whichever suits the map: kEither below). It walks the q-tile's entries of the tile map: fully masked k-tiles are never
 // visited, FULL tiles skip masking, PARTIAL tiles mask each row with its two spans.
 //
 // What bounds it and why this split (8 pages, 34107 packed tokens, 16 / 2 heads; clock64 timelines):
@@ -93,6 +93,7 @@ struct TcPrefillParams {
     const int8_t *tile_kind;
     int64_t T;
     int32_t num_q_heads, num_kv_heads, num_q_tiles;
+    float over;             // kEither: (q-tile, head) units an SM, less one
     float scale_log2;
     float *lse;
     int *err;
@@ -116,7 +117,20 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, int
 
 __device__ __forceinline__ int clamp_tile(int x) { return min(max(x, 0), kKT); }
 
-template <int NH, int CG>
+constexpr int kEitherTiles = 160;   // q-tiles a kEither call may have (two units an SM, two heads and more)
+
+// Whether a call of 1 + over (q-tile, head) units an SM is faster with one head a CTA than with two (see the
+// launch). One head's longest unit takes 0.65 of the time less a tile, but the units then come in two waves:
+// the second adds about 0.75 of the mean unit's tiles and a unit's start and end for its share of the SMs.
+__device__ __forceinline__ bool one_head_units(int longest, int total, int q_tiles, float over)
+{
+    return 0.65f * (float)longest >= 2.f + over * (1.f + 0.75f * (float)total / (float)q_tiles);
+}
+
+// kEither (NH 2, one CTA): the grid has a CTA per (q-tile, head). Where the map is better run as that, only
+// head 0's warps work; else the first half of the CTAs run units of two heads, and the others, past the
+// units, are taken back by those that run (or end at once).
+template <int NH, int CG, bool kEither = false>
 __global__ void __launch_bounds__(kThreads, 1)
 prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap kmap,
                   const __grid_constant__ CUtensorMap vmap, const __grid_constant__ CUtensorMap omap, const TcPrefillParams prm)
@@ -138,6 +152,26 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (a value the compiler knows to be warp-uniform)
     const uint32_t rank = CG == 2 ? cluster_rank() : 0;
+    static_assert(!kEither || (NH == 2 && CG == 1), "");
+    // every warp reads the map's row pointers, which are on their way while the barriers are set up
+    int rows[kEither ? kEitherTiles / 32 : 1][2], total = 0;
+    if (kEither) {
+        total = prm.row_ptr[prm.num_q_tiles];
+#pragma unroll
+        for (int k = 0; k < kEitherTiles / 32; ++k) {
+            const int i = min(32 * k + lane, prm.num_q_tiles - 1);
+            rows[k][0] = prm.row_ptr[i];
+            rows[k][1] = prm.row_ptr[i + 1];
+        }
+    }
+    auto one_head = [&]() {
+        int longest = 0;
+#pragma unroll
+        for (int k = 0; k < kEitherTiles / 32; ++k) longest = max(longest, rows[k][1] - rows[k][0]);
+        return one_head_units(__reduce_max_sync(0xffffffffu, longest), __shfl_sync(0xffffffffu, total, 0), prm.num_q_tiles, prm.over);
+    };
+    if constexpr (kEither)
+        if ((int)blockIdx.y >= prm.num_q_tiles && !one_head()) return;
     auto bar = [&](int i) { return smem_u32(&bars[i]); };
     // a barrier of the pair's first CTA, which issues the MMAs and announces the units
     auto lead_bar = [&](int i) { return CG == 2 ? cluster_map(bar(i), 0) : bar(i); };
@@ -168,6 +202,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
     if (CG == 2) cluster_sync();   // no arrival or copy for the other CTA before its barriers are set up
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    bool single = false;
+    if constexpr (kEither) single = one_head();
     // the n-th unit, as every lane of a reading warp sees it
     auto read_unit = [&](int n, Unit &u, int site) {
         const bool r = wait_or_abort<CG == 2>(bar(C::B_UFULL + (n & 1)), (n >> 1) & 1, prm.err, site, abort_flag);
@@ -179,7 +215,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
         u.e0 = __shfl_sync(0xffffffffu, v.e0, 0);
         u.ne = __shfl_sync(0xffffffffu, v.ne, 0);
         __syncwarp();
-        if (lane == 0) arrive_lead(C::B_UEMPTY + (n & 1));
+        if (lane == 0) {
+            arrive_lead(C::B_UEMPTY + (n & 1));
+            if (single) arrive_lead(C::B_UEMPTY + (n & 1));   // (for head 1's warps, which have ended)
+        }
         return true;
     };
 
@@ -220,7 +259,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
                 ++nq[i];
                 return true;
             };
-            int n = 0;
+            int n = 0, asks = 0;   // units announced, questions answered
             for (;; ++n) {
                 Unit u = {0, 0, 0, -1};
                 if (rank == 0) {
@@ -228,6 +267,11 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
                     if (more) {
                         u.h0 = x * NH;
                         u.qt = prm.num_q_tiles - 1 - y;   // heavier tiles (later in a page) first
+                        if (single) {
+                            const int i = y * (int)gridDim.x + x;
+                            u.h0 = i % prm.num_q_heads;
+                            u.qt = prm.num_q_tiles - 1 - i / prm.num_q_heads;
+                        }
                         u.e0 = prm.row_ptr[u.qt];
                         u.ne = prm.row_ptr[u.qt + 1] - u.e0;
                     }
@@ -258,7 +302,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
                         box(kb + b * C::kKPanel, &kmap, g * kD + 64 * (b & 1),
                             kt * kKT + 64 * (b >> 1) + 64 / CG * (int)rank, C::B_KFULL + s);
                     ++tk;
-                    if (j == 0 && NH == 2 && !(ok = load_q(1, h + 1, u.qt))) break;
+                    if (j == 0 && NH == 2 && !single && !(ok = load_q(1, h + 1, u.qt))) break;
                     if (tv >= kStages && !(ok = wait(C::B_VEMPTY + s, (tv / kStages - 1) & 1, 23))) break;
                     uint8_t *vb = sv + s * C::kHalf;
                     expect(C::B_VFULL + s, C::kHalf);
@@ -275,16 +319,23 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
                     mbar_arrive_cluster<true>(lead_bar(C::B_UEMPTY + (n & 1)));
                 } else {
                     if (u.ne == 0) ask();
-                    if (!wait(C::B_NEXT, n & 1, 26)) break;
-                    asked = false;
-                    more = launch_control_answer(smem_u32(answer), x, y);
-                    fence_proxy_async_smem();   // the answer is read before the next one may be written
+                    for (;;) {
+                        if (!(ok = wait(C::B_NEXT, asks & 1, 26))) break;
+                        ++asks;
+                        asked = false;
+                        more = launch_control_answer(smem_u32(answer), x, y);
+                        fence_proxy_async_smem();   // the answer is read before the next one may be written
+                        // kEither: a CTA past the units of two heads had nothing to run, and there may be more
+                        if (!(kEither && more && !single && y >= prm.num_q_tiles)) break;
+                        ask();
+                    }
+                    if (!ok) break;
                 }
             }
             // copies still in flight must land before the CTA's shared memory is released (CG 2: the first
             // CTA sees both CTAs' land, and both stay until the cluster barrier below; after a wait that
             // ran out the other CTA may never issue its part, so the copies get a millisecond to land)
-            if (asked) mbar_wait_bounded(bar(C::B_NEXT), n & 1, prm.err, 27);
+            if (asked) mbar_wait_bounded(bar(C::B_NEXT), asks & 1, prm.err, 27);
             if (CG == 2 && *abort_flag) {
                 const uint64_t t0 = padoc_globaltimer();
                 while (padoc_globaltimer() - t0 < 1000000ull) {
@@ -297,7 +348,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
                 for (int t = max(tv - kStages, 0); t < tv; ++t)
                     mbar_wait_bounded(bar(C::B_VFULL + t % kStages), (t / kStages) & 1, prm.err, 29);
             }
-        } else if (warp >= 9 && warp < 9 + NH && rank == 0) {
+        } else if (warp >= 9 && warp < 9 + (single ? 1 : NH) && rank == 0) {
             // ------------------------------------------------------------ MMA issuers (a whole warp per head)
             const int i = warp - 9;
             constexpr uint32_t idS = umma_idesc_bf16(128 * CG, 64, false);
@@ -320,6 +371,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
                 if (h == 1) {
                     if (last) commit(C::B_QEMPTY + i);
                     commit(C::B_KEMPTY + stage);
+                    if (single) commit(C::B_KEMPTY + stage);   // (for head 1)
                 }
             };
             int n = 0;   // units read
@@ -349,6 +401,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
                 umma_bf16_ts_k64_mn_warp<CG>(tO, tS + 64 * h, dv + ((s * C::kHalf + h * 8192) >> 4), idPV, !first);
                 commit(C::B_PVDONE + 2 * i + h);
                 if (h == 1) commit(C::B_VEMPTY + s);
+                if (h == 1 && single) commit(C::B_VEMPTY + s);
                 return true;
             };
             for (int w = 0; ok && ne > 0; ++w) {
@@ -381,7 +434,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
             else umma_commit_warp(bar(C::B_FINAL + i));
             mbar_wait_bounded(bar(C::B_FINAL + i), 0, prm.err, 38);
         }
-    } else if (warp / 4 < NH) {
+    } else if (warp / 4 < (single ? 1 : NH)) {
         // ---------------------------------------------------------------- softmax + epilogue
         const int hi = warp / 4;                    // head index inside the unit
         const int row = tid & 127;
@@ -554,16 +607,16 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
     }
 }
 
-template <int NH, int CG>
+template <int NH, int CG, bool kEither = false>
 padoc_status launch(const CUtensorMap &qmap, const CUtensorMap &kmap, const CUtensorMap &vmap, const CUtensorMap &omap,
                     const TcPrefillParams &prm,
                     unsigned nqt, cudaStream_t stream)
 {
-    auto kernel = prefill_tc_kernel<NH, CG>;
+    auto kernel = prefill_tc_kernel<NH, CG, kEither>;
     constexpr size_t bytes = Cfg<NH, CG>::kSmemBytes;
     if (const padoc_status st = padoc_set_max_smem((const void *)kernel, (int)bytes)) return st;
     cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3((unsigned)(prm.num_q_heads / NH), nqt);
+    lc.gridDim = dim3((unsigned)(prm.num_q_heads / NH), kEither ? 2 * nqt : nqt);
     lc.blockDim = dim3(kThreads);
     lc.dynamicSmemBytes = bytes;
     lc.stream = stream;
@@ -572,7 +625,7 @@ padoc_status launch(const CUtensorMap &qmap, const CUtensorMap &kmap, const CUte
     attr[0].val.clusterDim.x = CG;
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     lc.attrs = attr;
-    lc.numAttrs = 1;
+    lc.numAttrs = CG == 1 ? 0 : 1;   // (304 single CTAs as clusters of one took 15.9 us, as plain ones 14.1)
     PADOC_CUDA_TRY(cudaLaunchKernelEx(&lc, kernel, qmap, kmap, vmap, omap, prm));
     return padoc_launch_status();
 }
@@ -590,14 +643,17 @@ padoc_status padoc_launch_prefill_tc(const void *q, const void *k, const void *v
     if (!err) return PADOC_ERR_CUDA;
     const int64_t nqt = (total_tokens + kQT - 1) / kQT;
     if (nqt > 65535) return PADOC_ERR_UNSUPPORTED;
-    // Up to two (q-tile, head) units an SM, a CTA per unit: a call then lasts as long as its longest units,
-    // and a head alone takes ~1000 cycles a half where two share the tensor cores (1450). At 16 / 2 heads, one
-    // page of 500 / 1000 / 2048 tokens takes 12.4 / 16.5 / 27.0 us against 16.5 / 21.5 / 32.9 in pairs; 3000
-    // tokens (384 units) 44.7 against 42.6. Above that, CTA pairs when the heads of a KV head come in fours
-    // (34107 tokens: 332 us against 400 with two heads on a CTA), else a CTA with two heads or one.
+    // Up to one (q-tile, head) unit an SM, a CTA per unit: the call lasts as long as its longest unit, and a head
+    // alone takes ~1000 cycles a half where two share the tensor cores (1450). Up to two an SM that is right
+    // while the longest units set the time, but short units then come in two waves where two heads a CTA need
+    // one: the kernel decides by the map (one_head_units, fitted to 200 calls timed with both: within 0.4% of the
+    // better one on the mean, 12% at most). At 256 units, 16 / 2 heads, one head / two heads a CTA: 2045 tokens
+    // as one causal page 24.2 / 30.8 us, as 12 short pages 15.7 / 11.9. Above two an SM, CTA pairs when the heads
+    // of a KV head come in fours (34107 tokens: 332 us against 400 with two heads on a CTA), else two or one.
     const int group = num_q_heads / num_kv_heads;
-    const bool small = nqt * num_q_heads <= 2 * padoc_default_ctas();
-    const int cg = !small && group % 4 == 0 ? 2 : 1;
+    const int64_t units = nqt * num_q_heads, sms = padoc_default_ctas();
+    const bool small = units <= (group % 2 == 0 ? sms : 2 * sms), either = !small && units <= 2 * sms && nqt <= kEitherTiles;
+    const int cg = !small && !either && group % 4 == 0 ? 2 : 1;
     CUtensorMap qmap, kmap, vmap, omap;
     if (!padoc_make_tmap_bf16(&qmap, q, (uint64_t)num_q_heads * kD, total_tokens, (uint64_t)num_q_heads * kD * 2, 64, kQT) ||
         !padoc_make_tmap_bf16(&kmap, k, (uint64_t)num_kv_heads * kD, total_tokens, (uint64_t)num_kv_heads * kD * 2, 64, 64 / cg) ||
@@ -613,9 +669,11 @@ padoc_status padoc_launch_prefill_tc(const void *q, const void *k, const void *v
     prm.num_q_heads = num_q_heads;
     prm.num_kv_heads = num_kv_heads;
     prm.num_q_tiles = (int32_t)nqt;
+    prm.over = (float)units / (float)sms - 1.f;
     prm.scale_log2 = scale_log2;
     prm.lse = lse;
     prm.err = err;
+    if (either) return launch<2, 1, true>(qmap, kmap, vmap, omap, prm, (unsigned)nqt, stream);
     if (cg == 2) return launch<2, 2>(qmap, kmap, vmap, omap, prm, (unsigned)nqt, stream);
     if (!small && group % 2 == 0) return launch<2, 1>(qmap, kmap, vmap, omap, prm, (unsigned)nqt, stream);
     return launch<1, 1>(qmap, kmap, vmap, omap, prm, (unsigned)nqt, stream);
