@@ -709,16 +709,8 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
             for (int j = 0; j < ne; ++j) {
                 if (j == 1 && u + 1 < u1) fetch_cut();
                 if (j == ne - 1) fetch_slots();
-                // E4M3: for the 16-column blocks 4 hc .. 4 hc + 3 of this thread's column half, the K factor and
-                // the V scale's log2 (an offset of the exponent)
-                float4 kcb = {}, vlb = {};
-                if constexpr (kE4M3) {
-                    const int e = cnt0 % kSclEntries;   // cnt0: tiles so far (every piece has M-tile 0)
-                    ok = ok && wait_all(B_SCL + e, (cnt0 / kSclEntries) & 1, 72);
-                    const float4 *f = reinterpret_cast<const float4 *>(scl + e * kSclFloats + 16) + hc;
-                    kcb = f[0];
-                    vlb = f[2];
-                }
+                const int scl_e = cnt0 % kSclEntries;   // E4M3: the tile's scales (cnt0: tiles so far, every piece has M-tile 0)
+                if constexpr (kE4M3) ok = ok && wait_all(B_SCL + scl_e, (cnt0 / kSclEntries) & 1, 72);
                 // one M-tile's turn
                 auto turn = [&](auto mi_, float &m_ref, float &l, float &a_ref) {
                     const int mi = mi_;
@@ -732,6 +724,14 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                     if (!ok) {
                         swap_row(0.f);
                         return;
+                    }
+                    // E4M3: for the 16-column blocks 4 hc .. 4 hc + 3 of this thread's column half, the K factor and the V
+                    // scale's log2 (an offset of the exponent); read in each turn (held over both they spill, 0.6 us)
+                    [[maybe_unused]] float4 kcb = {}, vlb = {};
+                    if constexpr (kE4M3) {
+                        const float4 *f = reinterpret_cast<const float4 *>(scl + scl_e * kSclFloats + 16) + hc;
+                        kcb = f[0];
+                        vlb = f[2];
                     }
                     tc_fence_after();
                     uint32_t sr[2][32];
@@ -809,7 +809,7 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                     // by it, stays the block's part of the row sum.
                     uint64_t rs2[4] = {0ull, 0ull, 0ull, 0ull};
                     uint32_t pk[32];
-                    float off4[4], aoff = 0.f;
+                    [[maybe_unused]] float off4[4], aoff = 0.f;
                     if constexpr (kE4M3) {
                         aoff = a_ref == -INFINITY ? 0.f : a_ref;
                         const float up = m_ref == -INFINITY ? -INFINITY : 6.f - m_ref, low = -54.f - aoff;
