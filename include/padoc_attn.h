@@ -412,8 +412,12 @@ padoc_status padoc_append_inputs_e4m3(const padoc_kv_pool_e4m3 *pool, const void
  * [num_streams][Hq][128], lse fp32. Attention is over the dequantized values code_value * scale:
  * codes become f16 exactly, each query row f16 under a power-of-two scale, the K scale multiplies each
  * 16-token block's scores and the V scale the block's probabilities in fp32 before they are rounded to
- * f16. Hq / Hkv = 8,
- * block_size 16, head_dim 128. Errors: INVALID_ARGUMENT, UNSUPPORTED, WORKSPACE_TOO_SMALL, CUDA. */
+ * f16; the softmax's denominator is of the fp32 probabilities, whatever the V scales. f16 holds five
+ * exponent bits: of a query row, elements below 2^-28 of its largest lose bits, and a token whose
+ * probability x V scale is below 2^-20 of its history's largest loses bits of its V, below 2^-30 all of it.
+ * NaN codes: a stream is not affected by rows it does not see (past its end, or of the shared stream past
+ * its cutoff); in a piece's rows that some of its streams do not see, a NaN code of V counts as the
+ * largest magnitude for those that do. Hq / Hkv = 8, block_size 16, head_dim 128. Errors: INVALID_ARGUMENT, UNSUPPORTED, WORKSPACE_TOO_SMALL, CUDA. */
 padoc_status padoc_branch_decode_attn_e4m3(const padoc_kv_pool_e4m3 *pool, const padoc_decode_plan *info,
                                            const int32_t *plan_dev, const int32_t *page_block_table,
                                            int32_t page_table_stride, const int32_t *stream_block_table,

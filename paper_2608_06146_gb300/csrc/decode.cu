@@ -7,9 +7,9 @@
 // query heads fill dense M = 128 tiles read their shared stream on the tensor cores
 // (decode_tc.cu): each K/V tile is fetched once for all of the page's streams. Every private
 // history, and the shared stream of pages with few branches, is read by the warp path
-// (decode_warp.cuh), which the same grid runs (bf16): its CTAs run their tensor-core pieces first,
-// the rest start on the warp lists at once; for the E4M3 pool the warp lists run in a grid of their
-// own. A split-K merge then joins each (stream, head)'s partials.
+// (decode_warp.cuh), which the same grid runs: its CTAs run their tensor-core pieces first, the rest
+// start on the warp lists at once (over the E4M3 pool too). A split-K merge then joins each
+// (stream, head)'s partials.
 #include <math.h>
 #include <stddef.h>
 
@@ -173,23 +173,10 @@ constexpr int kMergeCluster = 8;
 #define PADOC_MERGE_CLUSTER_MAX_KEYS 8
 #endif
 
-__device__ __forceinline__ uint32_t cluster_ctarank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-__device__ __forceinline__ void cluster_barrier()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 // The state at shared address `addr` of cluster CTA `rank`.
 __device__ __forceinline__ MergeState load_remote_state(uint32_t addr, uint32_t rank)
 {
-    uint32_t ra;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(addr), "r"(rank));
+    const uint32_t ra = cluster_map(addr, rank);
     MergeState o;
     asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(o.mref), "=f"(o.ssum) : "r"(ra) : "memory");
     asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
@@ -208,7 +195,7 @@ __global__ void __launch_bounds__(512, 2) decode_combine_cluster_kernel(
     const int32_t *__restrict__ slot_ptr, const int32_t *__restrict__ merge_keys, const __nv_bfloat16 *__restrict__ part_o,
     const float *__restrict__ part_lse, __nv_bfloat16 *__restrict__ out, float *__restrict__ lse_out)
 {
-    const uint32_t rank = cluster_ctarank();
+    const uint32_t rank = cluster_rank();
     const int kidx = (int)(blockIdx.x / kMergeCluster);
     const int key = kIndexed ? merge_keys[kidx] : kidx;
     const int p0 = slot_ptr[key], n = slot_ptr[key + 1] - p0;
@@ -228,14 +215,14 @@ __global__ void __launch_bounds__(512, 2) decode_combine_cluster_kernel(
         for (int k = 1; k < 4; ++k) merge_join(ms, st[k][tid]);
         st[0][tid] = ms;
     }
-    cluster_barrier();
+    cluster_sync();
     if (rank == 0 && q == 0) {
         const uint32_t addr = smem_u32(&st[0][tid]);
 #pragma unroll 1
         for (uint32_t r = 1; r < (uint32_t)kMergeCluster; ++r) merge_join(ms, load_remote_state(addr, r));
         merge_store(ms, key, h, part, out, lse_out);
     }
-    cluster_barrier();
+    cluster_sync();
 }
 
 template <class Slots, class OutT>

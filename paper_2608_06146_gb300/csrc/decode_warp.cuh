@@ -1,6 +1,5 @@
-// decode_warp.cuh -- C2/C5: the warp path of one decode step, shared by the stand-alone warp
-// kernel (decode.cu) and the fused decode grid, whose CTAs run it after their tensor-core pieces
-// (decode_tc.cu).
+// decode_warp.cuh -- C2/C5: the warp path of one decode step, over either pool: the decode grid's CTAs run
+// it after their tensor-core pieces, or from the start where they have none (decode_tc.cu).
 //
 // Every warp owns one work item and runs on its own: a 3-deep ring of 16-token
 // paged blocks fetched with cp.async (each lane copies 16 of the block's 512 16-byte chunks into

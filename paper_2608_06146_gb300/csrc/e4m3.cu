@@ -18,9 +18,10 @@ constexpr int kQuantWarps = 8;  // warps per CTA of the quantize kernel, one (bl
 // every value pays an IEEE division of its own. With inv = 1 / s correctly rounded and q within one unit
 // of the last place of x / s, r = x - q s is exact and q + r inv, rounded once, is x / s correctly rounded
 // (Markstein 1990, theorem on the final division step); the first such step brings x inv within that unit,
-// the second rounds: five packed instructions for two values. Exact for 2^-80 < s < 2^80: r then stays
-// above the subnormals for every |x / s| >= 2^-20 (smaller quotients have the code 0 with or without the
-// last rounding). Other scales take the division.
+// the second rounds: five packed instructions for two values. Exact for 2^-80 < s < 2^80 and every
+// |x / s| >= 2^-20 (smaller quotients have the code 0 with or without the last rounding): q is a multiple
+// of 2^-43 and s of 2^-103, so r is one of 2^-146 and is held exactly, as a subnormal too: the packed
+// instructions must not flush them. Other scales take the division.
 struct Scale {
     float s, inv;
     bool fast;
