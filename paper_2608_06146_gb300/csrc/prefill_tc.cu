@@ -153,7 +153,15 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (a value the compiler knows to be warp-uniform)
     const uint32_t rank = CG == 2 ? cluster_rank() : 0;
     static_assert(!kEither || (NH == 2 && CG == 1), "");
-    // every warp reads the map's row pointers, which are on their way while the barriers are set up
+    // the first unit's entries (for the producer), on their way while the barriers are set up: a call of one tile
+    // a q-tile waits for each global read in turn
+    int first_e0 = 0, first_end = 0;
+    if (warp == 8 && (!kEither || (int)blockIdx.y < prm.num_q_tiles)) {
+        const int qt = prm.num_q_tiles - 1 - (int)blockIdx.y;
+        first_e0 = prm.row_ptr[qt];
+        first_end = prm.row_ptr[qt + 1];
+    }
+    // kEither: every warp reads the map's row pointers
     int rows[kEither ? kEitherTiles / 32 : 1][2], total = 0;
     if (kEither) {
         total = prm.row_ptr[prm.num_q_tiles];
@@ -272,8 +280,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
                             u.h0 = i % prm.num_q_heads;
                             u.qt = prm.num_q_tiles - 1 - i / prm.num_q_heads;
                         }
-                        u.e0 = prm.row_ptr[u.qt];
-                        u.ne = prm.row_ptr[u.qt + 1] - u.e0;
+                        const bool read = n > 0 || single;
+                        u.e0 = read ? prm.row_ptr[u.qt] : first_e0;
+                        u.ne = (read ? prm.row_ptr[u.qt + 1] : first_end) - u.e0;
                     }
                     units[n & 1] = u;
                     mbar_arrive(bar(C::B_UFULL + (n & 1)));
