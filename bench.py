@@ -49,7 +49,7 @@ FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustain
 # step, the mean of two consecutive steps; E4M3: the decode grid and the merge, cold caches, the mean
 # of two consecutive steps). Prefill: cold caches. Prefill backward: both passes, cold caches.
 TRAFFIC_BYTES = {"decode": 201_274_880,
-                 "decode_e4m3": 113_394_432,
+                 "decode_e4m3": 112_220_800,
                  "prefill": 263_395_840,
                  "prefill_bwd": 1_612_553_728}
 
