@@ -155,12 +155,16 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
     static_assert(!kEither || (NH == 2 && CG == 1), "");
     // the first unit's entries (for the producer), on their way while the barriers are set up: a call of one tile
     // a q-tile waits for each global read in turn
-    int first_e0 = 0, first_end = 0;
-    if (warp == 8 && (!kEither || (int)blockIdx.y < prm.num_q_tiles)) {
-        const int qt = prm.num_q_tiles - 1 - (int)blockIdx.y;
-        first_e0 = prm.row_ptr[qt];
-        first_end = prm.row_ptr[qt + 1];
-    }
+    // ([1]: as one head's unit)
+    int first[kEither ? 2 : 1][2] = {};
+    if (warp == 8)
+#pragma unroll
+        for (int k = 0; k < (kEither ? 2 : 1); ++k) {
+            const int y = k ? (int)(blockIdx.y * gridDim.x + blockIdx.x) / prm.num_q_heads : (int)blockIdx.y;
+            const int qt = max(prm.num_q_tiles - 1 - y, 0);   // (kEither: y past the units of two heads)
+            first[k][0] = prm.row_ptr[qt];
+            first[k][1] = prm.row_ptr[qt + 1];
+        }
     // kEither: every warp reads the map's row pointers
     int rows[kEither ? kEitherTiles / 32 : 1][2], total = 0;
     if (kEither) {
@@ -280,9 +284,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
                             u.h0 = i % prm.num_q_heads;
                             u.qt = prm.num_q_tiles - 1 - i / prm.num_q_heads;
                         }
-                        const bool read = n > 0 || single;
-                        u.e0 = read ? prm.row_ptr[u.qt] : first_e0;
-                        u.ne = (read ? prm.row_ptr[u.qt + 1] : first_end) - u.e0;
+                        constexpr int kOne = kEither ? 1 : 0;
+                        u.e0 = n > 0 ? prm.row_ptr[u.qt] : single ? first[kOne][0] : first[0][0];
+                        u.ne = (n > 0 ? prm.row_ptr[u.qt + 1] : single ? first[kOne][1] : first[0][1]) - u.e0;
                     }
                     units[n & 1] = u;
                     mbar_arrive(bar(C::B_UFULL + (n & 1)));
@@ -306,6 +310,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
                     if (tk >= kStages && !(ok = wait(C::B_KEMPTY + s, (tk / kStages - 1) & 1, 21))) break;
                     uint8_t *kb = sk + s * C::kHalf;
                     expect(C::B_KFULL + s, C::kHalf);
+                    if (single) mbar_arrive(bar(C::B_KEMPTY + s));   // (for head 1, as below)
 #pragma unroll
                     for (int b = 0; b < 4; ++b)   // [key half][dim half]
                         box(kb + b * C::kKPanel, &kmap, g * kD + 64 * (b & 1),
@@ -315,6 +320,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
                     if (tv >= kStages && !(ok = wait(C::B_VEMPTY + s, (tv / kStages - 1) & 1, 23))) break;
                     uint8_t *vb = sv + s * C::kHalf;
                     expect(C::B_VFULL + s, C::kHalf);
+                    if (single) mbar_arrive(bar(C::B_VEMPTY + s));
                     box(vb, &vmap, g * kD + 64 * (int)rank, kt * kKT, C::B_VFULL + s);
                     if (CG == 1) box(vb + kPanel, &vmap, g * kD + 64, kt * kKT, C::B_VFULL + s);
                     ++tv;
@@ -380,7 +386,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
                 if (h == 1) {
                     if (last) commit(C::B_QEMPTY + i);
                     commit(C::B_KEMPTY + stage);
-                    if (single) commit(C::B_KEMPTY + stage);   // (for head 1)
                 }
             };
             int n = 0;   // units read
@@ -410,7 +415,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
                 umma_bf16_ts_k64_mn_warp<CG>(tO, tS + 64 * h, dv + ((s * C::kHalf + h * 8192) >> 4), idPV, !first);
                 commit(C::B_PVDONE + 2 * i + h);
                 if (h == 1) commit(C::B_VEMPTY + s);
-                if (h == 1 && single) commit(C::B_VEMPTY + s);
                 return true;
             };
             for (int w = 0; ok && ne > 0; ++w) {
