@@ -813,11 +813,8 @@ __device__ __forceinline__ void decode_tc_role(const CUtensorMap &kmap, const CU
                     if constexpr (kE4M3) {
                         aoff = a_ref == -INFINITY ? 0.f : a_ref;
                         const float up = m_ref == -INFINITY ? -INFINITY : 6.f - m_ref, low = -54.f - aoff;
-                        const uint64_t up2 = f2_pack(up, up);
-                        f2_unpack(f2_add(f2_pack(vlb.x, vlb.y), up2), off4[0], off4[1]);
-                        f2_unpack(f2_add(f2_pack(vlb.z, vlb.w), up2), off4[2], off4[3]);
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) off4[b] = fmaxf(off4[b], low);
+                        off4[0] = fmaxf(vlb.x + up, low); off4[1] = fmaxf(vlb.y + up, low);
+                        off4[2] = fmaxf(vlb.z + up, low); off4[3] = fmaxf(vlb.w + up, low);
                     }
 #pragma unroll
                     for (int b = 0; b < 4; ++b) {

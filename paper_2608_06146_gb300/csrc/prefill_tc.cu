@@ -659,7 +659,7 @@ padoc_status padoc_launch_prefill_tc(const void *q, const void *k, const void *v
     // Up to one (q-tile, head) unit an SM, a CTA per unit: the call lasts as long as its longest unit, and a head
     // alone takes ~1000 cycles a half where two share the tensor cores (1450). Up to two an SM that is right
     // while the longest units set the time, but short units then come in two waves where two heads a CTA need
-    // one: the kernel decides by the map (one_head_units, fitted to 200 calls timed with both: within 0.4% of the
+    // one: the kernel decides by the map (one_head_units, fitted to 175 calls timed with both: within 0.4% of the
     // better one on the mean, 12% at most). At 256 units, 16 / 2 heads, one head / two heads a CTA: 2045 tokens
     // as one causal page 24.2 / 30.8 us, as 12 short pages 15.7 / 11.9. Above two an SM, CTA pairs when the heads
     // of a KV head come in fours (34107 tokens: 332 us against 400 with two heads on a CTA), else two or one.
